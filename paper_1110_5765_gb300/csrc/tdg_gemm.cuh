@@ -32,28 +32,33 @@
 // its TMEM and returns without storing.
 #pragma once
 
+#include <type_traits>
+
 #include "tdg_common.cuh"
+#include "tdg_digits.cuh"
 #include "tdg_internal.h"
 
 namespace tdg {
 
-template <typename T>
-struct Vec4;
-template <>
-struct Vec4<float> {
-    __device__ static inline void load(const float *p, float *o) {
-        float4 v = *reinterpret_cast<const float4 *>(p);
-        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+// N consecutive values of a shared-memory row (N = 4, or 1 and 2 for fp64)
+template <int N>
+__device__ inline void frag_load(const float *p, float *o) {
+    static_assert(N == 4, "fp32 fragments are 4 wide");
+    float4 v = *reinterpret_cast<const float4 *>(p);
+    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+}
+template <int N>
+__device__ inline void frag_load(const double *p, double *o) {
+    if constexpr (N == 1) {
+        o[0] = *p;
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 2) {
+            double2 v = *reinterpret_cast<const double2 *>(p + i);
+            o[i] = v.x; o[i + 1] = v.y;
+        }
     }
-};
-template <>
-struct Vec4<double> {
-    __device__ static inline void load(const double *p, double *o) {
-        double2 v0 = *reinterpret_cast<const double2 *>(p);
-        double2 v1 = *reinterpret_cast<const double2 *>(p + 2);
-        o[0] = v0.x; o[1] = v0.y; o[2] = v1.x; o[3] = v1.y;
-    }
-};
+}
 
 __device__ inline float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
@@ -184,13 +189,15 @@ __host__ __device__ constexpr int pow2_at_least(int v) {
 template <typename T, int FORM, int W, int BM, int BN, int TM, int TN, int BK, int STAGES>
 struct GemmCfg {
     static constexpr int NT = (BM / TM) * (BN / TN);   // threads (16 x 16)
-    static constexpr int RG = TM / 4, CG = TN / 4;     // 4-wide fragment groups
+    static constexpr int GR = TM < 4 ? TM : 4, GC = TN < 4 ? TN : 4;   // fragment group widths
+    static constexpr int RG = TM / GR, CG = TN / GC;   // fragment groups
     static constexpr int NCACC = FORM == G_ASYM ? W : 1;
     // running de-companded sums in TMEM (fp32 packed forms) or registers
     static constexpr bool TMEMC = FORM != G_PLAIN && sizeof(T) == 4;
     static constexpr int NC = NCACC * TM * TN;         // sums per thread
     static constexpr int TMEM_COLS = pow2_at_least(2 * NC);
-    static constexpr int MIN_CTAS = TMEMC ? 2 : 1;
+    // fp64: two CTAs per SM, so one's slab end overlaps the other's fma chains
+    static constexpr int MIN_CTAS = (TMEMC || (sizeof(T) == 8 && NC <= 16)) ? 2 : 1;
     static constexpr size_t STAGE_A = (size_t)BK * BM * sizeof(T);
     static constexpr size_t STAGE_B = (size_t)BK * BN * sizeof(T);
     static constexpr size_t RING = STAGES * (STAGE_A + STAGE_B) + STAGES * sizeof(uint64_t) + 16;
@@ -235,12 +242,12 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                        const __grid_constant__ CUtensorMap mapPB, const GemmArgs<T> g) {
     pdl_entry();
     using Cfg = GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES>;
-    constexpr int RG = Cfg::RG, CG = Cfg::CG, NCACC = Cfg::NCACC;
+    constexpr int RG = Cfg::RG, CG = Cfg::CG, GR = Cfg::GR, GC = Cfg::GC, NCACC = Cfg::NCACC;
     constexpr bool TMEMC = Cfg::TMEMC;
     static_assert(!MIX || (FORM == G_SYM && !KEEP), "mixed tiles: symmetric form only");
 
     // the device planner chose another packing
-    if (g.plan->W != W) return;
+    if (g.plan->W != g.W) return;
     // both rounding variants queued: the one the plan does not select exits
     if constexpr (sizeof(T) == 4 && ((FORM == G_SYM && W == 2) || FORM == G_ASYM) && !KEEP) {
         if (g.small_t < 0 && small_round_ok(FORM, W, g.plan->q, g.plan->gA) != SMALL_T) return;
@@ -327,33 +334,35 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
     }
 
     T z = T(1), Q = T(1);
+    int q = 0;
     if (FORM != G_PLAIN) {
-        z = pow2_t(T(0), -g.plan->q);
-        Q = pow2_t(T(0), g.plan->q);
+        q = g.plan->q;
+        z = pow2_t(T(0), -q);
+        Q = pow2_t(T(0), q);
     }
 
     // row-block index of every fragment row (clamped inside the grid): rows
-    // are m (a 4-row group never straddles a block since L % 16 == 0) or, for
+    // are m (a group of up to 4 rows never straddles a block since L % 16 == 0) or, for
     // the asymmetric form, packed rows with P = ceil(L / W) per block, which
     // can straddle when P % 4 != 0 (W = 3)
     int iblk[TM], jblk[CG];
 #pragma unroll
     for (int gi = 0; gi < RG; ++gi)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            long long xr = x0 + gi * (BM / RG) + ty * 4 + e;
+        for (int e = 0; e < GR; ++e) {
+            long long xr = x0 + gi * (BM / RG) + ty * GR + e;
             long long ib = FORM == G_ASYM ? xr / g.P : xr / g.L;
-            iblk[gi * 4 + e] = (int)min(ib, (long long)g.nM - 1);
+            iblk[gi * GR + e] = (int)min(ib, (long long)g.nM - 1);
         }
 #pragma unroll
     for (int hj = 0; hj < CG; ++hj) {
-        long long nc = n0 + hj * (BN / CG) + tx * 4;
+        long long nc = n0 + hj * (BN / CG) + tx * GC;
         jblk[hj] = (int)min(nc / g.L, (long long)g.nN - 1);
     }
 
     // global coordinates of fragment element (i, j), digit d
     auto out_row = [&](int i, int d) -> long long {
-        const long long xr = x0 + (i / 4) * (BM / RG) + ty * 4 + (i % 4);
+        const long long xr = x0 + (i / GR) * (BM / RG) + ty * GR + (i % GR);
         if (FORM == G_ASYM) {
             const long long ib = xr / g.P, jr = xr % g.P;
             const long long inblk = jr * W + d;
@@ -362,7 +371,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
         }
         return xr;
     };
-    auto out_col = [&](int j) -> long long { return n0 + (j / 4) * (BN / CG) + tx * 4 + (j % 4); };
+    auto out_col = [&](int j) -> long long { return n0 + (j / GC) * (BN / CG) + tx * GC + (j % GC); };
     auto store_c = [&](long long row, long long col, T v) {
         if (row < 0 || row >= g.M || col >= g.N) return;
         T *p = g.C + row * g.ldc + col;
@@ -373,6 +382,11 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
     // whole 256-byte row segments, which also keeps C written to host memory
     // over the CPU link in full lines
     auto store_c4 = [&](long long row, long long col, const T *v) {
+        if constexpr (GC < 4) {
+#pragma unroll
+            for (int q = 0; q < GC; ++q) store_c(row, col + q, v[q]);
+            return;
+        }
         const bool c_vec = g.beta_zero && (g.ldc % 4 == 0) &&
                            ((reinterpret_cast<uintptr_t>(g.C) & (4 * sizeof(T) - 1)) == 0);
         if (c_vec && row >= 0 && row < g.M && col + 4 <= g.N) {
@@ -416,10 +430,10 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                     T a[TM], b[TN];
 #pragma unroll
                     for (int gi = 0; gi < RG; ++gi)
-                        Vec4<T>::load(As + kk * BM + gi * (BM / RG) + ty * 4, a + 4 * gi);
+                        frag_load<GR>(As + kk * BM + gi * (BM / RG) + ty * GR, a + GR * gi);
 #pragma unroll
                     for (int hj = 0; hj < CG; ++hj)
-                        Vec4<T>::load(Bs + kk * BN + hj * (BN / CG) + tx * 4, b + 4 * hj);
+                        frag_load<GC>(Bs + kk * BN + hj * (BN / CG) + tx * GC, b + GC * hj);
                     outer_fma(acc, a, b);
                 }
             } else {
@@ -427,10 +441,10 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                     T a[TM], b[TN];
 #pragma unroll
                     for (int gi = 0; gi < RG; ++gi)
-                        Vec4<T>::load(As + kk * BM + gi * (BM / RG) + ty * 4, a + 4 * gi);
+                        frag_load<GR>(As + kk * BM + gi * (BM / RG) + ty * GR, a + GR * gi);
 #pragma unroll
                     for (int hj = 0; hj < CG; ++hj)
-                        Vec4<T>::load(Bs + kk * BN + hj * (BN / CG) + tx * 4, b + 4 * hj);
+                        frag_load<GC>(Bs + kk * BN + hj * (BN / CG) + tx * GC, b + GC * hj);
                     outer_fma(acc, a, b);
                 }
             }
@@ -443,8 +457,8 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
         // (e = i * TN + j the fragment element, d the asymmetric digit).
         const bool first = l == 0;
         // this slab's de-companding factors, all loads issued before any use:
-        // one per 4-row group (sym: a group never straddles a block) or per
-        // packed row (asym), times one per 4-column group
+        // one per row group (sym: a group never straddles a block) or per
+        // packed row (asym), times one per column group
         constexpr int PR = FORM == G_ASYM ? TM : RG;
         T prs[PR][CG];
         const T *pl_tab = g.pair + (long long)l * g.nM * g.nN;
@@ -452,7 +466,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
         for (int pi = 0; pi < PR; ++pi)
 #pragma unroll
             for (int hj = 0; hj < CG; ++hj)
-                prs[pi][hj] = __ldg(pl_tab + (long long)iblk[FORM == G_ASYM ? pi : 4 * pi] * g.nN + jblk[hj]);
+                prs[pi][hj] = __ldg(pl_tab + (long long)iblk[FORM == G_ASYM ? pi : GR * pi] * g.nN + jblk[hj]);
         float v[16];
         if constexpr (KEEP) {
             if (split) {
@@ -460,7 +474,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                 // the ordered sum over slabs runs in the unpack kernel
 #pragma unroll
                 for (int i = 0; i < TM; ++i) {
-                    const long long xr = x0 + (i / 4) * (BM / RG) + ty * 4 + (i % 4);
+                    const long long xr = x0 + (i / GR) * (BM / RG) + ty * GR + (i % GR);
 #pragma unroll
                     for (int j = 0; j < TN; ++j) {
                         const long long nc = out_col(j);
@@ -517,19 +531,25 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
             tmem_wait_st();
             continue;
         }
+        // fp64: the digits by integer arithmetic (tdg_digits.cuh), in 32-bit
+        // words where q allows
+        auto slab_end = [&](auto narrow) {
 #pragma unroll
         for (int e = 0; e < TM * TN; ++e) {
             const int i = e / TN, j = e % TN;
-            const T pr = prs[FORM == G_ASYM ? i : i / 4][j / 4];
+            const T pr = prs[FORM == G_ASYM ? i : i / GR][j / GC];
             const T r = acc[i][j];
             acc[i][j] = T(0);
             if constexpr (KEEP) {
-                const long long xr = x0 + (i / 4) * (BM / RG) + ty * 4 + (i % 4);
+                const long long xr = x0 + (i / GR) * (BM / RG) + ty * GR + (i % GR);
                 const long long nc = out_col(j);
                 if (xr < g.Mrows && nc < g.N) g.Rbar[((long long)l * g.Mrows + xr) * g.N + nc] = r;
             }
             T digit[NCACC];
-            if (FORM == G_SYM) {
+            if constexpr (sizeof(T) == 8) {
+                if constexpr (FORM == G_SYM) digit[0] = sym_digit<decltype(narrow)::value>(r, q);
+                else if constexpr (FORM == G_ASYM) asym_digits<NCACC>(r, q, digit);
+            } else if (FORM == G_SYM) {
                 const T u = rint_epi(r);                        // eq. 9
                 const T t = rint_epi(mul_rn(z, u));
                 digit[0] = fma_rn(-Q, t, u);                    // eq. 10
@@ -549,7 +569,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                     if (slot == 0) {
                         if (first) {
 #pragma unroll
-                            for (int q = 0; q < 16; ++q) v[q] = 0.f;
+                            for (int k = 0; k < 16; ++k) v[k] = 0.f;
                         } else {
                             tmem_ld16(tcol + (uint32_t)f, v);
                         }
@@ -560,6 +580,13 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                     cacc[d][i][j] = fma_rn(digit[d], pr, cacc[d][i][j]);
                 }
             }
+        }
+        };
+        if constexpr (sizeof(T) == 8 && FORM == G_SYM) {
+            if (q <= 31) slab_end(std::true_type{});
+            else slab_end(std::false_type{});
+        } else {
+            slab_end(std::false_type{});
         }
         if constexpr (TMEMC) tmem_wait_st();
     }
@@ -577,7 +604,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
         for (int i = 0; i < TM; ++i) {
             const long long row = out_row(i, 0);
 #pragma unroll
-            for (int j = 0; j < TN; j += 4) store_c4(row, out_col(j), &acc[i][j]);
+            for (int j = 0; j < TN; j += GC) store_c4(row, out_col(j), &acc[i][j]);
         }
     } else if constexpr (TMEMC) {
         // ------------------------------------------------------------ store C
@@ -612,7 +639,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
             for (int d = 0; d < NCACC; ++d) {
                 const long long row = out_row(i, d);
 #pragma unroll
-                for (int j = 0; j < TN; j += 4)
+                for (int j = 0; j < TN; j += GC)
                     store_c4(row, out_col(j), FORM == G_PLAIN ? &acc[i][j] : &cacc[d][i][j]);
             }
     }
@@ -677,7 +704,7 @@ cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStre
 // that code.
 template <typename T, int FORM, int W, typename C>
 cudaError_t launch_cfg(const GemmArgs<T> &g, const GemmOperands &ops, cudaStream_t st) {
-    if constexpr (FORM == G_SYM) {
+    if constexpr (FORM == G_SYM && C::TM >= 4) {
         if (g.kmask) {
             if (g.Rbar || !ops.pa.base || !ops.pb.base) return cudaErrorInvalidValue;
             if constexpr (sizeof(T) == 4 && W == 2) {
@@ -692,7 +719,9 @@ cudaError_t launch_cfg(const GemmArgs<T> &g, const GemmOperands &ops, cudaStream
         }
     }
     if (g.kmask) return cudaErrorInvalidValue;
-    if (FORM != G_PLAIN && g.Rbar) return launch_grid<T, FORM, W, C, true, false>(g, ops, st);
+    if constexpr (FORM != G_PLAIN) {
+        if (g.Rbar) return launch_grid<T, FORM, W, C, true, false>(g, ops, st);
+    }
     if (g.groups > 1) return cudaErrorInvalidValue;     // slab splitting stores r-bar
     if constexpr (sizeof(T) == 4 && ((FORM == G_SYM && W == 2) || (FORM == G_ASYM && W >= 2))) {
         // the unpack's roundings as a compile-time variant: known on the host

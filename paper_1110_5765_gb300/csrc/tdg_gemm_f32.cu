@@ -10,8 +10,11 @@ static cudaError_t go(const GemmArgs<float> &g, const GemmOperands &ops, cudaStr
 }
 
 template <>
-cudaError_t launch_packed_gemm<float>(int form, int W, const GemmArgs<float> &g,
+cudaError_t launch_packed_gemm<float>(int form, int W, const GemmArgs<float> &g0,
                                       const GemmOperands &ops, cudaStream_t st) {
+    if (W < 1 || W > kMaxW) return cudaErrorNotSupported;
+    GemmArgs<float> g = g0;
+    g.W = W;
     using S = TilesF32;
     using A = TilesF32Asym;
     using A2 = TilesF32AsymW2;
@@ -21,12 +24,8 @@ cudaError_t launch_packed_gemm<float>(int form, int W, const GemmArgs<float> &g,
         return go<G_PLAIN, 1, S>(g, ops, st);
     }
     if (form == G_SYM) {
-        switch (W) {
-            case 1: return go<G_SYM, 1, S>(g, ops, st);
-            case 2: return go<G_SYM, 2, S>(g, ops, st);
-            case 3: return go<G_SYM, 3, S>(g, ops, st);
-            case 4: return go<G_SYM, 4, S>(g, ops, st);
-        }
+        // W = 2 has the add-subtract rounding variant; the others share a kernel
+        return W == 2 ? go<G_SYM, 2, S>(g, ops, st) : go<G_SYM, 1, S>(g, ops, st);
     }
     if (form == G_ASYM) {
         switch (W) {

@@ -5,30 +5,26 @@
 
 namespace tdg {
 
-template <int FORM, int W, typename C>
+template <int FORM, int W>
 static cudaError_t go(const GemmArgs<double> &g, const GemmOperands &ops, cudaStream_t st) {
-    return launch_cfg<double, FORM, W, C>(g, ops, st);
+    return launch_cfg<double, FORM, W, TilesF64>(g, ops, st);
 }
 
 template <>
-cudaError_t launch_packed_gemm<double>(int form, int W, const GemmArgs<double> &g,
+cudaError_t launch_packed_gemm<double>(int form, int W, const GemmArgs<double> &g0,
                                        const GemmOperands &ops, cudaStream_t st) {
-    using D = TilesF64;
-    if (form == G_PLAIN) return go<G_PLAIN, 1, D>(g, ops, st);
-    if (form == G_SYM) {
-        switch (W) {
-            case 1: return go<G_SYM, 1, D>(g, ops, st);
-            case 2: return go<G_SYM, 2, D>(g, ops, st);
-            case 3: return go<G_SYM, 3, D>(g, ops, st);
-            case 4: return go<G_SYM, 4, D>(g, ops, st);
-        }
-    }
+    if (W < 1 || W > kMaxW) return cudaErrorNotSupported;
+    GemmArgs<double> g = g0;
+    g.W = W;
+    if (form == G_PLAIN) return go<G_PLAIN, 1>(g, ops, st);
+    // the symmetric kernel is the same for every W
+    if (form == G_SYM) return go<G_SYM, 1>(g, ops, st);
     if (form == G_ASYM) {
         switch (W) {
-            case 1: return go<G_ASYM, 1, D>(g, ops, st);
-            case 2: return go<G_ASYM, 2, D>(g, ops, st);
-            case 3: return go<G_ASYM, 3, D>(g, ops, st);
-            case 4: return go<G_ASYM, 4, D>(g, ops, st);
+            case 1: return go<G_ASYM, 1>(g, ops, st);
+            case 2: return go<G_ASYM, 2>(g, ops, st);
+            case 3: return go<G_ASYM, 3>(g, ops, st);
+            case 4: return go<G_ASYM, 4>(g, ops, st);
         }
     }
     return cudaErrorNotSupported;

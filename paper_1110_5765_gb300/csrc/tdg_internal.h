@@ -119,6 +119,7 @@ struct GemmArgs {
     // starting them first keeps the last wave short)
     const int *tile_order;
     const T *cApx, *cBpx;   // pair-exact companders [(i nK + l) nN + j] (else unused)
+    int W;                  // set by the launcher: the packing this launch computes (1: plain)
     int ntn;                // set by the launcher: tiles per row of the 1-D tile grid
     long long ntiles;       // set by the launcher: tiles in the grid
     // slab splitting (needs Rbar): > 1 asks for that many groups of slabs, each

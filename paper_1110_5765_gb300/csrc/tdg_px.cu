@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(PxCfg<T, W, C>::NT, sizeof(T) == 4 ? 2 : 1)
 #pragma unroll
             for (int j = 0; j < TN; ++j) cacc[i][j] = T(0);
     }
-    const T z = pow2_t(T(0), -g.plan->q), Q = pow2_t(T(0), g.plan->q);
+    const int q = g.plan->q;
+    const T z = pow2_t(T(0), -q), Q = pow2_t(T(0), q);
 
     bool ok = true;
     T ca = T(0), cb = T(0);
@@ -198,10 +199,10 @@ __global__ void __launch_bounds__(PxCfg<T, W, C>::NT, sizeof(T) == 4 ? 2 : 1)
             T a[TM], b[TN];
 #pragma unroll
             for (int gi = 0; gi < RG; ++gi)
-                Vec4<T>::load(pkA + kk * PA + gi * (BM / RG) + ty * 4, a + 4 * gi);
+                frag_load<4>(pkA + kk * PA + gi * (BM / RG) + ty * 4, a + 4 * gi);
 #pragma unroll
             for (int hj = 0; hj < CG; ++hj)
-                Vec4<T>::load(pkB + kk * BN + hj * (BN / CG) + tx * 4, b + 4 * hj);
+                frag_load<4>(pkB + kk * BN + hj * (BN / CG) + tx * 4, b + 4 * hj);
             outer_fma(acc, a, b);
         }
         if (s != sps - 1) continue;
@@ -215,15 +216,20 @@ __global__ void __launch_bounds__(PxCfg<T, W, C>::NT, sizeof(T) == 4 ? 2 : 1)
             const int i = e / TN, j = e % TN;
             const T r = acc[i][j];
             acc[i][j] = T(0);
-            const T u = rint_epi(r);                        // eq. 9
-            const T t = rint_epi(mul_rn(z, u));
-            const T digit = fma_rn(-Q, t, u);               // eq. 10
+            T digit;
+            if constexpr (sizeof(T) == 8) {
+                digit = sym_digit<false>(r, q);             // eqs. 9-10 in integers
+            } else {
+                const T u = rint_epi(r);                    // eq. 9
+                const T t = rint_epi(mul_rn(z, u));
+                digit = fma_rn(-Q, t, u);                   // eq. 10
+            }
             if constexpr (TMEMC) {
                 const int slot = e % 16;
                 if (slot == 0) {
                     if (first) {
 #pragma unroll
-                        for (int q = 0; q < 16; ++q) v[q] = 0.f;
+                        for (int k = 0; k < 16; ++k) v[k] = 0.f;
                     } else {
                         tmem_ld16(tcol + (uint32_t)e, v);
                     }

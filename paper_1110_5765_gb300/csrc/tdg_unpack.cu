@@ -11,6 +11,7 @@
 //
 // tdgemm_snr: fp64 sums of ref^2, (C - ref)^2 and (C - ref) for eq. 20.
 #include "tdg_common.cuh"
+#include "tdg_digits.cuh"
 #include "tdg_internal.h"
 
 namespace tdg {
@@ -48,7 +49,16 @@ __global__ void unpack_kernel(GemmArgs<T> g, int W, int64_t *rint_out) {
         for (int l = 0; l < g.nK; ++l) {
             const T rbar = g.Rbar[((long long)l * g.Mrows + xr) * g.N + n];
             T rt;
-            if (ASYM) {
+            if constexpr (sizeof(T) == 8) {
+                // digits in integer arithmetic, as the fused epilogue takes them
+                if constexpr (ASYM) {
+                    double dg[kMaxW];
+                    asym_digits<kMaxW>(rbar, q, dg);
+                    rt = d == 0 ? dg[0] : d == 1 ? dg[1] : d == 2 ? dg[2] : dg[3];
+                } else {
+                    rt = sym_digit<false>(rbar, q);
+                }
+            } else if (ASYM) {
                 T x = rbar;
                 rt = rint_d(x);
                 for (int k = 0; k < d; ++k) {
