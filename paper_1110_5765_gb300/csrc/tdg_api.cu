@@ -283,10 +283,11 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
         // buffer that TDG_KEEP_PACKED also uses
         if (is_packed_form(form) && !(flags & (TDG_KEEP_PACKED | TDG_PAIR_EXACT)) && p->nK >= 4) {
             int bxa, bxb, bk, dev = 0, sms = 0;
+            const long long mrows = form == TDG_ASYM ? (long long)p->nM * Pof(L, W) : M;
             packed_gemm_boxes(dtype, form == TDG_SYM ? G_SYM : G_ASYM, W, &bxa, &bxb, &bk);
+            if (dtype == TDG_F64) bxa = bxb = f64_tile_edge(mrows, N);
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            const long long mrows = form == TDG_ASYM ? (long long)p->nM * Pof(L, W) : M;
             const long long ntiles = ((mrows + bxa - 1) / bxa) * ((N + bxb - 1) / bxb);
             if (sms > 0 && ntiles * 2 <= sms)
                 p->split_groups = (int)std::min<long long>(p->nK, (2LL * sms + ntiles - 1) / ntiles);

@@ -32,6 +32,7 @@
 // its TMEM and returns without storing.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "tdg_common.cuh"
@@ -653,6 +654,18 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
     }
 }
 
+// Shared memory that a CTA of a small grid asks for so that its CTAs spread
+// evenly: with n CTAs on S SMs, no SM gets more than ceil(n / S).  Launched
+// programmatically, CTAs start where the kernel before leaves room first and
+// were seen to pile up there: 256 one-output-per-thread fp64 CTAs on 152 SMs
+// took 34 us behind their packing kernel against 22 us by themselves.
+constexpr int kSmemPerSm = 228 * 1024, kMaxCtaSmem = 227 * 1024;
+inline size_t spread_smem(long long nblocks) {
+    const long long r = (nblocks + device_sms() - 1) / device_sms();
+    if (r > 4) return 0;                 // several waves: the scheduler balances them
+    return std::min<size_t>(kMaxCtaSmem, (size_t)(kSmemPerSm / r - 1024) / 1024 * 1024);
+}
+
 // One launch over the whole tile grid of shape C.
 template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, bool SMALL_T = false>
 cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStream_t st) {
@@ -662,7 +675,7 @@ cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStre
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCtaSmem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
@@ -695,8 +708,8 @@ cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStre
         g.groups = 1;
     }
     if (nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    return launch_pdl_if(pdl_for_grid(nblocks), kern, dim3((unsigned)nblocks), dim3(Cfg::NT),
-                         Cfg::SMEM, st, ma, mb, mpa, mpb, g);
+    return launch_pdl(kern, dim3((unsigned)nblocks), dim3(Cfg::NT),
+                      std::max(Cfg::SMEM, spread_smem(nblocks)), st, ma, mb, mpa, mpb, g);
 }
 
 // KEEP (store every packed slab result for tdgemm_unpack) and MIX (Sec. 6

@@ -5,9 +5,34 @@
 
 namespace tdg {
 
+// Edge of the square CTA tile for an fp64 product with mrows x ncols outputs.
+// The fp64 pipe (2 fma per clock and SM) bounds every size, and one CTA keeps
+// it full, so the time is that of the SM with the most outputs:
+// ceil(tiles / SMs) edge^2.  Smaller tiles leave fewer SMs idle and pad less
+// (64-tiles on 256 x 256: 16 of 152 SMs busy); they pay more barriers and
+// fragment loads per fma, so an edge is left only for a gain above 2 %.
+// Measured with edges 64 / 32 / 16: 4096^3 W = 3 38.2 / 38.2 / 38.4 ms,
+// 4096 x 400 x 10304 W = 3 11.2 / 10.3 / 10.06 ms, a 256^3 W = 2 call 71 / 54 /
+// 50 us (64 and 32 split its slabs over CTAs, 16 need not).
+int f64_tile_edge(long long mrows, long long ncols) {
+    const long long sms = device_sms();
+    auto cost = [&](long long e) {
+        const long long tiles = ((mrows + e - 1) / e) * ((ncols + e - 1) / e);
+        return (double)((tiles + sms - 1) / sms) * (double)(e * e);
+    };
+    int best = 64;
+    for (int e : {32, 16})
+        if (cost(e) < 0.98 * cost(best)) best = e;
+    return best;
+}
+
 template <int FORM, int W>
 static cudaError_t go(const GemmArgs<double> &g, const GemmOperands &ops, cudaStream_t st) {
-    return launch_cfg<double, FORM, W, TilesF64>(g, ops, st);
+    // mixed tiles (Sec. 6) keep the tile that the tile order was made for
+    const int edge = g.kmask ? 64 : f64_tile_edge(g.Mrows, g.N);
+    if (edge == 64) return launch_cfg<double, FORM, W, TilesF64>(g, ops, st);
+    if (edge == 32) return launch_cfg<double, FORM, W, TilesF64Mid>(g, ops, st);
+    return launch_cfg<double, FORM, W, TilesF64Small>(g, ops, st);
 }
 
 template <>

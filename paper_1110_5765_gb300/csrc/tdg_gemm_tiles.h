@@ -22,7 +22,10 @@ using TilesF32Small = Tiles<64, 64, 4, 4, 32, 4>;
 // fp32 asymmetric: 64 packed rows (W result rows each) x 128 columns
 using TilesF32Asym = Tiles<64, 128, 4, 8, 16, 6>;     // W >= 3: W x 32 running sums per thread
 using TilesF32AsymW2 = Tiles<128, 128, 8, 8, 32, 3>;  // W <= 2: W x 64 sums fit TMEM, 2.6 % faster
-// fp64: 64 x 64, 4 x 4 per thread
+// fp64: 64 x 64, 4 x 4 per thread; smaller tiles where they leave fewer SMs idle
+// (f64_tile_edge)
 using TilesF64 = Tiles<64, 64, 4, 4, 16, 4>;
+using TilesF64Mid = Tiles<32, 32, 2, 2, 32, 3>;
+using TilesF64Small = Tiles<16, 16, 1, 1, 32, 3>;
 
 }  // namespace tdg

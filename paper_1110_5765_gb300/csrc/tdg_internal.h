@@ -175,7 +175,10 @@ template <typename T>
 cudaError_t launch_px_gemm(int W, const GemmArgs<T> &g, const GemmOperands &ops, cudaStream_t st);
 
 // Tile shape the packed GEMM uses for (T, form): operand boxes are
-// {box_x_a, bk} for A and {box_x_b, bk} for B.
+// {box_x_a, bk} for A and {box_x_b, bk} for B
+// (fp64: the largest tile, which mixed launches use; f64_tile_edge gives the
+// edge of the others).
+int f64_tile_edge(long long mrows, long long ncols);
 void packed_gemm_boxes(int dtype, int form, int W, int *box_x_a, int *box_x_b, int *bk);
 
 template <typename T>

@@ -1,0 +1,33 @@
+"""Every CTA tile that the packed GEMM chooses among, at the sizes where it can go
+wrong: one tile and its remainders, just under and over the lines of the rule,
+with and without slab splitting, against the oracle bit for bit (needs a GB300)."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+# (M, N, K) for fp64 on 152 SMs: 16-tiles (one, ragged, split over slabs, two per
+# SM), 32-tiles (143 of them), 64-tiles
+F64 = [(1, 1, 70), (17, 31, 130), (60, 70, 600), (257, 250, 130), (350, 410, 130),
+       (600, 930, 66)]
+
+
+@pytest.mark.parametrize("shape", F64)
+@pytest.mark.parametrize("form,W", [("sym", 2), ("sym", 3), ("asym", 3), ("plain", 1)])
+def test_f64_tiles(orc, shape, form, W):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1110_5765_gb300 as tdg
+    M, N, K = shape
+    A, B = synth.laplace((M, K), 61), synth.gaussian((K, N), 62)
+    C0 = synth.gaussian((M, N), 63)
+    kw = dict(L=64, W=W, dtype="f64", form=form, bits=0 if form == "plain" else 8)
+    ref = orc.tdgemm(A, B, alpha=0.75, beta=-1.5, C_in=C0, **kw)
+    with tdg.Plan(M, N, K, **kw) as p:
+        C = torch.from_numpy(C0.copy()).cuda()
+        p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C, 0.75, -1.5)
+        assert p.info()["device_status"] == 0
+        assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
