@@ -14,6 +14,7 @@
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
 #include "tdg_pack.h"
+#include "tdg_planner.cuh"
 #include "tdgemm.h"
 
 using namespace tdg;
@@ -91,6 +92,8 @@ struct tdgemm_plan_s {
     size_t ws_bytes = 0;
     DevPlan *dplan = nullptr;
     double *mA, *eA, *mB, *eB, *sA, *sB, *stab, *agg;
+    unsigned int *slab_done = nullptr;    // [nK], zero between calls
+    bool clear_record = false;            // a pack failed half-way: counters to zero first
     void *cA, *cB, *pair;
     void *Abuf, *Bbuf, *Rbar;
     void *cApx = nullptr, *cBpx = nullptr, *pairpx = nullptr;   // TDG_PAIR_EXACT
@@ -256,6 +259,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     const size_t nAblk = (size_t)p->nM * p->nK, nBblk = (size_t)p->nK * p->nN;
     size_t off = 0;
     size_t o_plan = off; off += up(sizeof(DevPlan));
+    size_t o_done = off; off += up((size_t)p->nK * sizeof(unsigned int));
     size_t o_agg = off;
     off += up(((size_t)4 * p->nK + (size_t)kLevelRecDoubles * (kMaxW - 1) * kMaxLevels) * 8);
     size_t o_mA = off; off += up(nAblk * 8);
@@ -323,6 +327,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
         return fail(TDG_ECUDA, "cudaMemset: %s", cudaGetErrorString(e));
     }
     p->dplan = (DevPlan *)(p->ws + o_plan);
+    p->slab_done = (unsigned int *)(p->ws + o_done);
     p->agg = (double *)(p->ws + o_agg);
     p->mA = (double *)(p->ws + o_mA); p->eA = (double *)(p->ws + o_eA);
     p->mB = (double *)(p->ws + o_mB); p->eB = (double *)(p->ws + o_eB);
@@ -497,39 +502,40 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
                             bool reuse_b = false) {
     // reuse_b: B, its statistics, companders and packed copy are those of the
     // previous pack (the caller keeps B unchanged); only A is processed
-    CU_TRY(cudaMemsetAsync(p->dplan, 0, sizeof(DevPlan), st));
+    // the record and its counters are zero where they must be after every
+    // complete call (and at the plan's creation), so a call clears them only
+    // when the one before it failed between its launches
+    if (p->clear_record) {
+        CU_TRY(cudaMemsetAsync(p->dplan, 0, sizeof(DevPlan), st));
+        CU_TRY(cudaMemsetAsync(p->slab_done, 0, (size_t)p->nK * sizeof(unsigned int), st));
+    }
+    p->clear_record = true;               // until every launch below is queued
     if (p->stab_dirty) {
         CU_TRY(cudaMemcpyAsync(p->stab, p->stab_host.data(), p->stab_host.size() * 8,
                                cudaMemcpyHostToDevice, st));
         p->stab_dirty = false;
     }
     const bool nA = p->tA == 'N', nB = p->tB == 'N';
+    PlanParams pp = params_of(p);
+    const double *stab = p->have_table ? p->stab : nullptr;
+    const SlabFinish fin{pp, p->mA, p->eA, p->mB, p->eB, stab, p->agg, p->slab_done,
+                         (unsigned int)(p->nM + (reuse_b ? 0 : p->nN))};
     // tensor-core forms whose compander is gamma / max|x| of the block alone:
     // statistics, companders and codes in one pass over each input
-    const bool tc_fused = is_tc_form(p->form) && p->mode == MODE_FIXED && p->L <= 128 &&
-                          p->L % 64 == 0;
+    const bool tc_fused = is_tc_form(p->form) && p->mode == MODE_FIXED &&
+                          (p->L == 128 || p->L == 64);
     if (tc_fused) {
-        if constexpr (sizeof(T) == 4) {
-            const long long ldk = round_up(p->K, 128);
-            const int fp8 = p->form == TDG_TC_FP8;
-            const double gamma = fp8 ? kFp8Max : (double)((1 << (p->bits - 1)) - 1);
-            PackOperand<float> oa = operand_A<float>(p, A, nullptr);
-            PackOperand<float> ob = operand_B<float>(p, B, nullptr);
-            CU_TRY(launch_codes_stats(oa, p->mA, p->eA, (float *)p->cA, p->sA, p->Abuf,
-                                      reuse_b ? nullptr : &ob, p->mB, p->eB, (float *)p->cB,
-                                      p->sB, p->Bbuf, fp8, gamma, ldk, p->dplan, st));
-        }
+        // with the codes, below
     } else if (p->form != TDG_PLAIN && p->mode != MODE_MANUAL) {
         // stats of op(A): stored rows x cols; op block grid nM x nK
         CU_TRY(launch_block_stats<T>(A, nA ? p->M : p->K, nA ? p->K : p->M, p->lda, nA ? 0 : 1,
                                      p->nK, p->mA, p->eA, B, reuse_b ? 0 : (nB ? p->K : p->N),
                                      nB ? p->N : p->K, p->ldb, nB ? 0 : 1, p->nN, p->mB, p->eB,
-                                     p->L, p->dplan, st));
+                                     p->L, p->dplan, fin, st));
     }
-    PlanParams pp = params_of(p);
-    const double *stab = p->have_table ? p->stab : nullptr;
-    CU_TRY(launch_planner<T>(pp, p->mA, p->eA, p->mB, p->eB, stab, p->dplan, p->agg, (T *)p->cA,
-                             p->sA, (T *)p->cB, p->sB, (T *)p->pair, st, tc_fused));
+    if (!is_tc_form(p->form))
+        CU_TRY(launch_planner<T>(pp, p->mA, p->eA, p->mB, p->eB, stab, p->dplan, p->agg,
+                                 (T *)p->cA, p->sA, (T *)p->cB, p->sB, (T *)p->pair, st));
     const bool px = (p->flags & TDG_PAIR_EXACT) != 0;
     if (px)
         CU_TRY(launch_px_scales<T>(pp, p->mA, p->eA, p->mB, p->eB, p->dplan, (T *)p->cApx,
@@ -556,16 +562,14 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
     }
     if (is_tc_form(p->form)) {
         if constexpr (sizeof(T) == 4) {
-            if (!tc_fused) {       // (the fused path wrote the codes with the statistics)
-                const long long ldk = round_up(p->K, 128);
-                const int fp8 = p->form == TDG_TC_FP8;
-                // B first, as for the packs: its blocks were read last
-                if (!reuse_b)
-                    CU_TRY(launch_codes(operand_B<float>(p, B, (const float *)p->cB), fp8,
-                                        p->Bbuf, ldk, st));
-                CU_TRY(launch_codes(operand_A<float>(p, A, (const float *)p->cA), fp8, p->Abuf,
-                                    ldk, st));
-            }
+            const int fp8 = p->form == TDG_TC_FP8;
+            // (target mode: the plan's gammas)
+            const double gamma =
+                fp8 ? kFp8Max : p->bits > 0 ? (double)((1 << (p->bits - 1)) - 1) : 0.0;
+            const PackOperand<float> ob = operand_B<float>(p, B, nullptr);
+            CU_TRY(launch_codes(operand_A<float>(p, A, nullptr), p->mA, p->eA, p->sA, p->Abuf,
+                                reuse_b ? nullptr : &ob, p->mB, p->eB, p->sB, p->Bbuf, fp8,
+                                tc_fused, gamma, round_up(p->K, 128), p->dplan, fin, st));
         }
     } else {
         for (int w : candidates(p)) {
@@ -602,6 +606,7 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
             }
         }
     }
+    p->clear_record = false;
     p->A_user = A;
     p->B_user = B;
     p->packed = true;
@@ -741,7 +746,7 @@ extern "C" tdg_status tdgemm_gemm(tdgemm_plan_t p, void *C, double alpha, double
         TcArgs a;
         a.plan = p->dplan; a.M = p->M; a.N = p->N; a.K = p->K;
         a.L = p->L; a.nM = p->nM; a.nK = p->nK; a.nN = p->nN;
-        a.pair = (const float *)p->pair; a.C = (float *)C; a.ldc = p->ldc;
+        a.sA = p->sA; a.sB = p->sB; a.C = (float *)C; a.ldc = p->ldc;
         a.alpha = (float)alpha; a.beta = (float)beta; a.beta_zero = beta == 0.0;
         // C through TMA stores where it can be mapped (beta = 0 and 16-byte
         // aligned rows), else through plain stores

@@ -29,14 +29,16 @@ struct DevPlan {
     int Wef;           // eq. 16
     int level;         // chosen R_max level (target mode), -1 otherwise
     int status;        // tdg_status raised on the device (0 = ok)
-    int nonfinite;     // set by the statistics kernel
+    int nonfinite;     // NaN or Inf among the inputs of the last pack
     double pred_snr;   // model SNR (dB), NaN if not modelled
     double s_rep;      // representation-noise RMSE the model used (0 if none)
     double S, T1, T2, T3;  // noise-model aggregates
+    // zero between calls (the decision, which writes the record, leaves them so)
     unsigned int levels_done;  // candidate-level CTAs finished (the last one decides)
-    // planner inputs, written by the last per-slab aggregate CTA before the
-    // decision: the slab sums S, T1, T2, T3 (unscaled) and rho = sqrt(T2 / T1)
-    unsigned int aggs_done;
+    unsigned int slabs_done;   // slabs whose aggregates are written
+    int nonfinite_seen;        // set by the statistics kernels
+    // target mode, written by the statistics' last warp: the slab sums S, T1,
+    // T2, T3 (unscaled) and rho = sqrt(T2 / T1)
     double tS, tT1, tT2, tT3, trho;
 };
 
@@ -48,14 +50,15 @@ __device__ inline void slab_aggregate_warp(int l, int nM, int nK, int nN,
                                            const double *mB, const double *vB, double *agg) {
     const int lane = threadIdx.x & 31;
     double X = 0, MA = 0, Y = 0, MB = 0;
+    // (written by other CTAs of the same grid: read from L2)
     for (int i = lane; i < nM; i += 32) {
-        X += vA[(long long)i * nK + l];
-        const double m = mA[(long long)i * nK + l];
+        X += __ldcg(&vA[(long long)i * nK + l]);
+        const double m = __ldcg(&mA[(long long)i * nK + l]);
         MA += m * m;
     }
     for (int j = lane; j < nN; j += 32) {
-        Y += vB[(long long)l * nN + j];
-        const double m = mB[(long long)l * nN + j];
+        Y += __ldcg(&vB[(long long)l * nN + j]);
+        const double m = __ldcg(&mB[(long long)l * nN + j]);
         MB += m * m;
     }
 #pragma unroll

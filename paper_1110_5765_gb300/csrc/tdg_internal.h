@@ -23,7 +23,10 @@ struct PackOperand {
     int L;
 };
 
-// Per L x L block max|x| and sigma^2 of op(A) and op(B), one launch.  Each
+struct SlabFinish;     // tdg_planner.cuh: what the statistics' last warps do
+
+// Per L x L block max|x| and sigma^2 of op(A) and op(B), one launch, and the
+// sums over them that the planner needs (fin).  Each
 // operand is given as stored (rows_s x cols_s, leading dimension ld) with
 // trans = 1 when op() transposes it; nbc = block columns of op(); results
 // go to mx / var at op() block index i * nbc + j.
@@ -32,20 +35,19 @@ cudaError_t launch_block_stats(const T *A, long long rows_a, long long cols_a, l
                                int trans_a, int nbc_a, double *mxA, double *varA, const T *B,
                                long long rows_b, long long cols_b, long long ldb, int trans_b,
                                int nbc_b, double *mxB, double *varB, int L, DevPlan *plan,
-                               cudaStream_t st);
+                               const SlabFinish &fin, cudaStream_t st);
 
-// Planner: per-slab aggregates into agg (4 nK + kLevelRecDoubles (kMaxW - 1)
-// kMaxLevels doubles of workspace: the aggregates, then one record per
-// candidate (W, level)), the
+// Planner, after the statistics (which leave the sums over slabs in the plan
+// record or, outside target mode, the plan): agg is 4 nK + kLevelRecDoubles
+// (kMaxW - 1) kMaxLevels doubles of workspace, the per-slab aggregates and one
+// record per candidate (W, level).  Writes the
 // choice of W / z / companders into *plan, then c, s per block and the
 // de-companding factors.
-// scales_done: c and s per block were already written (the fused tensor-core
-// path), so the compander kernel is not launched.
 template <typename T>
 cudaError_t launch_planner(const PlanParams &pp, const double *mA, const double *eA,
                            const double *mB, const double *eB, const double *stab,
                            DevPlan *plan, double *agg, T *cA, double *sA, T *cB, double *sB,
-                           T *pair, cudaStream_t st, bool scales_done = false);
+                           T *pair, cudaStream_t st);
 
 // Launch order of the tiles of a mixed (Sec. 6) launch: the tiles of
 // unaccelerated inner kernels first, then the accelerated ones, each group in
@@ -82,18 +84,15 @@ template <typename T>
 cudaError_t launch_pack_x(const PackOperand<T> &o, int W, const DevPlan *plan, int expectW,
                           int wsign, T *out, long long ldo, cudaStream_t st);
 
-cudaError_t launch_codes(const PackOperand<float> &o, int fp8, void *out, long long ldo,
-                         cudaStream_t st);
-
-// Tensor-core forms whose compander depends only on the block's own maximum
-// (c = gamma / max|x|: fixed bits, or gamma = 448 for E4M3): statistics,
-// companders (c in fp32, s = 1/c in fp64) and codes of op(A) and, when b is
-// given, op(B) in one launch reading each input once.  L in {64, 128}.
-cudaError_t launch_codes_stats(const PackOperand<float> &a, double *mxA, double *varA,
-                               float *cA, double *sA, void *outA, const PackOperand<float> *b,
-                               double *mxB, double *varB, float *cB, double *sB, void *outB,
-                               int fp8, double gamma, long long ldo, DevPlan *plan,
-                               cudaStream_t st);
+// Codes of op(A) and, when b is given, op(B) for the tensor-core forms, with s =
+// 1/c in fp64 per block.  fused: companders of the block's own maximum (c =
+// gamma / max|x|: fixed bits, or gamma = 448 for E4M3), L in {64, 128}: the
+// statistics too, reading each input once, and the plan's decision.  Else the
+// block maxima in mx and the plan's gammas give c.
+cudaError_t launch_codes(const PackOperand<float> &a, double *mxA, double *varA, double *sA,
+                         void *outA, const PackOperand<float> *b, double *mxB, double *varB,
+                         double *sB, void *outB, int fp8, bool fused, double gamma, long long ldo,
+                         DevPlan *plan, const SlabFinish &fin, cudaStream_t st);
 
 // Arguments of the CUDA-core packed GEMM (steps c and d).
 template <typename T>
@@ -197,7 +196,7 @@ struct TcArgs {
     const DevPlan *plan;
     long long M, N, K;
     int L, nM, nK, nN;
-    const float *pair;
+    const double *sA, *sB;    // 1/c per block: s_A[i nK + l], s_B[l nN + j]
     float *C;
     long long ldc;
     float alpha, beta;

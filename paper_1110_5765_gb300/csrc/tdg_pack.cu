@@ -16,18 +16,9 @@
 //                      shared memory with vector loads, then written along x.
 //   pack along x   out[k][i P + j]  (eq. 11, asymmetric A), tile staged in
 //                  shared memory.
-//   k-major codes  out[x][k] (tensor-core forms): integer-valued fp16, or E4M3
-//                  (round to nearest even, saturating).
-//   fused codes    for companders that depend on their own block only (fixed
-//                  bits, E4M3) and L <= 128: one 512-thread CTA per block
-//                  reads it once into registers, reduces max|x| and sum x^2,
-//                  writes c and s and encodes the codes.
 // P = ceil(L / W) packed numbers per block.  Each kernel first reads the
 // device plan and returns unless the planner chose its packing; the grids are
 // capped and loop over tiles so that such early exits cost little.
-#include <cuda_fp16.h>
-#include <cuda_fp8.h>
-
 #include <mutex>
 
 #include "tdg_common.cuh"
@@ -402,325 +393,6 @@ __global__ void __launch_bounds__(256) pack_x_kernel(Src<T> S, int P, const DevP
     }
 }
 
-// ------------------------------------------------------------------ k-major codes
-// out[x][k] as integer-valued fp16 or E4M3; the compander of a 64 x 64 tile
-// is one value (tiles are 64-aligned and L % 64 == 0)
-template <int FP8>
-__device__ inline void encode8(const float *v, unsigned char *dst) {
-    if constexpr (FP8) {
-        uint2 w;
-        uint32_t b[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) b[i] = __nv_cvt_float_to_fp8(v[i], __NV_SATFINITE, __NV_E4M3);
-        w.x = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
-        w.y = b[4] | (b[5] << 8) | (b[6] << 16) | (b[7] << 24);
-        *reinterpret_cast<uint2 *>(dst) = w;
-    } else {
-        __half h[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) h[i] = __float2half_rn(rintf(v[i]));
-        *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(h);
-    }
-}
-
-// k contiguous in the input: one item = 8 consecutive k of one row x
-template <int FP8>
-__global__ void __launch_bounds__(256) codes_kc_kernel(Src<float> S, unsigned char *out,
-                                                       long long ldo, int vec_ok) {
-    pdl_entry();
-    constexpr int ES = FP8 ? 1 : 2;
-    const long long nk8 = (S.K + 7) / 8;
-    const long long items = S.X * nk8;
-    for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < items;
-         it += (long long)gridDim.x * blockDim.x) {
-        const long long x = it / nk8, k = (it - x * nk8) * 8;
-        const float c = S.c[(x / S.L) * S.cx + (k / S.L) * S.cl];
-        const float *src = S.p + x * S.sx + k;
-        float v[8];
-        if (vec_ok && k + 8 <= S.K) {
-            float4 a = __ldg(reinterpret_cast<const float4 *>(src));
-            float4 b = __ldg(reinterpret_cast<const float4 *>(src + 4));
-            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-        } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = (k + i < S.K) ? src[i] : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = __fmul_rn(v[i], c);
-        unsigned char *dst = out + (x * ldo + k) * ES;
-        if (k + 8 <= ldo) {
-            encode8<FP8>(v, dst);   // ldo is padded to 128: the tail lands in padding
-        }
-    }
-}
-
-// x contiguous in the input: 64 x 64 tiles transposed through shared memory
-// (s[k][x], pitch 65: the row-wise writes and the column-wise reads of the
-// store phase are free of bank conflicts).  A thread issues its four 16-byte
-// loads of a tile before it uses any of them.  256 threads per CTA.
-template <int FP8>
-__global__ void __launch_bounds__(256) codes_xc_kernel(Src<float> S, unsigned char *out,
-                                                       long long ldo, int vec_ok) {
-    pdl_entry();
-    constexpr int ES = FP8 ? 1 : 2;
-    constexpr int T64 = 64;
-    constexpr int PITCH = T64 + 1;               // floats
-    constexpr int NLD = T64 * (T64 / 4) / 256;   // float4 loads per thread and tile
-    constexpr int NST = T64 * (T64 / 8) / 256;   // 8-value stores per thread and tile
-    __shared__ float s[T64 * PITCH];             // s[k][x]
-    const long long xt = (S.X + T64 - 1) / T64, kt = (S.K + T64 - 1) / T64;
-    for (long long t = blockIdx.x; t < xt * kt; t += gridDim.x) {
-        const long long x0 = (t % xt) * T64, k0 = (t / xt) * T64;
-        const float c = S.c[(x0 / S.L) * S.cx + (k0 / S.L) * S.cl];
-        float v[NLD][4];
-#pragma unroll
-        for (int u = 0; u < NLD; ++u) {
-            const int e = threadIdx.x + u * 256;
-            const int kr = e / (T64 / 4), xc = (e % (T64 / 4)) * 4;
-            const long long k = k0 + kr, x = x0 + xc;
-            if (k < S.K && vec_ok && x + 4 <= S.X) {
-                const float4 a = __ldg(reinterpret_cast<const float4 *>(S.p + k * S.sk + x));
-                v[u][0] = a.x; v[u][1] = a.y; v[u][2] = a.z; v[u][3] = a.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    v[u][i] = (k < S.K && x + i < S.X) ? S.p[k * S.sk + x + i] : 0.f;
-            }
-        }
-        __syncthreads();   // the previous tile's readers are done with s
-#pragma unroll
-        for (int u = 0; u < NLD; ++u) {
-            const int e = threadIdx.x + u * 256;
-            const int kr = e / (T64 / 4), xc = (e % (T64 / 4)) * 4;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) s[kr * PITCH + xc + i] = __fmul_rn(v[u][i], c);
-        }
-        __syncthreads();
-        // store: rows x, 8 k per item
-#pragma unroll
-        for (int u = 0; u < NST; ++u) {
-            const int e = threadIdx.x + u * 256;
-            const int xr = e / (T64 / 8), kc = (e % (T64 / 8)) * 8;
-            const long long x = x0 + xr, k = k0 + kc;
-            if (x >= S.X || k >= ldo) continue;
-            float w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) w[i] = (k + i < S.K) ? s[(kc + i) * PITCH + xr] : 0.f;
-            encode8<FP8>(w, out + (x * ldo + k) * ES);
-        }
-    }
-}
-
-// ------------------------------------------------------------------ fused statistics + codes
-// The tensor-core forms with companders that depend only on the block's own
-// maximum (fixed bits: c = gamma / max|x|; E4M3: c = 448 / max|x|): one CTA
-// per L x L block of op(X) (L <= 128) reads the block once, keeps it in
-// registers, reduces max|x| (exact) and sum x^2 (double-float, as the
-// statistics kernel does), sets c (fp64, rounded to fp32) and s = 1/c, and
-// writes the block's codes out[x][k] -- the statistics pass, the compander
-// kernel and the code pass of the general path in one read of the input.
-struct FusedOp {
-    Src<float> S;
-    long long nbx, nbk;             // blocks along x and k
-    double *mx, *var;               // per block, index bi * S.cx + bk * S.cl
-    float *c;
-    double *s;
-    unsigned char *out;
-};
-
-__device__ inline void df_add2(float &hi, float &lo, float bh, float bl) {
-    const float s = __fadd_rn(hi, bh);
-    const float v = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(bh, v));
-    const float t = __fadd_rn(e, __fadd_rn(lo, bl));
-    hi = __fadd_rn(s, t);
-    lo = __fsub_rn(t, __fsub_rn(hi, s));
-}
-
-// exact square as hi + err (TwoProduct), TwoSum into (hi, lo)
-__device__ inline void df_add_sq(float &hi, float &lo, float x) {
-    const float p = __fmul_rn(x, x);
-    const float e = __fmaf_rn(x, x, -p);
-    const float t = __fadd_rn(hi, p);
-    const float bp = __fsub_rn(t, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-    hi = t;
-    lo = __fadd_rn(lo, __fadd_rn(err, e));
-}
-
-constexpr int kFusedThreads = 512;   // 32 values per thread at L = 128 (two CTAs, 32 warps per SM)
-
-// block statistics of the values this thread holds, reduced over the CTA;
-// thread 0 writes them with the compander, every thread returns c
-template <int NVAL>
-__device__ inline float fused_block_companders(const float (&v)[NVAL], const FusedOp &o,
-                                               long long bx, long long bk, int xn, int kn,
-                                               double gamma, DevPlan *plan) {
-    __shared__ float red_h[32], red_l[32];
-    __shared__ unsigned int red_m[32];
-    __shared__ int red_b[32];
-    __shared__ float c_sh;
-    float hi = 0.f, lo = 0.f;
-    unsigned int mb = 0;
-    int bad = 0;
-#pragma unroll
-    for (int u = 0; u < NVAL; ++u) {
-        const unsigned int b = __float_as_uint(v[u]) & 0x7fffffffu;
-        mb = max(mb, b);
-        bad |= (b >= 0x7f800000u);
-        df_add_sq(hi, lo, v[u]);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto warp_reduce = [&]() {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, hi, off);
-            const float ol = __shfl_xor_sync(0xffffffffu, lo, off);
-            df_add2(hi, lo, oh, ol);
-            mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, off));
-            bad |= __shfl_xor_sync(0xffffffffu, bad, off);
-        }
-    };
-    warp_reduce();
-    if (lane == 0) { red_h[warp] = hi; red_l[warp] = lo; red_m[warp] = mb; red_b[warp] = bad; }
-    __syncthreads();
-    if (warp == 0) {
-        const bool in = lane < kFusedThreads / 32;
-        hi = in ? red_h[lane] : 0.f;
-        lo = in ? red_l[lane] : 0.f;
-        mb = in ? red_m[lane] : 0u;
-        bad = in ? red_b[lane] : 0;
-        warp_reduce();
-        if (lane == 0) {
-            const double m = (double)__uint_as_float(mb);
-            const long long idx = bx * o.S.cx + bk * o.S.cl;
-            // eq. 3's compander: c = gamma / max|x| in fp64, rounded to fp32
-            const double c = m > 0.0 ? __ddiv_rn(gamma, m) : 0.0;
-            o.mx[idx] = m;
-            o.var[idx] = ((double)hi + (double)lo) / ((double)xn * (double)kn);
-            o.c[idx] = (float)c;
-            o.s[idx] = c > 0.0 ? __ddiv_rn(1.0, c) : 0.0;
-            c_sh = (float)c;
-            if (bad) atomicExch(&plan->nonfinite, 1);
-        }
-    }
-    __syncthreads();
-    return c_sh;
-}
-
-template <int FP8, int L>
-__global__ void __launch_bounds__(kFusedThreads, 2)
-    codes_stats_kernel(FusedOp A, FusedOp B, long long nblkA, double gamma, long long ldo,
-                       DevPlan *plan) {
-    pdl_entry();
-    constexpr int ES = FP8 ? 1 : 2;
-    constexpr int NV = L * L / kFusedThreads;    // values per thread: 32 at L = 128
-    extern __shared__ float s_tile[];            // x-contiguous inputs: s[k][x], pitch L + 1
-    const bool isA = (long long)blockIdx.x < nblkA;
-    const FusedOp &o = isA ? A : B;
-    const long long blk = isA ? (long long)blockIdx.x : (long long)blockIdx.x - nblkA;
-    const long long bx = blk / o.nbk, bk = blk - bx * o.nbk;
-    const Src<float> &S = o.S;
-    const long long x0 = bx * L, k0 = bk * L;
-    const int xn = (int)min((long long)L, S.X - x0), kn = (int)min((long long)L, S.K - k0);
-    float v[NV];
-    if (S.sk == 1) {
-        // k contiguous: item = 8 consecutive k of one row x, loaded, counted
-        // and encoded by the same thread
-#pragma unroll
-        for (int u = 0; u < NV / 8; ++u) {
-            const int e = threadIdx.x + u * kFusedThreads;
-            const int xr = e / (L / 8), kr = (e % (L / 8)) * 8;
-            const float *src = S.p + (x0 + xr) * S.sx + k0 + kr;
-            const bool full = xr < xn && kr + 8 <= kn && ((reinterpret_cast<uintptr_t>(src) & 15) == 0);
-            if (full) {
-                const float4 a = __ldg(reinterpret_cast<const float4 *>(src));
-                const float4 b = __ldg(reinterpret_cast<const float4 *>(src + 4));
-                v[8 * u] = a.x; v[8 * u + 1] = a.y; v[8 * u + 2] = a.z; v[8 * u + 3] = a.w;
-                v[8 * u + 4] = b.x; v[8 * u + 5] = b.y; v[8 * u + 6] = b.z; v[8 * u + 7] = b.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    v[8 * u + i] = (xr < xn && kr + i < kn) ? src[i] : 0.f;
-            }
-        }
-        const float c = fused_block_companders(v, o, bx, bk, xn, kn, gamma, plan);
-#pragma unroll
-        for (int u = 0; u < NV / 8; ++u) {
-            const int e = threadIdx.x + u * kFusedThreads;
-            const int xr = e / (L / 8), kr = (e % (L / 8)) * 8;
-            const long long k = k0 + kr;
-            if (xr >= xn || k >= ldo) continue;
-            float w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) w[i] = __fmul_rn(v[8 * u + i], c);
-            encode8<FP8>(w, o.out + ((x0 + xr) * ldo + k) * ES);
-        }
-    } else {
-        // x contiguous: 4 consecutive x of one row k per load, transposed
-        // through shared memory for the k-contiguous codes
-        constexpr int P = L + 1;
-#pragma unroll
-        for (int u = 0; u < NV / 4; ++u) {
-            const int e = threadIdx.x + u * kFusedThreads;
-            const int kr = e / (L / 4), xr = (e % (L / 4)) * 4;
-            const float *src = S.p + (k0 + kr) * S.sk + x0 + xr;
-            const bool full = kr < kn && xr + 4 <= xn && ((reinterpret_cast<uintptr_t>(src) & 15) == 0);
-            if (full) {
-                const float4 a = __ldg(reinterpret_cast<const float4 *>(src));
-                v[4 * u] = a.x; v[4 * u + 1] = a.y; v[4 * u + 2] = a.z; v[4 * u + 3] = a.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    v[4 * u + i] = (kr < kn && xr + i < xn) ? src[i] : 0.f;
-            }
-        }
-        const float c = fused_block_companders(v, o, bx, bk, xn, kn, gamma, plan);
-#pragma unroll
-        for (int u = 0; u < NV / 4; ++u) {
-            const int e = threadIdx.x + u * kFusedThreads;
-            const int kr = e / (L / 4), xr = (e % (L / 4)) * 4;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) s_tile[kr * P + xr + i] = v[4 * u + i];
-        }
-        __syncthreads();
-        // items: 8 consecutive k of one row x, lanes along x (conflict-free
-        // reads), encoded into the code tile cs[x][k] (row pitch CP bytes:
-        // the lanes' 8- or 16-byte writes fall in distinct banks) ...
-        constexpr int CP = FP8 ? L + 8 : 2 * L + 16;
-        unsigned char *cs = reinterpret_cast<unsigned char *>(s_tile + L * P);
-        for (int e = threadIdx.x; e < L * L / 8; e += kFusedThreads) {
-            const int xr = e % L, kr = (e / L) * 8;
-            float w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) w[i] = __fmul_rn(s_tile[(kr + i) * P + xr], c);
-            encode8<FP8>(w, cs + xr * CP + kr * ES);
-        }
-        __syncthreads();
-        // ... and copied out row by row: consecutive lanes write consecutive
-        // 8 bytes (E4M3) or 16 bytes (fp16) of one row of codes
-        constexpr int UB = FP8 ? 8 : 16;             // bytes per unit
-        constexpr int UPR = L * ES / UB;             // units per row of the tile
-        for (int e = threadIdx.x; e < L * UPR; e += kFusedThreads) {
-            const int xr = e / UPR, u = e % UPR;
-            const long long k = k0 + (long long)u * (UB / ES);
-            if (xr >= xn || k >= ldo) continue;
-            unsigned char *dst = o.out + ((x0 + xr) * ldo + k) * ES;
-            if constexpr (FP8)
-                *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(cs + xr * CP + u * UB);
-            else
-                *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(cs + xr * CP + u * UB);
-        }
-    }
-}
-
-// dynamic shared memory of codes_stats_kernel for x-contiguous inputs: the
-// fp32 tile s[k][x] (pitch L + 1) and the code tile (pitch L + 8 or 2 L + 16 bytes)
-constexpr size_t fused_xc_smem(int fp8, int L) {
-    return (size_t)L * (L + 1) * sizeof(float) + (size_t)L * (fp8 ? L + 8 : 2 * L + 16);
-}
-
 template <typename T>
 Src<T> make_src(const PackOperand<T> &o) {
     Src<T> S;
@@ -877,68 +549,6 @@ cudaError_t launch_pack_x(const PackOperand<T> &o, int W, const DevPlan *plan, i
         case 4: return launch_pack_x_w<T, 4>(o, plan, expectW, wsign, out, ldo, st);
     }
     return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_codes(const PackOperand<float> &o, int fp8, void *out, long long ldo,
-                         cudaStream_t st) {
-    Src<float> S = make_src(o);
-    unsigned char *ob = reinterpret_cast<unsigned char *>(out);
-    const bool aligned = ((uintptr_t)o.src % 16 == 0) && ((uintptr_t)out % 16 == 0) && ldo % 8 == 0;
-    if (o.sk == 1) {
-        const int vec_ok = aligned && (o.sx % 4 == 0);
-        const long long items = o.X * ((o.K + 7) / 8);
-        const int g = capped((items + 255) / 256);
-        return fp8 ? launch_pdl(codes_kc_kernel<1>, dim3(g), dim3(256), 0, st, S, ob, ldo, vec_ok)
-                   : launch_pdl(codes_kc_kernel<0>, dim3(g), dim3(256), 0, st, S, ob, ldo, vec_ok);
-    } else {
-        const int vec_ok = aligned && o.sx == 1 && (o.sk % 4 == 0);
-        const long long tiles = ((o.X + 63) / 64) * ((o.K + 63) / 64);
-        const int g = capped(tiles);
-        return fp8 ? launch_pdl(codes_xc_kernel<1>, dim3(g), dim3(256), 0, st, S, ob, ldo, vec_ok)
-                   : launch_pdl(codes_xc_kernel<0>, dim3(g), dim3(256), 0, st, S, ob, ldo, vec_ok);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_codes_stats(const PackOperand<float> &a, double *mxA, double *varA,
-                               float *cA, double *sA, void *outA, const PackOperand<float> *b,
-                               double *mxB, double *varB, float *cB, double *sB, void *outB,
-                               int fp8, double gamma, long long ldo, DevPlan *plan,
-                               cudaStream_t st) {
-    const int L = a.L;
-    if (L > 128 || L % 64) return cudaErrorInvalidValue;
-    auto op = [&](const PackOperand<float> &o, double *mx, double *var, float *c, double *s,
-                  void *out) {
-        FusedOp f;
-        f.S = make_src(o);
-        f.nbx = (o.X + L - 1) / L;
-        f.nbk = (o.K + L - 1) / L;
-        f.mx = mx; f.var = var; f.c = c; f.s = s;
-        f.out = reinterpret_cast<unsigned char *>(out);
-        return f;
-    };
-    FusedOp fa = op(a, mxA, varA, cA, sA, outA);
-    FusedOp fb = b ? op(*b, mxB, varB, cB, sB, outB) : fa;
-    const long long na = fa.nbx * fa.nbk, nb = b ? fb.nbx * fb.nbk : 0;
-    if (na + nb > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    const bool xc = a.sk != 1 || (b && b->sk != 1);
-    const size_t smem = xc ? fused_xc_smem(fp8, L) : 0;
-    auto kern = L == 128 ? (fp8 ? codes_stats_kernel<1, 128> : codes_stats_kernel<0, 128>)
-                         : (fp8 ? codes_stats_kernel<1, 64> : codes_stats_kernel<0, 64>);
-    static std::once_flag attr_once;
-    cudaError_t attr_err = cudaSuccess;
-    std::call_once(attr_once, [&]() {
-        // the L = 128 tiles need 82-99 KB of dynamic shared memory
-        for (int f8 = 0; f8 < 2; ++f8) {
-            cudaError_t e = cudaFuncSetAttribute(f8 ? codes_stats_kernel<1, 128> : codes_stats_kernel<0, 128>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)fused_xc_smem(f8, 128));
-            if (e != cudaSuccess) attr_err = e;
-        }
-    });
-    if (attr_err != cudaSuccess) return attr_err;
-    return launch_pdl(kern, dim3((unsigned)(na + nb)), dim3(kFusedThreads), smem, st, fa, fb, na,
-                      gamma, ldo, plan);
 }
 
 template cudaError_t launch_pack_k_pair<float>(const PackOperand<float> &, const PackOperand<float> &,

@@ -1,0 +1,289 @@
+// The planner's device code that both the statistics kernels (whose last warp
+// takes the sums over slabs and, outside target mode, decides the plan) and the
+// candidate kernel of target mode run.
+#pragma once
+
+#include <math.h>
+
+#include "tdg_common.cuh"
+
+namespace tdg {
+
+// The plain product (form PLAIN, or the W = 1 fallback of target mode for the
+// packed forms) uses no companders.
+__device__ inline bool needs_companders(const PlanParams &pp, const DevPlan &a) {
+    if (pp.form == TDG_PLAIN) return false;
+    if ((pp.form == TDG_SYM || pp.form == TDG_ASYM) && pp.mode == MODE_TARGET && a.W == 1)
+        return false;
+    return true;
+}
+
+__device__ inline int t_max_for(int p) { return p == 24 ? 4 * 24 : 4 * 40; }
+
+
+// eq. 21 summed over (i, l, j); operation order as written above.  With rms
+// the representation term is scaled by the blocks' crest factors (s measured
+// on uniform integers, RMS = max / sqrt(3)): 9 s^2 sum(sigma_A^2 sigma_B^2).
+__device__ inline double model_noise(const DevPlan &a, int L, double gA, double gB, double s,
+                                     int rms) {
+    double t1 = __ddiv_rn(__dmul_rn((double)L, a.T1), __dmul_rn(__dmul_rn(12.0, gB), gB));
+    double t2 = __ddiv_rn(__dmul_rn((double)L, a.T2), __dmul_rn(__dmul_rn(12.0, gA), gA));
+    const double g2 = __dmul_rn(__dmul_rn(__dmul_rn(gA, gA), gB), gB);
+    if (!rms) {
+        double t3 = __ddiv_rn(__dmul_rn(a.T3, __dadd_rn(__ddiv_rn((double)L, 144.0), __dmul_rn(s, s))), g2);
+        return __dadd_rn(__dadd_rn(t1, t2), t3);
+    }
+    double t3 = __ddiv_rn(__dmul_rn(a.T3, __ddiv_rn((double)L, 144.0)), g2);
+    double t4 = __ddiv_rn(__dmul_rn(__dmul_rn(9.0, __ddiv_rn(a.S, (double)L)), __dmul_rn(s, s)), g2);
+    return __dadd_rn(__dadd_rn(__dadd_rn(t1, t2), t3), t4);
+}
+
+__device__ inline double snr_db(double S, double N) {
+    return N <= 0.0 ? INFINITY : 10.0 * log10(S / N);
+}
+
+// S / L, T1, T2, T3: products of the per-slab aggregates summed over slabs by
+// one warp (lanes over l, then a fixed xor tree); every caller gets the same
+// bits.
+__device__ inline void slab_totals(const PlanParams &pp, const double *__restrict__ agg,
+                                   double &S, double &T1, double &T2, double &T3) {
+    const int lane = threadIdx.x & 31;
+    S = T1 = T2 = T3 = 0.0;
+    if (pp.mode != MODE_MANUAL) {
+        for (int l = lane; l < pp.nK; l += 32) {
+            const double X = __ldcg(&agg[4 * (long long)l]), MA = __ldcg(&agg[4 * (long long)l + 1]);
+            const double Y = __ldcg(&agg[4 * (long long)l + 2]), MB = __ldcg(&agg[4 * (long long)l + 3]);
+            S += X * Y;
+            T1 += X * MB;
+            T2 += Y * MA;
+            T3 += MA * MB;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        S += __shfl_xor_sync(0xffffffffu, S, off);
+        T1 += __shfl_xor_sync(0xffffffffu, T1, off);
+        T2 += __shfl_xor_sync(0xffffffffu, T2, off);
+        T3 += __shfl_xor_sync(0xffffffffu, T3, off);
+    }
+}
+
+__device__ inline double rho_of(double T1, double T2) {
+    return (T1 <= 0.0 || T2 <= 0.0) ? 1.0 : sqrt(T2 / T1);
+}
+
+// Target mode, packed forms: every candidate (W, R_max level t) evaluated in
+// full by one lane (companders, z, representation noise, model noise and
+// SNR), 32 candidates per CTA spread over SMs: fp64 divisions, square roots
+// and logarithms are slow on GB300 and would serialise on one SM.  n < 0
+// marks a level without usable companders or representation-noise value.
+struct LevelRec {
+    double n, pred, s;
+    long long R;
+    int gA, gB, q, Wef;
+};
+static_assert(sizeof(LevelRec) == kLevelRecDoubles * sizeof(double), "planner workspace record");
+
+// a candidate record written by another CTA of the same grid: read from L2
+__device__ inline LevelRec load_rec(const LevelRec *p) {
+    LevelRec r;
+    r.n = __ldcg(&p->n);
+    r.pred = __ldcg(&p->pred);
+    r.s = __ldcg(&p->s);
+    r.R = __ldcg(&p->R);
+    r.gA = __ldcg(&p->gA);
+    r.gB = __ldcg(&p->gB);
+    r.q = __ldcg(&p->q);
+    r.Wef = __ldcg(&p->Wef);
+    return r;
+}
+
+// The plan, decided by one full warp: fixed bits, manual parameters, the
+// tensor-core forms, or (target mode, packed forms) the choice among the
+// candidate records res: for W from the request down to 2 the level of least
+// model noise (eq. 27's argmax of the SNR; ties to the lower level), the first
+// W whose SNR meets the target; else the plain product (fallback) or
+// TDG_EUNREACHABLE.  Lane 0 writes the plan.
+static __device__ __noinline__ void decide_plan(const PlanParams &pp,
+                                                const double *__restrict__ stab,
+                                                const LevelRec *res, DevPlan *plan, double S,
+                                                double T1, double T2, double T3, double rho) {
+    const int lane = threadIdx.x & 31;
+    const int L = pp.L;
+    DevPlan a{};
+    a.S = (double)L * S;
+    a.T1 = T1;
+    a.T2 = T2;
+    a.T3 = T3;
+    a.status = 0;
+    a.level = -1;
+    a.pred_snr = NAN;
+    a.s_rep = 0.0;
+
+    if (pp.form == TDG_PLAIN) {
+        a.W = 1; a.q = 0; a.gA = a.gB = 0; a.R = 0; a.Wef = 0;
+    } else if (pp.form == TDG_TC_FP8) {
+        a.W = 1; a.q = 0; a.gA = a.gB = (int)kFp8Max; a.R = 0; a.Wef = 0;
+    } else if (pp.form == TDG_TC_INT) {
+        int gA, gB;
+        if (pp.mode == MODE_FIXED) {
+            gA = gB = (1 << (pp.bits - 1)) - 1;
+        } else {
+            split_gammas((long long)kTcIntExact, L, rho, gA, gB);
+            gA = min(gA, kTcIntMaxGamma);
+            gB = min(min(gB, kTcIntMaxGamma), (int)((long long)kTcIntExact / ((long long)L * gA)));
+        }
+        a.W = 1; a.gA = gA; a.gB = gB; a.R = (long long)L * gA * gB;
+        a.q = q_for(a.R); a.Wef = w_ef(a.R, a.q, pp.p);
+        a.pred_snr = snr_db(a.S, model_noise(a, L, gA, gB, 0.0, pp.noise_rms));
+        if (pp.mode == MODE_TARGET && a.pred_snr < pp.target_db) a.status = TDG_EUNREACHABLE;
+    } else if (pp.mode == MODE_MANUAL) {
+        a.W = pp.Wreq; a.q = pp.manual_q; a.gA = a.gB = 0; a.R = 0; a.Wef = 0;
+    } else if (pp.mode == MODE_FIXED) {
+        int g = (1 << (pp.bits - 1)) - 1;
+        a.W = pp.Wreq; a.gA = a.gB = g; a.R = (long long)L * g * g;
+        a.q = q_for(a.R); a.Wef = w_ef(a.R, a.q, pp.p);
+        double s = -1.0;
+        if (a.W <= a.Wef) {
+            s = 0.0;
+        } else if (stab) {
+            int tbest = -1;
+            for (int t = 0; t <= t_max_for(pp.p); ++t)
+                if (r_level(t) <= a.R) tbest = t;
+            if (tbest >= pp.t0 && tbest < pp.t0 + pp.nt)
+                s = stab[(pp.Wreq - 2) * pp.nt + (tbest - pp.t0)];
+        }
+        if (s >= 0.0) {
+            a.pred_snr = snr_db(a.S, model_noise(a, L, g, g, s, pp.noise_rms));
+            a.s_rep = s;
+        }
+    } else {  // MODE_TARGET, packed forms
+        int t_lo = 0;
+        while (r_level(t_lo) < L) ++t_lo;
+        const int t_hi = t_max_for(pp.p);
+        bool chosen = false;
+        DevPlan first{};
+        bool have_first = false;
+        for (int W = pp.Wreq; W >= 2 && !chosen; --W) {
+            // argmin of N over the levels (ties to the lower level); N >= 0,
+            // so its bit pattern orders like its value (integer compares)
+            // every load of the lane's levels issued before any is used
+            constexpr int kPerLane = (kMaxLevels + 31) / 32;
+            double nv[kPerLane];
+#pragma unroll
+            for (int u = 0; u < kPerLane; ++u) {
+                const int t = t_lo + lane + 32 * u;
+                nv[u] = t <= t_hi ? __ldcg(&res[(W - 2) * kMaxLevels + t].n) : -1.0;
+            }
+            unsigned long long bn = ~0ull;
+            int bt = -1;
+#pragma unroll
+            for (int u = 0; u < kPerLane; ++u) {     // lanes scan ascending t
+                if (nv[u] < 0.0) continue;
+                const unsigned long long nb = (unsigned long long)__double_as_longlong(nv[u]);
+                if (nb < bn) { bn = nb; bt = t_lo + lane + 32 * u; }
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const unsigned long long n2 = __shfl_xor_sync(0xffffffffu, bn, off);
+                const int t2 = __shfl_xor_sync(0xffffffffu, bt, off);
+                if (t2 >= 0 && (bt < 0 || n2 < bn || (n2 == bn && t2 < bt))) {
+                    bn = n2;
+                    bt = t2;
+                }
+            }
+            const int t = bt;                          // the same in every lane
+            if (t < 0) continue;
+            const LevelRec r = load_rec(&res[(W - 2) * kMaxLevels + t]);
+            DevPlan c = a;
+            c.W = W;
+            c.q = r.q;
+            c.gA = r.gA;
+            c.gB = r.gB;
+            c.R = r.R;
+            c.Wef = r.Wef;
+            c.level = t;
+            c.pred_snr = r.pred;
+            c.s_rep = r.s;
+            if (!have_first) { first = c; have_first = true; }
+            if (c.pred_snr >= pp.target_db) { a = c; chosen = true; }
+        }
+        if (!chosen) {
+            if (pp.allow_fallback) {
+                a.W = 1; a.q = 0; a.gA = a.gB = 0; a.R = 0; a.Wef = 0; a.level = -1;
+                a.pred_snr = INFINITY;
+            } else if (have_first) {
+                a = first;
+                a.status = TDG_EUNREACHABLE;
+            } else {
+                a.W = pp.Wreq; a.q = q_for(L); a.gA = a.gB = 1; a.R = L; a.Wef = 0;
+                a.status = TDG_EUNREACHABLE;
+            }
+        }
+    }
+    if (lane == 0) {
+        // the record's counters and the statistics' flag return to zero here,
+        // for the next call's kernels
+        const int nf = __ldcg(&plan->nonfinite_seen);
+        a.nonfinite = nf;
+        if (nf && a.status == 0) a.status = TDG_ENONFINITE;
+        *plan = a;
+    }
+}
+
+// Called by one full warp of a statistics CTA once its block of slab l is
+// written by lane 0: the last of the slab's blocks takes the slab's aggregates
+// (lanes over the blocks, as slab_aggregate_warp orders them), the last slab
+// the sums over slabs and rho -- and decides the plan, except for the packed
+// forms' target mode, whose candidates need a kernel of their own.  Counters
+// only, no waiting; each returns to zero with its last arrival.  (A kernel of
+// its own for the aggregates, and one for the decision, took 7-9 and 2.5-8 us
+// of a call.)
+struct SlabFinish {
+    PlanParams pp;
+    const double *mA, *vA, *mB, *vB;   // block maxima and variances of op(A), op(B)
+    const double *stab;
+    double *agg;
+    unsigned int *slab_done;           // [nK], zero between calls
+    unsigned int blocks;               // arrivals per slab
+};
+
+static __device__ __noinline__ void slab_finish(const SlabFinish &f, int l, DevPlan *plan) {
+    const int lane = threadIdx.x & 31;
+    unsigned int prev = 0;
+    if (lane == 0) {
+        __threadfence();
+        prev = atomicAdd(&f.slab_done[l], 1u);
+    }
+    prev = __shfl_sync(0xffffffffu, prev, 0);
+    if (prev + 1 != f.blocks) return;
+    __threadfence();
+    const bool modelled = f.pp.form != TDG_TC_FP8;      // E4M3 has no noise model
+    if (modelled) slab_aggregate_warp(l, f.pp.nM, f.pp.nK, f.pp.nN, f.mA, f.vA, f.mB, f.vB, f.agg);
+    if (lane == 0) {
+        f.slab_done[l] = 0;
+        __threadfence();
+        prev = atomicAdd(&plan->slabs_done, 1u);
+    }
+    prev = __shfl_sync(0xffffffffu, prev, 0);
+    if (prev + 1 != (unsigned int)f.pp.nK) return;
+    __threadfence();
+    double S = 0.0, T1 = 0.0, T2 = 0.0, T3 = 0.0;
+    if (modelled) slab_totals(f.pp, f.agg, S, T1, T2, T3);
+    const double rho = rho_of(T1, T2);
+    if (f.pp.mode == MODE_TARGET && (f.pp.form == TDG_SYM || f.pp.form == TDG_ASYM)) {
+        if (lane == 0) {
+            plan->tS = S;
+            plan->tT1 = T1;
+            plan->tT2 = T2;
+            plan->tT3 = T3;
+            plan->trho = rho;
+            plan->slabs_done = 0;
+        }
+    } else {
+        decide_plan(f.pp, f.stab, nullptr, plan, S, T1, T2, T3, rho);
+    }
+}
+
+}  // namespace tdg
+

@@ -37,6 +37,7 @@
 
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
+#include "tdg_planner.cuh"
 #include "tdgemm.h"
 
 namespace tdg {
@@ -104,6 +105,8 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
     const size_t o_plan = take(sizeof(DevPlan));
+    const size_t o_done = take((size_t)nK * sizeof(unsigned int));
+    const size_t cleared = off;
     const size_t o_agg =
         take(((size_t)4 * nK + (size_t)kLevelRecDoubles * (kMaxW - 1) * kMaxLevels) * 8);
     const size_t o_mA = take(nA_blk * 8), o_eA = take(nA_blk * 8);
@@ -129,18 +132,20 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     T *cA = (T *)(ws + o_cA), *cB = (T *)(ws + o_cB), *pair = (T *)(ws + o_pair);
     T *Abuf = (T *)(ws + o_A), *Bbuf = (T *)(ws + o_B);
 
-    // the plan record carries the device status, the non-finite flag and the
-    // planner's counter: start at zero
-    ST_TRY(cudaMemsetAsync(dplan, 0, sizeof(DevPlan), st));
-    ST_TRY(launch_block_stats<T>(A, nA ? M : K, nA ? K : M, lda, nA ? 0 : 1, nK, mA, eA, B,
-                                 nB ? K : N, nB ? N : K, ldb, nB ? 0 : 1, nN, mB, eB, L, dplan,
-                                 st));
+    // the plan record and the slab counters start at zero (the array holds
+    // whatever the call before left, of another shape)
+    ST_TRY(cudaMemsetAsync(ws, 0, cleared, st));
     PlanParams pp{};
     pp.mode = MODE_FIXED; pp.form = form; pp.dtype = sizeof(T) == 8 ? TDG_F64 : TDG_F32;
     pp.L = L; pp.Wreq = W; pp.p = sizeof(T) == 8 ? 53 : 24; pp.bits = bits;
     pp.allow_fallback = 0; pp.noise_rms = 0; pp.target_db = NAN;
     pp.nM = nM; pp.nK = nK; pp.nN = nN; pp.M = M; pp.N = N; pp.K = K;
     pp.t0 = 0; pp.nt = 0;
+    const SlabFinish fin{pp, mA, eA, mB, eB, nullptr, agg, (unsigned int *)(ws + o_done),
+                         (unsigned int)(nM + nN)};
+    ST_TRY(launch_block_stats<T>(A, nA ? M : K, nA ? K : M, lda, nA ? 0 : 1, nK, mA, eA, B,
+                                 nB ? K : N, nB ? N : K, ldb, nB ? 0 : 1, nN, mB, eB, L, dplan,
+                                 fin, st));
     ST_TRY(launch_planner<T>(pp, mA, eA, mB, eB, nullptr, dplan, agg, cA, sA, cB, sB, pair, st));
     PackOperand<T> oa{}, ob{};
     oa.src = A; oa.X = M; oa.K = K; oa.L = L; oa.c = cA; oa.cx = nK; oa.cl = 1;

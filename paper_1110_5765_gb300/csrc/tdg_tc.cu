@@ -421,44 +421,43 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const int ew = warp - 2;
         const int quad = warp & 3;                     // TMEM lanes 32*quad .. +31
         const int cgrp = ew >> 2;                      // columns [EPI_COLS*cgrp, +EPI_COLS)
-        const long long lstride = (long long)g.nM * g.nN;
         const uint32_t acc_empty_cl[2] = {cluster_addr(&acc_empty[0], 0),
                                           cluster_addr(&acc_empty[1], 0)};
         bool ok = true;
-        // the thread's EPI_COLS columns lie in one column block (L % 64 == 0,
-        // column groups 64-aligned), so one factor per slab, fetched a slab
-        // ahead -- across tiles too: the next tile's first factor is fetched
-        // during this tile's last slab, so the tile change costs the MMA
-        // issuer as little as possible
-        auto factor_row = [&](int k) -> const float * {
+        // the warp's 32 rows and EPI_COLS columns lie in one row and one column
+        // block (L % 64 == 0), so it needs one factor (float)(s_A s_B) per slab:
+        // lane u forms slab u's of the next 32 (one fp64 product), and a slab
+        // takes its own by a shuffle.  The next 32 are fetched a batch ahead,
+        // across tiles too.
+        auto fetch_factors = [&](int k, int l0, double &fa, double &fb) {
+            if (k >= my_tiles) return;
             long long m0, n0;
             tile_origin(k, m0, n0);
-            const long long row = m0 + quad * 32 + lane;
-            const long long col0 = n0 + cgrp * EPI_COLS;
-            const int iblk = (int)min((long long)((unsigned long long)row / (unsigned)g.L),
-                                      (long long)g.nM - 1);
-            const int jblk = (int)min((long long)((unsigned long long)col0 / (unsigned)g.L),
-                                      (long long)g.nN - 1);
-            return g.pair + (long long)iblk * g.nN + jblk;
+            const int iblk = (int)min((m0 + quad * 32) / g.L, (long long)g.nM - 1);
+            const int jblk = (int)min((n0 + cgrp * EPI_COLS) / g.L, (long long)g.nN - 1);
+            const int l = min(l0 + lane, nslab - 1);
+            fa = __ldg(g.sA + (long long)iblk * g.nK + l);
+            fb = __ldg(g.sB + (long long)l * g.nN + jblk);
         };
-        const float *prow = my_tiles > 0 ? factor_row(0) : g.pair;
-        float pr_next = my_tiles > 0 ? __ldg(prow) : 0.f;
+        double fa = 0.0, fb = 0.0;
+        fetch_factors(0, 0, fa, fb);
+        float fac_next = (float)__dmul_rn(fa, fb);
         for (int kt = 0; kt < my_tiles && ok; ++kt) {
-            const float *prow_n = prow;
+            float fac = 0.f;
             float cacc[EPI_COLS];
 #pragma unroll
             for (int c = 0; c < EPI_COLS; ++c) cacc[c] = 0.f;
             for (int l = 0; l < nslab; ++l) {
                 const int gs = kt * nslab + l;
                 const int b = gs & 1;
-                const float pr = pr_next;
-                if (l + 1 < nslab) {
-                    pr_next = __ldg(prow + (long long)(l + 1) * lstride);
-                } else if (kt + 1 < my_tiles) {
-                    prow_n = factor_row(kt + 1);
-                    pr_next = __ldg(prow_n);
+                if ((l & 31) == 0) {
+                    fac = fac_next;
+                    const bool more = l + 32 < nslab;
+                    fetch_factors(more ? kt : kt + 1, more ? l + 32 : 0, fa, fb);
                 }
+                const float pr = __shfl_sync(0xffffffffu, fac, l & 31);
                 if (!tc_wait_epilogue<FP8>(&acc_full[b], (gs >> 1) & 1)) { ok = false; break; }
+                if ((l & 31) == 0) fac_next = (float)__dmul_rn(fa, fb);   // (fetched before the wait)
                 tc_fence_after();
                 const uint32_t base =
                     tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * BN + cgrp * EPI_COLS);
@@ -498,7 +497,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             tile_origin(kt, m0, n0);
             const long long rbase = m0 + quad * 32;
             const long long col0 = n0 + cgrp * EPI_COLS;
-            prow = prow_n;
             if (g.c_tma) {
                 // beta = 0: alpha C_acc staged in the C map's 64-byte swizzle
                 // (16-byte unit u of row r at u ^ ((r >> 1) & 3)), written by
