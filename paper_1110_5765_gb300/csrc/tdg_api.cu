@@ -286,15 +286,16 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
         // the ordered sum over slabs in the unpack kernel; needs the r-bar
         // buffer that TDG_KEEP_PACKED also uses
         if (is_packed_form(form) && !(flags & (TDG_KEEP_PACKED | TDG_PAIR_EXACT)) && p->nK >= 4) {
-            int bxa, bxb, bk, dev = 0, sms = 0;
             const long long mrows = form == TDG_ASYM ? (long long)p->nM * Pof(L, W) : M;
-            packed_gemm_boxes(dtype, form == TDG_SYM ? G_SYM : G_ASYM, W, &bxa, &bxb, &bk);
-            if (dtype == TDG_F64) bxa = bxb = f64_tile_edge(mrows, N);
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            const long long ntiles = ((mrows + bxa - 1) / bxa) * ((N + bxb - 1) / bxb);
-            if (sms > 0 && ntiles * 2 <= sms)
-                p->split_groups = (int)std::min<long long>(p->nK, (2LL * sms + ntiles - 1) / ntiles);
+            if (dtype == TDG_F64) {
+                const long long sms = device_sms(), edge = f64_tile_edge(mrows, N);
+                const long long ntiles = ((mrows + edge - 1) / edge) * ((N + edge - 1) / edge);
+                if (ntiles * 2 <= sms)
+                    p->split_groups = (int)std::min<long long>(p->nK, (2 * sms + ntiles - 1) / ntiles);
+            } else {
+                p->split_groups = f32_tile(mrows, N, p->nK, form == TDG_SYM ? Pof(L, W) : L,
+                                           form == TDG_SYM, true).groups;
+            }
         }
         for (int w : candidates(p)) {
             OpShape s = op_shape(p, w);
@@ -481,19 +482,19 @@ static PlanParams params_of(const tdgemm_plan_s *p) {
 
 // op(A)[m][k] and op(B)[k][n] as (x, k) operands of the pack kernels
 template <typename T>
-static PackOperand<T> operand_A(const tdgemm_plan_s *p, const T *A, const T *c) {
+static PackOperand<T> operand_A(const tdgemm_plan_s *p, const T *A) {
     PackOperand<T> o;
     o.src = A; o.X = p->M; o.K = p->K; o.L = p->L;
     if (p->tA == 'N') { o.sx = p->lda; o.sk = 1; } else { o.sx = 1; o.sk = p->lda; }
-    o.c = c; o.cx = p->nK; o.cl = 1;            // c_A[i][l]
+    o.mx = p->mA; o.cx = p->nK; o.cl = 1;       // [i][l]
     return o;
 }
 template <typename T>
-static PackOperand<T> operand_B(const tdgemm_plan_s *p, const T *B, const T *c) {
+static PackOperand<T> operand_B(const tdgemm_plan_s *p, const T *B) {
     PackOperand<T> o;
     o.src = B; o.X = p->N; o.K = p->K; o.L = p->L;
     if (p->tB == 'N') { o.sx = 1; o.sk = p->ldb; } else { o.sx = p->ldb; o.sk = 1; }
-    o.c = c; o.cx = 1; o.cl = p->nN;            // c_B[l][j]
+    o.mx = p->mB; o.cx = 1; o.cl = p->nN;       // [l][j]
     return o;
 }
 
@@ -533,9 +534,7 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
                                      nB ? p->N : p->K, p->ldb, nB ? 0 : 1, p->nN, p->mB, p->eB,
                                      p->L, p->dplan, fin, st));
     }
-    if (!is_tc_form(p->form))
-        CU_TRY(launch_planner<T>(pp, p->mA, p->eA, p->mB, p->eB, stab, p->dplan, p->agg,
-                                 (T *)p->cA, p->sA, (T *)p->cB, p->sB, (T *)p->pair, st));
+    CU_TRY(launch_planner(pp, stab, p->dplan, p->agg, st));
     const bool px = (p->flags & TDG_PAIR_EXACT) != 0;
     if (px)
         CU_TRY(launch_px_scales<T>(pp, p->mA, p->eA, p->mB, p->eB, p->dplan, (T *)p->cApx,
@@ -550,15 +549,6 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
             CU_TRY(launch_tile_order(p->kmask, p->nN, p->L, bm, bn, p->ktiles_m, p->ktiles_n,
                                      p->korder, st));
         }
-        OpShape s0 = op_shape(p, 0);
-        const bool directA = !nA && (p->lda * (long long)sizeof(T)) % 16 == 0 && ((uintptr_t)A & 15) == 0;
-        const bool directB = nB && (p->ldb * (long long)sizeof(T)) % 16 == 0 && ((uintptr_t)B & 15) == 0;
-        if (!directA)
-            CU_TRY(launch_pack_k<T>(operand_A<T>(p, A, nullptr), 1, p->dplan, 0, 0, (T *)p->kA,
-                                    s0.a_ld, s0.a_rows, st));
-        if (!directB && !reuse_b)
-            CU_TRY(launch_pack_k<T>(operand_B<T>(p, B, nullptr), 1, p->dplan, 0, 0, (T *)p->kB,
-                                    s0.b_ld, s0.b_rows, st));
     }
     if (is_tc_form(p->form)) {
         if constexpr (sizeof(T) == 4) {
@@ -566,44 +556,41 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
             // (target mode: the plan's gammas)
             const double gamma =
                 fp8 ? kFp8Max : p->bits > 0 ? (double)((1 << (p->bits - 1)) - 1) : 0.0;
-            const PackOperand<float> ob = operand_B<float>(p, B, nullptr);
-            CU_TRY(launch_codes(operand_A<float>(p, A, nullptr), p->mA, p->eA, p->sA, p->Abuf,
+            const PackOperand<float> ob = operand_B<float>(p, B);
+            CU_TRY(launch_codes(operand_A<float>(p, A), p->mA, p->eA, p->sA, p->Abuf,
                                 reuse_b ? nullptr : &ob, p->mB, p->eB, p->sB, p->Bbuf, fp8,
                                 tc_fused, gamma, round_up(p->K, 128), p->dplan, fin, st));
         }
     } else {
-        for (int w : candidates(p)) {
-            OpShape s = op_shape(p, w);
-            if (w == 0 || p->form == TDG_PLAIN) {
-                // plain product: k-major copies unless the caller's layout already is
-                const bool directA = !nA && (p->lda * (long long)sizeof(T)) % 16 == 0 &&
-                                     ((uintptr_t)A & 15) == 0;
-                const bool directB = nB && (p->ldb * (long long)sizeof(T)) % 16 == 0 &&
-                                     ((uintptr_t)B & 15) == 0;
-                if (!directA)
-                    CU_TRY(launch_pack_k<T>(operand_A<T>(p, A, nullptr), 1, p->dplan, 1, 0,
-                                            (T *)p->Abuf, s.a_ld, s.a_rows, st));
-                if (!directB && !reuse_b)
-                    CU_TRY(launch_pack_k<T>(operand_B<T>(p, B, nullptr), 1, p->dplan, 1, 0,
-                                            (T *)p->Bbuf, s.b_ld, s.b_rows, st));
-            } else if (px) {
-                // each CTA compands and packs its own tiles from A and B
-            } else if (p->form == TDG_SYM) {
-                if (!reuse_b)
-                    CU_TRY(launch_pack_k_pair<T>(operand_A<T>(p, A, (const T *)p->cA),
-                                                 operand_B<T>(p, B, (const T *)p->cB), w,
-                                                 p->dplan, w, (T *)p->Abuf, s.a_ld, s.a_rows,
-                                                 (T *)p->Bbuf, s.b_ld, s.b_rows, st));   // eqs. 6, 7
-                else
-                    CU_TRY(launch_pack_k<T>(operand_A<T>(p, A, (const T *)p->cA), w, p->dplan, w,
-                                            -1, (T *)p->Abuf, s.a_ld, s.a_rows, st));   // eq. 6
-            } else {
-                if (!reuse_b)
-                    CU_TRY(launch_pack_k<T>(operand_B<T>(p, B, (const T *)p->cB), 1, p->dplan, w,
-                                            0, (T *)p->Bbuf, s.b_ld, s.b_rows, st));       // b~ only
-                CU_TRY(launch_pack_x<T>(operand_A<T>(p, A, (const T *)p->cA), w, p->dplan, w, -1,
-                                        (T *)p->Abuf, s.a_ld, st));                   // eq. 11
-            }
+        PackArgs<T> a{};
+        a.A = operand_A<T>(p, A);
+        a.B = operand_B<T>(p, B);
+        // the plain product reads an operand in place where its layout and
+        // alignment fit
+        a.directA = !nA && (p->lda * (long long)sizeof(T)) % 16 == 0 && ((uintptr_t)A & 15) == 0;
+        a.directB = nB && (p->ldb * (long long)sizeof(T)) % 16 == 0 && ((uintptr_t)B & 15) == 0;
+        a.skipB = reuse_b;
+        a.L = p->L; a.nM = p->nM; a.nK = p->nK; a.nN = p->nN;
+        a.target = p->mode == MODE_TARGET;
+        a.plain = p->form == TDG_PLAIN;
+        a.plain_only = px;                    // (each CTA compands and packs its own tiles)
+        a.manual = p->mode == MODE_MANUAL;
+        a.manual_cA = p->manual_cA;
+        a.manual_cB = p->manual_cB;
+        a.outA = (T *)p->Abuf;
+        a.outB = (T *)p->Bbuf;
+        for (int w = 0; w <= kMaxW; ++w) a.ldoA[w] = op_shape(p, w).a_ld;
+        a.ldoB = op_shape(p, p->W).b_ld;
+        a.pair = p->form == TDG_PLAIN || px ? nullptr : (T *)p->pair;
+        if (!px || a.target) CU_TRY(launch_pack<T>(p->form == TDG_ASYM, a, p->dplan, st));
+        if (p->kctrl_mode) {
+            // Sec. 6: plain copies for the inner kernels left unaccelerated
+            a.plain = 1;
+            a.pair = nullptr;
+            a.outA = (T *)p->kA;
+            a.outB = (T *)p->kB;
+            if (!(a.directA && (a.directB || reuse_b)))
+                CU_TRY(launch_pack<T>(false, a, p->dplan, st));
         }
     }
     p->clear_record = false;
@@ -658,8 +645,23 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
             ((uintptr_t)p->B_user & 15) == 0)
             b = {p->B_user, s.b_cols, s.b_rows, p->ldb};
     };
+    // a distortion target's product: the symmetric form in one launch for every
+    // candidate, the asymmetric one in a launch per W, the last of them holding
+    // the plain fallback too (mixed, pair-exact and large fp32 products: apart)
+    bool one_launch = p->mode == MODE_TARGET && is_packed_form(p->form) && !p->kctrl_mode &&
+                      !(p->flags & TDG_PAIR_EXACT);
+    if constexpr (sizeof(T) == 4) {
+        if (one_launch) {
+            GemmArgs<float> g{};
+            g.M = p->M; g.N = p->N; g.nK = p->nK; g.L = p->L; g.Rbar = (float *)p->Rbar;
+            // (one rule for all candidates: that of W = 2)
+            g.Mrows = op_shape(p, 2).a_cols;
+            one_launch = f32_target_in_one_launch(p->form == TDG_SYM ? G_SYM : G_ASYM, 2, g);
+        }
+    }
     for (int w : candidates(p)) {
         const bool plain = (w == 0 || p->form == TDG_PLAIN);
+        if (one_launch && (w == 0 || (p->form == TDG_SYM && w > 2))) continue;
         const int gform = plain ? G_PLAIN : (p->form == TDG_SYM ? G_SYM : G_ASYM);
         const int Wk = plain ? 1 : w;
         OpShape s = op_shape(p, w);
@@ -682,6 +684,11 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
         g.alpha = (T)alpha; g.beta = (T)beta; g.beta_zero = beta == 0.0;
         g.Rbar = (!plain && (p->flags & TDG_KEEP_PACKED)) ? (T *)p->Rbar : nullptr;
         g.stall_ns = p->stall_ns;
+        if (one_launch) {
+            g.target = 1;
+            g.fallback = w == 2 && (p->flags & TDG_ALLOW_FALLBACK);
+            if (g.fallback) plain_ops(p->Abuf, p->Bbuf, ops.pa, ops.pb);
+        }
         if (p->mode == MODE_FIXED) {
             const long long gam = (1LL << (p->bits - 1)) - 1;
             g.small_t = small_round_ok(gform, Wk, q_for((long long)p->L * gam * gam), (int)gam) ? 1 : 0;
@@ -717,7 +724,9 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
             return fail(TDG_ECUDA, "packed GEMM: an operand could not be mapped for TMA");
         if (e != cudaSuccess)
             return fail(TDG_ECUDA, "packed GEMM launch failed: %s", cudaGetErrorString(e));
-        if (split) CU_TRY(launch_unpack<T>(gform, Wk, g, nullptr, st));   // sum over slabs, C
+        // sum over slabs, C (symmetric targets: whichever W the plan holds)
+        if (split)
+            CU_TRY(launch_unpack<T>(gform, one_launch && gform == G_SYM ? 0 : Wk, g, nullptr, st));
     }
     return TDG_OK;
 }

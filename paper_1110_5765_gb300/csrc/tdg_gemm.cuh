@@ -187,8 +187,10 @@ __host__ __device__ constexpr int pow2_at_least(int v) {
     return p;
 }
 
-template <typename T, int FORM, int W, int BM, int BN, int TM, int TN, int BK, int STAGES>
+template <typename T, int FORM, int W, typename C>
 struct GemmCfg {
+    static constexpr int BM = C::BM, BN = C::BN, TM = C::TM, TN = C::TN, BK = C::BK,
+                         STAGES = C::STAGES;
     static constexpr int NT = (BM / TM) * (BN / TN);   // threads (16 x 16)
     static constexpr int GR = TM < 4 ? TM : 4, GC = TN < 4 ? TN : 4;   // fragment group widths
     static constexpr int RG = TM / GR, CG = TN / GC;   // fragment groups
@@ -215,14 +217,15 @@ struct GemmCfg {
 template <typename T, int FORM>
 struct SlabWalk {
     const GemmArgs<T> &g;
+    int P;
     __device__ inline int nslab() const { return FORM == G_PLAIN ? 1 : g.nK; }
     __device__ inline int len(int l) const {
-        if (FORM == G_SYM) return g.P;
+        if (FORM == G_SYM) return P;
         if (FORM == G_ASYM) return (int)min((long long)g.L, g.K - (long long)l * g.L);
         return (int)g.K;
     }
     __device__ inline long long row0(int l) const {
-        if (FORM == G_SYM) return (long long)l * g.P;
+        if (FORM == G_SYM) return (long long)l * P;
         if (FORM == G_ASYM) return (long long)l * g.L;
         return 0;
     }
@@ -233,26 +236,17 @@ struct SlabWalk {
 // chain over all of K from the plain operands, no slab epilogue) instead of
 // the packed one.  Tiles never straddle inner kernels (L is a multiple of the
 // tile), and the block scheduler balances the two kinds of tile.
-template <typename T, int FORM, int W, int BM, int BN, int TM, int TN, int BK, int STAGES,
-          bool KEEP, bool MIX, bool SMALL_T = false>
-__global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES>::NT,
-                                  GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES>::MIN_CTAS)
-    packed_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
-                       const __grid_constant__ CUtensorMap mapB,
-                       const __grid_constant__ CUtensorMap mapPA,
-                       const __grid_constant__ CUtensorMap mapPB, const GemmArgs<T> g) {
-    pdl_entry();
-    using Cfg = GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES>;
+// Wp: the packing that runs; P: its packed numbers per block.
+template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, int RND>
+__device__ __forceinline__ void packed_gemm_tile(const CUtensorMap &mapA, const CUtensorMap &mapB,
+                                                 const CUtensorMap &mapPA, const CUtensorMap &mapPB,
+                                                 const GemmArgs<T> &g, const int Wp, const int P) {
+    constexpr int BM = C::BM, BN = C::BN, TM = C::TM, TN = C::TN, BK = C::BK, STAGES = C::STAGES;
+    using Cfg = GemmCfg<T, FORM, W, C>;
     constexpr int RG = Cfg::RG, CG = Cfg::CG, GR = Cfg::GR, GC = Cfg::GC, NCACC = Cfg::NCACC;
     constexpr bool TMEMC = Cfg::TMEMC;
     static_assert(!MIX || (FORM == G_SYM && !KEEP), "mixed tiles: symmetric form only");
 
-    // the device planner chose another packing
-    if (g.plan->W != g.W) return;
-    // both rounding variants queued: the one the plan does not select exits
-    if constexpr (sizeof(T) == 4 && ((FORM == G_SYM && W == 2) || FORM == G_ASYM) && !KEEP) {
-        if (g.small_t < 0 && small_round_ok(FORM, W, g.plan->q, g.plan->gA) != SMALL_T) return;
-    }
     // this CTA's tile, row-major over ntn tiles per row; with slab splitting
     // (KEEP instantiation, groups > 1) CTA b takes tile b % ntiles and the
     // slabs of group b / ntiles
@@ -261,6 +255,8 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
     if constexpr (MIX) {
         if (g.tile_order) tix = g.tile_order[blockIdx.x];
     }
+    // (a launch that may compute one of two products has CTAs for the larger grid)
+    if ((long long)blockIdx.x >= g.ntiles * g.groups) return;
     const long long tmi = tix / g.ntn;
     const long long x0 = tmi * BM;                      // first A-operand column (m or packed row)
     const long long n0 = (tix - tmi * g.ntn) * BN;
@@ -280,8 +276,8 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
-    const SlabWalk<T, FORM> walk{g};
-    const SlabWalk<T, G_PLAIN> pwalk{g};
+    const SlabWalk<T, FORM> walk{g, P};
+    const SlabWalk<T, G_PLAIN> pwalk{g, P};
     const int nslab_all = plain_tile ? 1 : walk.nslab();
     const int l_begin = split ? (int)((long long)blockIdx.x / g.ntiles) * g.spg : 0;
     const int nslab = split ? min(nslab_all, l_begin + g.spg) : nslab_all;   // end of this CTA's slabs
@@ -336,6 +332,8 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
 
     T z = T(1), Q = T(1);
     int q = 0;
+    // which of the two roundings the plan's values allow (RND = 2: known here only)
+    const bool small = RND == 2 && small_round_ok(FORM, Wp, g.plan->q, g.plan->gA);
     if (FORM != G_PLAIN) {
         q = g.plan->q;
         z = pow2_t(T(0), -q);
@@ -352,7 +350,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
 #pragma unroll
         for (int e = 0; e < GR; ++e) {
             long long xr = x0 + gi * (BM / RG) + ty * GR + e;
-            long long ib = FORM == G_ASYM ? xr / g.P : xr / g.L;
+            long long ib = FORM == G_ASYM ? xr / P : xr / g.L;
             iblk[gi * GR + e] = (int)min(ib, (long long)g.nM - 1);
         }
 #pragma unroll
@@ -365,7 +363,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
     auto out_row = [&](int i, int d) -> long long {
         const long long xr = x0 + (i / GR) * (BM / RG) + ty * GR + (i % GR);
         if (FORM == G_ASYM) {
-            const long long ib = xr / g.P, jr = xr % g.P;
+            const long long ib = xr / P, jr = xr % P;
             const long long inblk = jr * W + d;
             if (inblk >= g.L) return -1;
             return ib * g.L + inblk;
@@ -495,6 +493,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
             uint64_t z2, nq2;
             asm("mov.b64 %0, {%1, %1};" : "=l"(z2) : "f"((float)z));
             asm("mov.b64 %0, {%1, %1};" : "=l"(nq2) : "f"(-(float)Q));
+            auto slab_end = [&](auto small) {
 #pragma unroll
             for (int e = 0; e < TM * TN; e += 2) {
                 const int i = e / TN, j = e % TN, slot = e % 16;
@@ -507,7 +506,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                 asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t2) : "l"(z2), "l"(u2));
                 float t0, t1;
                 asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(t2));
-                if constexpr (SMALL_T) {
+                if constexpr (decltype(small)::value) {
                     t0 = rint_small(t0);
                     t1 = rint_small(t1);
                 } else {
@@ -529,12 +528,20 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                 asm("mov.b64 {%0, %1}, %2;" : "=f"(v[slot]), "=f"(v[slot + 1]) : "l"(v2));
                 if (slot == 14) tmem_st16(tcol + (uint32_t)(e - 14), v);
             }
+            };
+            if constexpr (RND == 2) {
+                if (small) slab_end(std::true_type{});
+                else slab_end(std::false_type{});
+            } else {
+                slab_end(std::bool_constant<RND == 1>{});
+            }
             tmem_wait_st();
             continue;
         }
         // fp64: the digits by integer arithmetic (tdg_digits.cuh), in 32-bit
         // words where q allows
-        auto slab_end = [&](auto narrow) {
+        // (fp32: variant = the add-subtract rounding)
+        auto slab_end = [&](auto variant) {
 #pragma unroll
         for (int e = 0; e < TM * TN; ++e) {
             const int i = e / TN, j = e % TN;
@@ -548,7 +555,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
             }
             T digit[NCACC];
             if constexpr (sizeof(T) == 8) {
-                if constexpr (FORM == G_SYM) digit[0] = sym_digit<decltype(narrow)::value>(r, q);
+                if constexpr (FORM == G_SYM) digit[0] = sym_digit<decltype(variant)::value>(r, q);
                 else if constexpr (FORM == G_ASYM) asym_digits<NCACC>(r, q, digit);
             } else if (FORM == G_SYM) {
                 const T u = rint_epi(r);                        // eq. 9
@@ -558,7 +565,7 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
                 T x = r;
 #pragma unroll
                 for (int d = 0; d < NCACC; ++d) {               // eqs. 13-14
-                    if constexpr (SMALL_T) digit[d] = rint_small(x);
+                    if constexpr (decltype(variant)::value) digit[d] = rint_small(x);
                     else digit[d] = rint_epi(x);
                     if (d + 1 < NCACC) x = mul_rn(Q, sub_rn(x, digit[d]));
                 }
@@ -586,8 +593,11 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
         if constexpr (sizeof(T) == 8 && FORM == G_SYM) {
             if (q <= 31) slab_end(std::true_type{});
             else slab_end(std::false_type{});
+        } else if constexpr (FORM == G_ASYM && RND == 2) {
+            if (small) slab_end(std::true_type{});
+            else slab_end(std::false_type{});
         } else {
-            slab_end(std::false_type{});
+            slab_end(std::bool_constant<RND == 1>{});
         }
         if constexpr (TMEMC) tmem_wait_st();
     }
@@ -654,6 +664,61 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, BM, BN, TM, TN, BK, STAGES
     }
 }
 
+// One product of known packing (fixed bits, manual companders, the plain form)
+// or one candidate's mixed tiles (Sec. 6).
+// RND: the fp32 unpack's roundings by add-subtract (1), by rint (0), or
+// whichever the plan's values allow (2).
+template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, int RND>
+__global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W, C>::MIN_CTAS)
+    packed_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
+                       const __grid_constant__ CUtensorMap mapB,
+                       const __grid_constant__ CUtensorMap mapPA,
+                       const __grid_constant__ CUtensorMap mapPB,
+                       const __grid_constant__ GemmArgs<T> g) {
+    pdl_entry();
+    // the device planner chose another packing
+    if (g.plan->W != g.W) return;
+    // both rounding variants queued: the one the plan does not select exits
+    if constexpr (sizeof(T) == 4 && FORM != G_PLAIN && !KEEP && RND < 2) {
+        if (g.small_t < 0 && small_round_ok(FORM, g.W, g.plan->q, g.plan->gA) != (RND == 1)) return;
+    }
+    packed_gemm_tile<T, FORM, W, C, KEEP, MIX, RND>(mapA, mapB, mapPA, mapPB, g, g.W, g.P);
+}
+
+// A distortion target's product in one launch: the packing, and whether the
+// target was met at all, are known on the device only.  The packed product
+// (symmetric: of any W, only the operand rows differ) is inlined, the plain
+// fallback (tile CP, arguments gp) called, which keeps their registers apart.
+// As launches of their own, the ones not chosen took 2 to 7 us each to return at
+// entry.  Not for the unsplit fp32 product in 8 x 8 thread tiles, which has no
+// register to spare (1.155 ms instead of 1.106 at 4096^3): there both rounding
+// variants and the fallback are queued.
+template <typename T, typename CP>
+static __device__ __noinline__ void plain_gemm_apart(const CUtensorMap &mapA,
+                                                     const CUtensorMap &mapB,
+                                                     const GemmArgs<T> &g) {
+    packed_gemm_tile<T, G_PLAIN, 1, CP, false, false, 0>(mapA, mapB, mapA, mapB, g, 1, 0);
+}
+
+template <typename T, int FORM, int W, typename C, typename CP, bool KEEP>
+__global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W, C>::MIN_CTAS)
+    target_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
+                       const __grid_constant__ CUtensorMap mapB,
+                       const __grid_constant__ CUtensorMap mapPA,
+                       const __grid_constant__ CUtensorMap mapPB,
+                       const __grid_constant__ GemmArgs<T> g,
+                       const __grid_constant__ GemmArgs<T> gp) {
+    pdl_entry();
+    const int Wp = g.plan->W;
+    if (Wp == 1) {
+        if (g.fallback) plain_gemm_apart<T, CP>(mapPA, mapPB, gp);
+        return;
+    }
+    if (FORM == G_ASYM && Wp != g.W) return;
+    packed_gemm_tile<T, FORM, W, C, KEEP, false, sizeof(T) == 4 && !KEEP ? 2 : 0>(
+        mapA, mapB, mapA, mapB, g, Wp, (g.L + Wp - 1) / Wp);
+}
+
 // Shared memory that a CTA of a small grid asks for so that its CTAs spread
 // evenly: with n CTAs on S SMs, no SM gets more than ceil(n / S).  Launched
 // programmatically, CTAs start where the kernel before leaves room first and
@@ -666,83 +731,116 @@ inline size_t spread_smem(long long nblocks) {
     return std::min<size_t>(kMaxCtaSmem, (size_t)(kSmemPerSm / r - 1024) / 1024 * 1024);
 }
 
-// One launch over the whole tile grid of shape C.
-template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, bool SMALL_T = false>
-cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStream_t st) {
-    using Cfg = GemmCfg<T, FORM, W, C::BM, C::BN, C::TM, C::TN, C::BK, C::STAGES>;
-    auto kern = packed_gemm_kernel<T, FORM, W, C::BM, C::BN, C::TM, C::TN, C::BK, C::STAGES, KEEP,
-                                   MIX, SMALL_T>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCtaSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+template <typename T, typename C>
+bool map_operand(CUtensorMap *m, const GemmOperand &o, int box) {
     const CUtensorMapDataType dt =
         sizeof(T) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-    auto map = [&](CUtensorMap *m, const GemmOperand &o, int box) {
-        return encode_map_2d(m, dt, sizeof(T), o.base, o.cols, o.rows, o.ld, box, C::BK,
-                             CU_TENSOR_MAP_SWIZZLE_NONE) == CUDA_SUCCESS;
-    };
-    CUtensorMap ma, mb, mpa, mpb;
-    if (!map(&ma, ops.a, C::BM) || !map(&mb, ops.b, C::BN)) return cudaErrorInvalidValue;
-    if (MIX) {
-        if (!map(&mpa, ops.pa, C::BM) || !map(&mpb, ops.pb, C::BN)) return cudaErrorInvalidValue;
-    } else {
-        mpa = ma;
-        mpb = mb;
-    }
-    GemmArgs<T> g = g0;
+    return encode_map_2d(m, dt, sizeof(T), o.base, o.cols, o.rows, o.ld, box, C::BK,
+                         CU_TENSOR_MAP_SWIZZLE_NONE) == CUDA_SUCCESS;
+}
+
+// the tile grid of shape C in g; returns its CTAs
+template <typename T, int FORM, typename C, bool KEEP>
+long long set_grid(GemmArgs<T> &g) {
     g.ntn = (int)((g.N + C::BN - 1) / C::BN);
-    const long long ntiles = ((g.Mrows + C::BM - 1) / C::BM) * g.ntn;
-    g.ntiles = ntiles;
-    long long nblocks = ntiles;
+    g.ntiles = ((g.Mrows + C::BM - 1) / C::BM) * g.ntn;
     if (KEEP && g.groups > 1) {
         // slab splitting: groups of spg consecutive slabs per CTA
         const int nsl = FORM == G_PLAIN ? 1 : g.nK;
         g.spg = (nsl + g.groups - 1) / g.groups;
         g.groups = (nsl + g.spg - 1) / g.spg;
-        nblocks = ntiles * g.groups;
     } else {
         g.groups = 1;
     }
+    return g.ntiles * g.groups;
+}
+
+// One launch over the whole tile grid of shape C.
+template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, int RND = 0>
+cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStream_t st) {
+    using Cfg = GemmCfg<T, FORM, W, C>;
+    auto kern = packed_gemm_kernel<T, FORM, W, C, KEEP, MIX, RND>;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCtaSmem);
+    if (attr != cudaSuccess) return attr;
+    CUtensorMap ma, mb, mpa, mpb;
+    if (!map_operand<T, C>(&ma, ops.a, C::BM) || !map_operand<T, C>(&mb, ops.b, C::BN))
+        return cudaErrorInvalidValue;
+    if (MIX) {
+        if (!map_operand<T, C>(&mpa, ops.pa, C::BM) || !map_operand<T, C>(&mpb, ops.pb, C::BN))
+            return cudaErrorInvalidValue;
+    } else {
+        mpa = ma;
+        mpb = mb;
+    }
+    GemmArgs<T> g = g0;
+    const long long nblocks = set_grid<T, FORM, C, KEEP>(g);
     if (nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     return launch_pdl(kern, dim3((unsigned)nblocks), dim3(Cfg::NT),
                       std::max(Cfg::SMEM, spread_smem(nblocks)), st, ma, mb, mpa, mpb, g);
 }
 
+// A distortion target's product (target_gemm_kernel); ops.pa, ops.pb: the plain
+// operands when g.fallback.
+template <typename T, int FORM, int W, typename C, typename CP, bool KEEP>
+cudaError_t launch_target(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStream_t st) {
+    using Cfg = GemmCfg<T, FORM, W, C>;
+    using CfgP = GemmCfg<T, G_PLAIN, 1, CP>;
+    static_assert((int)Cfg::NT == (int)CfgP::NT, "one block shape");
+    auto kern = target_gemm_kernel<T, FORM, W, C, CP, KEEP>;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCtaSmem);
+    if (attr != cudaSuccess) return attr;
+    CUtensorMap ma, mb, mpa, mpb;
+    if (!map_operand<T, C>(&ma, ops.a, C::BM) || !map_operand<T, C>(&mb, ops.b, C::BN))
+        return cudaErrorInvalidValue;
+    GemmArgs<T> g = g0, gp = g0;
+    long long nblocks = set_grid<T, FORM, C, KEEP>(g);
+    size_t smem = std::max(Cfg::SMEM, spread_smem(nblocks));
+    if (g.fallback) {
+        if (!map_operand<T, CP>(&mpa, ops.pa, CP::BM) || !map_operand<T, CP>(&mpb, ops.pb, CP::BN))
+            return cudaErrorInvalidValue;
+        gp.Mrows = gp.M;
+        gp.Rbar = nullptr;
+        gp.groups = 1;
+        nblocks = std::max(nblocks, set_grid<T, G_PLAIN, CP, false>(gp));
+        smem = std::max(smem, CfgP::SMEM);
+    } else {
+        mpa = ma;
+        mpb = mb;
+    }
+    if (nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    return launch_pdl(kern, dim3((unsigned)nblocks), dim3(Cfg::NT), smem, st, ma, mb, mpa, mpb, g, gp);
+}
+
 // KEEP (store every packed slab result for tdgemm_unpack) and MIX (Sec. 6
 // mixed tiles) are separate instantiations so the usual kernel carries none of
-// that code.
-template <typename T, int FORM, int W, typename C>
+// that code.  CP: the plain fallback's tile.
+template <typename T, int FORM, int W, typename C, typename CP>
 cudaError_t launch_cfg(const GemmArgs<T> &g, const GemmOperands &ops, cudaStream_t st) {
     if constexpr (FORM == G_SYM && C::TM >= 4) {
         if (g.kmask) {
             if (g.Rbar || !ops.pa.base || !ops.pb.base) return cudaErrorInvalidValue;
-            if constexpr (sizeof(T) == 4 && W == 2) {
-                // the packed tiles' unpack rounding as for the unmixed kernel
-                if (g.small_t > 0) return launch_grid<T, FORM, W, C, false, true, true>(g, ops, st);
-                if (g.small_t < 0) {
-                    cudaError_t e = launch_grid<T, FORM, W, C, false, true, true>(g, ops, st);
-                    if (e != cudaSuccess) return e;
-                }
-            }
+            if constexpr (sizeof(T) == 4)
+                return g.small_t < 0   ? launch_grid<T, FORM, W, C, false, true, 2>(g, ops, st)
+                       : g.small_t > 0 ? launch_grid<T, FORM, W, C, false, true, 1>(g, ops, st)
+                                       : launch_grid<T, FORM, W, C, false, true, 0>(g, ops, st);
             return launch_grid<T, FORM, W, C, false, true>(g, ops, st);
         }
     }
     if (g.kmask) return cudaErrorInvalidValue;
     if constexpr (FORM != G_PLAIN) {
+        if (g.target && g.Rbar) return launch_target<T, FORM, W, C, CP, true>(g, ops, st);
+        if constexpr (sizeof(T) == 8 || C::TM * C::TN < 64)
+            if (g.target) return launch_target<T, FORM, W, C, CP, false>(g, ops, st);
         if (g.Rbar) return launch_grid<T, FORM, W, C, true, false>(g, ops, st);
     }
     if (g.groups > 1) return cudaErrorInvalidValue;     // slab splitting stores r-bar
-    if constexpr (sizeof(T) == 4 && ((FORM == G_SYM && W == 2) || (FORM == G_ASYM && W >= 2))) {
-        // the unpack's roundings as a compile-time variant: known on the host
-        // for fixed-bit plans, else both queued and the plan picks one
-        if (g.small_t > 0) return launch_grid<T, FORM, W, C, false, false, true>(g, ops, st);
-        if (g.small_t < 0) {
-            cudaError_t e = launch_grid<T, FORM, W, C, false, false, true>(g, ops, st);
-            if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4 && FORM != G_PLAIN) {
+        // known on the host for fixed bits, else both queued and the plan picks one
+        if (g.small_t != 0) {
+            cudaError_t e = launch_grid<T, FORM, W, C, false, false, 1>(g, ops, st);
+            if (e != cudaSuccess || g.small_t > 0) return e;
         }
     }
     return launch_grid<T, FORM, W, C, false, false>(g, ops, st);

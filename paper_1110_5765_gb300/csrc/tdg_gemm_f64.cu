@@ -30,9 +30,9 @@ template <int FORM, int W>
 static cudaError_t go(const GemmArgs<double> &g, const GemmOperands &ops, cudaStream_t st) {
     // mixed tiles (Sec. 6) keep the tile that the tile order was made for
     const int edge = g.kmask ? 64 : f64_tile_edge(g.Mrows, g.N);
-    if (edge == 64) return launch_cfg<double, FORM, W, TilesF64>(g, ops, st);
-    if (edge == 32) return launch_cfg<double, FORM, W, TilesF64Mid>(g, ops, st);
-    return launch_cfg<double, FORM, W, TilesF64Small>(g, ops, st);
+    if (edge == 64) return launch_cfg<double, FORM, W, TilesF64, TilesF64>(g, ops, st);
+    if (edge == 32) return launch_cfg<double, FORM, W, TilesF64Mid, TilesF64Mid>(g, ops, st);
+    return launch_cfg<double, FORM, W, TilesF64Small, TilesF64Small>(g, ops, st);
 }
 
 template <>

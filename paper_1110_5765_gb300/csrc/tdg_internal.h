@@ -11,14 +11,14 @@ namespace tdg {
 
 enum GemmForm { G_PLAIN = 0, G_SYM = 1, G_ASYM = 2 };
 
-// One operand of a pack kernel: op(X)[x][k] = src[x * sx + k * sk], x < X,
-// k < K, with per-block companders c[(x / L) * cx + (k / L) * cl] (nullptr:
-// plain copy).
+// One operand of a pack or code kernel: op(X)[x][k] = src[x * sx + k * sk],
+// x < X, k < K, one of sx and sk 1; block (x / L, k / L) has index
+// (x / L) * cx + (k / L) * cl in the statistics (mx: its max|x|).
 template <typename T>
 struct PackOperand {
     const T *src;
     long long sx, sk, X, K;
-    const T *c;
+    const double *mx;
     long long cx, cl;
     int L;
 };
@@ -37,17 +37,12 @@ cudaError_t launch_block_stats(const T *A, long long rows_a, long long cols_a, l
                                int nbc_b, double *mxB, double *varB, int L, DevPlan *plan,
                                const SlabFinish &fin, cudaStream_t st);
 
-// Planner, after the statistics (which leave the sums over slabs in the plan
-// record or, outside target mode, the plan): agg is 4 nK + kLevelRecDoubles
-// (kMaxW - 1) kMaxLevels doubles of workspace, the per-slab aggregates and one
-// record per candidate (W, level).  Writes the
-// choice of W / z / companders into *plan, then c, s per block and the
-// de-companding factors.
-template <typename T>
-cudaError_t launch_planner(const PlanParams &pp, const double *mA, const double *eA,
-                           const double *mB, const double *eB, const double *stab,
-                           DevPlan *plan, double *agg, T *cA, double *sA, T *cB, double *sB,
-                           T *pair, cudaStream_t st);
+// Planner, where the statistics did not decide the plan: target mode's
+// candidates (agg: 4 nK + kLevelRecDoubles (kMaxW - 1) kMaxLevels doubles of
+// workspace, the per-slab aggregates and one record per candidate (W, level)),
+// and calls without statistics.
+cudaError_t launch_planner(const PlanParams &pp, const double *stab, DevPlan *plan, double *agg,
+                           cudaStream_t st);
 
 // Launch order of the tiles of a mixed (Sec. 6) launch: the tiles of
 // unaccelerated inner kernels first, then the accelerated ones, each group in
@@ -71,18 +66,6 @@ cudaError_t launch_kernel_control(const PlanParams &pp, const double *mA, const 
                                   int mode, double thr, long long k, double F,
                                   const Speedups &fw, double *ratio, unsigned char *mask,
                                   cudaStream_t st);
-
-// Pack kernels run only when the device plan's W equals expectW (expectW = 0:
-// always); W is the
-// packing of the kernel itself; wsign < 0 packs with z, > 0 with z^-1;
-// rows_out bounds the rows written to the k-major output.
-template <typename T>
-cudaError_t launch_pack_k(const PackOperand<T> &o, int W, const DevPlan *plan, int expectW,
-                          int wsign, T *out, long long ldo, long long rows_out, cudaStream_t st);
-
-template <typename T>
-cudaError_t launch_pack_x(const PackOperand<T> &o, int W, const DevPlan *plan, int expectW,
-                          int wsign, T *out, long long ldo, cudaStream_t st);
 
 // Codes of op(A) and, when b is given, op(B) for the tensor-core forms, with s =
 // 1/c in fp64 per block.  fused: companders of the block's own maximum (c =
@@ -128,10 +111,12 @@ struct GemmArgs {
     // test of the bounded waits: > 0 makes every CTA's first wait for operand
     // tiles wait on a barrier nothing completes, giving up after this many ns
     long long stall_ns;
-    // fp32 symmetric W = 2: whether the second rounding of eq. 10 may use the
-    // add-subtract form (|z u| < 2^22, see the kernel): 1 known yes, 0 known
-    // no, -1 decided on the device (both variants queued, one runs)
+    // fp32: whether the unpack's roundings may use the add-subtract form
+    // (small_round_ok): 1 known yes, 0 known no, -1 decided on the device
     int small_t;
+    // distortion targets: the device plan holds W (symmetric form: any) ...
+    int target;
+    int fallback;           // ... or 1, and this launch then computes the plain product
 };
 
 // 2-D TMA map over a row-major [rows][cols] array with leading dimension ld
@@ -178,6 +163,17 @@ cudaError_t launch_px_gemm(int W, const GemmArgs<T> &g, const GemmOperands &ops,
 // (fp64: the largest tile, which mixed launches use; f64_tile_edge gives the
 // edge of the others).
 int f64_tile_edge(long long mrows, long long ncols);
+// fp32 packed products: the tile, and how many groups the slabs are split into
+// (1: not split); wide: 128 x 64 tiles are among the choices (symmetric form)
+enum { F32_TILE_128 = 0, F32_TILE_MID = 1, F32_TILE_SMALL = 2 };
+struct F32Tile {
+    int tile, groups;
+};
+F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, bool wide,
+                 bool may_split);
+// whether a distortion target's product needs one launch only (symmetric: for
+// every W; with the plain fallback)
+bool f32_target_in_one_launch(int form, int W, const GemmArgs<float> &g);
 void packed_gemm_boxes(int dtype, int form, int W, int *box_x_a, int *box_x_b, int *bk);
 
 template <typename T>

@@ -1,25 +1,31 @@
 // Steps (a) and (b) on the data: companding and rounding (eq. 3) fused with
-// packing (eqs. 6, 7, 11) in one pass over each input.
+// packing (eqs. 6, 7, 11), both operands and every packing the planner may have
+// chosen in one launch, with the de-companding factors beside them.
 //
 // Every element is quantized as a~ = rint(fl_T(x * c_T)) with its block's
-// compander and the packed number is built by Horner's rule,
+// compander c = gamma / max|x| and the packed number is built by Horner's rule,
 //     acc = d_{W-1};  acc = fma(w, acc, d_i),  i = W-2 .. 0,
 // with w = z for eqs. 6 and 11 and w = z^-1 for eq. 7.  Digits outside the
-// L x L block or the matrix are zero (border clean-up, Sec. 2).
+// L x L block or the matrix are zero (border clean-up, Sec. 2).  P = ceil(L / W)
+// packed numbers per block.
 //
-//   pack along k   out[l P + j][x]  (eq. 6 for A, eq. 7 for B, W = 1 for the
-//                  unpacked operands and the plain copies):
-//                    - x contiguous in the input: 16-byte vector loads of the
-//                      W digit rows, vector stores, no shared memory;
-//                    - k contiguous in the input: a TILE x TILE W tile (TILE =
-//                      64 x-rows for fp32 with W <= 2, else 32) staged in
-//                      shared memory with vector loads, then written along x.
-//   pack along x   out[k][i P + j]  (eq. 11, asymmetric A), tile staged in
-//                  shared memory.
-// P = ceil(L / W) packed numbers per block.  Each kernel first reads the
-// device plan and returns unless the planner chose its packing; the grids are
-// capped and loop over tiles so that such early exits cost little.
-#include <mutex>
+//   along k  out[l P + j][x]  eq. 6 for A, eq. 7 for B; W = 1 for the unpacked
+//                             operands and the plain copies
+//   along x  out[k][i P + j]  eq. 11, the asymmetric A
+// A thread packs G consecutive numbers from whole 16-byte vectors where the
+// packing direction is the contiguous one, else one vector of numbers from W
+// rows.  Results that lie across the output's rows go through shared memory
+// (column c of a group's member g at g * groups + c: no bank conflicts either
+// way); the others are stored as vectors.
+//
+// The kernel reads W from the device plan: one launch serves every candidate of
+// a distortion target and the plain fallback, and takes c from the block maxima
+// itself.  Launched apart (companders, factors, one pack and one plain copy per
+// operand, each candidate's kernels returning at entry), this step was 6 to 9
+// launches and 15 to 20 us of a small product.
+#include <limits.h>
+
+#include <algorithm>
 
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
@@ -29,39 +35,9 @@ namespace tdg {
 
 namespace {
 
-constexpr int TILE = 32;
-constexpr int MAX_CTAS = 152 * 8;
-
-template <typename T>
-struct Src {
-    const T *p;
-    long long sx, sk;
-    long long X, K;
-    const T *c;       // nullptr: copy without companding
-    long long cx, cl;
-    int L;
-};
-
-template <typename T>
-__device__ inline T quant(T v, T c, bool compand) {
-    if (!compand) return v;
-    if constexpr (sizeof(T) == 4) return rintf(__fmul_rn(v, c));
-    else return rint(__dmul_rn(v, c));
-}
-
-template <typename T>
-__device__ inline T fma_t(T a, T b, T c) {
-    if constexpr (sizeof(T) == 4) return __fmaf_rn(a, b, c);
-    else return __fma_rn(a, b, c);
-}
-
-// w = z = 2^-q (wsign < 0) or z^-1 = 2^q (wsign > 0), q from the device plan
-template <typename T>
-__device__ inline T pack_weight(const DevPlan *plan, int wsign) {
-    int q = plan->q;
-    if constexpr (sizeof(T) == 4) return scalbnf(1.0f, wsign < 0 ? -q : q);
-    else return scalbn(1.0, wsign < 0 ? -q : q);
-}
+constexpr int NT = 256;
+constexpr int KSPAN = 128;          // values along the packed dimension per tile (132 for W = 3)
+constexpr int PAIR_TILE = 64;       // factors per tile and side
 
 template <typename T>
 struct VecT;
@@ -80,493 +56,412 @@ __device__ inline void vload(const T *p, T *o) {
         o[0] = v.x; o[1] = v.y;
     }
 }
-
 template <typename T>
 __device__ inline void vstore(T *p, const T *o) {
     if constexpr (sizeof(T) == 4) *reinterpret_cast<float4 *>(p) = make_float4(o[0], o[1], o[2], o[3]);
     else *reinterpret_cast<double2 *>(p) = make_double2(o[0], o[1]);
 }
 
-// ------------------------------------------------------------------ pack along k,
-// x contiguous in the input: one item = VEC consecutive x of one packed row
-// (the loop of CTA vb of vg working on this operand)
-template <typename T, int W>
-__device__ __forceinline__ void pack_k_xc_body(const Src<T> &S, int P, T w, T *out, long long ldo,
-                                               long long rows_out, int vec_ok, long long vb,
-                                               long long vg) {
-    constexpr int VEC = VecT<T>::n;
-    const bool compand = S.c != nullptr;
-    const int L = S.L;
-    const long long nx = (S.X + VEC - 1) / VEC;
-    const long long items = rows_out * nx;
-    for (long long it = vb * blockDim.x + threadIdx.x; it < items; it += vg * blockDim.x) {
-        const long long row = it / nx;                 // l * P + j
-        const long long x = (it - row * nx) * VEC;
-        const int l = (int)(row / P), j = (int)(row - (long long)l * P);
-        const long long kbase = (long long)l * L + (long long)W * j;
-        const long long klim = min((long long)(l + 1) * L, S.K);
-        const T c = compand ? S.c[(x / L) * S.cx + (long long)l * S.cl] : T(1);
-        T acc[VEC];
-        const bool full = vec_ok && x + VEC <= S.X;
+// n <= N values from p (vec: n = N and 16-byte aligned), zeros after them
+template <typename T, int N>
+__device__ inline void load_run(const T *p, int n, bool vec, T (&d)[N]) {
+    if (vec && n >= N) {
 #pragma unroll
-        for (int i = W - 1; i >= 0; --i) {
-            const long long k = kbase + i;
-            T d[VEC];
-            if (k < klim && W * j + i < L) {
-                const T *src = S.p + k * S.sk + x;
-                if (full) {
-                    vload(src, d);
+        for (int i = 0; i < N; i += VecT<T>::n) vload(p + i, d + i);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = i < n ? __ldg(p + i) : T(0);
+    }
+}
+
+template <typename T>
+__device__ inline T quant(T v, T c, bool compand) {
+    if (!compand) return v;
+    if constexpr (sizeof(T) == 4) return rintf(__fmul_rn(v, c));
+    else return rint(__dmul_rn(v, c));
+}
+template <typename T>
+__device__ inline T fma_t(T a, T b, T c) {
+    if constexpr (sizeof(T) == 4) return __fmaf_rn(a, b, c);
+    else return __fma_rn(a, b, c);
+}
+template <typename T>
+__device__ inline T pow2_of(int e) {
+    if constexpr (sizeof(T) == 4) return scalbnf(1.0f, e);
+    else return scalbn(1.0, e);
+}
+
+// How one operand is packed in this launch
+template <typename T>
+struct Job {
+    const PackOperand<T> *o;
+    T *out;
+    long long ldo;
+    int L, P;                 // block length and packed numbers per block
+    T w;                      // Horner's weight
+    bool compand, vec, vec_out;
+    bool manual;
+    double gamma;             // of the plan, or the manual compander itself
+    long long row_end;        // rows (along k) that the product reads
+    // c of the block at (x, k): the fp64 quotient rounded to T (fp32: the fp32
+    // quotient has the same bits, since 53 >= 2 * 24 + 2)
+    __device__ inline T compander(long long x, long long k) const {
+        if (!compand) return T(1);
+        if (manual) return (T)gamma;
+        const double m = __ldg(&o->mx[x / L * o->cx + k / L * o->cl]);
+        if constexpr (sizeof(T) == 4)
+            return m > 0.0 ? __fdiv_rn((float)gamma, (float)m) : 0.0f;
+        else
+            return m > 0.0 ? __ddiv_rn(gamma, m) : 0.0;
+    }
+};
+
+// packed numbers per thread along the contiguous dimension: whole vectors
+template <typename T, int W>
+constexpr int group_of() {
+    constexpr int V = VecT<T>::n;
+    return W % V == 0 ? 1 : (2 * W) % V == 0 ? 2 : 4;
+}
+// packed numbers a tile spans
+template <typename T, int W>
+constexpr int jspan() { return W == 3 ? 44 : KSPAN / W; }
+
+template <typename T, int W, int G>
+__device__ inline void horner(const T *d, T c, bool compand, T w, int n, T (&acc)[G]) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        acc[g] = W * g + W - 1 < n ? quant(d[W * g + W - 1], c, compand) : T(0);
+#pragma unroll
+        for (int i = W - 2; i >= 0; --i)
+            acc[g] = fma_t(w, acc[g], W * g + i < n ? quant(d[W * g + i], c, compand) : T(0));
+    }
+}
+
+// Packing direction contiguous in the input.  Tile: R rows of the other
+// dimension from r0, numbers [j0, j0 + jspan) of block b along the packed one.
+// ACROSS: numbers of a row lie across output rows (along k), staged in shared
+// memory; else along them (along x).
+template <typename T, int W, bool ACROSS>
+__device__ __forceinline__ void pack_contig(const Job<T> &jb, long long r0, long long rows,
+                                            long long ld, int b, int j0, long long len, T *s,
+                                            T *cs) {
+    constexpr int G = group_of<T, W>(), GV = G * W, JT = jspan<T, W>(), UPR = JT / G;
+    constexpr int R = ACROSS ? (sizeof(T) == 4 ? 64 : 32) : 32;
+    // units per thread, and per batch of loads issued before any is used
+    constexpr int NU = (R * UPR + NT - 1) / NT, UB = GV * sizeof(T) <= 16 ? 4 : 2;
+    constexpr int PITCH = JT + 1;
+    static_assert(JT % G == 0, "whole groups per tile");
+    const int L = jb.L, P = jb.P;
+    const long long v0 = (long long)b * L + (long long)W * j0;     // first value of the tile
+    const long long vlim = min((long long)(b + 1) * L, len);
+    __syncthreads();                      // the tile before is stored
+    if (threadIdx.x < R) {
+        const long long r = r0 + threadIdx.x;
+        cs[threadIdx.x] = r < rows ? (ACROSS ? jb.compander(r, (long long)b * L)
+                                             : jb.compander((long long)b * L, r))
+                                   : T(0);
+    }
+    __syncthreads();
+    for (int u0 = 0; u0 < NU; u0 += UB) {
+        T d[UB][GV];
+        int n[UB];
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int e = threadIdx.x + (u0 + u) * NT, r = e / UPR, q = e % UPR;
+            const long long v = v0 + (long long)GV * q;
+            const bool in = u0 + u < NU && r < R && r0 + r < rows && v < vlim;
+            n[u] = in ? (int)min((long long)GV, vlim - v) : 0;
+            load_run<T, GV>(jb.o->src + (r0 + r) * ld + v, n[u], jb.vec, d[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int e = threadIdx.x + (u0 + u) * NT, r = e / UPR, q = e % UPR;
+            if (u0 + u >= NU || r >= R) break;
+            T acc[G];
+            horner<T, W, G>(d[u], cs[r], jb.compand, jb.w, n[u], acc);
+            if constexpr (ACROSS) {
+#pragma unroll
+                for (int g = 0; g < G; ++g) s[r * PITCH + g * UPR + q] = acc[g];
+            } else {
+                // numbers G q .. of row r0 + r: out[k][b P + j]
+                T *dst = jb.out + (r0 + r) * jb.ldo + (long long)b * P + j0 + G * q;
+                if (r0 + r < rows) {
+#pragma unroll
+                    for (int g = 0; g < G; ++g)
+                        if (j0 + G * q + g < P) dst[g] = acc[g];
+                }
+            }
+        }
+    }
+    if constexpr (ACROSS) {
+        __syncthreads();
+        // out[b P + j][r]: lanes along r
+#pragma unroll 4
+        for (int e = threadIdx.x; e < JT * R; e += NT) {
+            const int j = e / R, r = e % R;
+            const long long row = (long long)b * P + j0 + j;
+            if (j0 + j >= P || r0 + r >= rows || row >= jb.row_end) continue;
+            jb.out[row * jb.ldo + r0 + r] = s[r * PITCH + j % G * UPR + j / G];
+        }
+    }
+}
+
+// Packing direction across the input's rows: a thread takes VEC contiguous
+// columns from W rows.  Tile: 32 VEC columns from c0, numbers [j0, j0 + JT).
+// ACROSS: out[k][b P + j] with the columns k (along x), staged; else out[b P +
+// j][x] with the columns x (along k).
+template <typename T, int W, bool ACROSS>
+__device__ __forceinline__ void pack_rows(const Job<T> &jb, long long c0, long long cols,
+                                          long long ld, int b, int j0, long long len, T *s,
+                                          T *cs) {
+    constexpr int V = VecT<T>::n, CT = 32 * V, JT = ACROSS ? 32 : jspan<T, W>();
+    constexpr int JW = (JT + 7) / 8;                 // numbers per warp
+    constexpr int UB = W == 1 ? 8 : W == 2 ? 4 : 2;
+    constexpr int PITCH = 33;
+    const int L = jb.L, P = jb.P, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __syncthreads();
+    if (threadIdx.x < CT / 16) {                     // blocks are multiples of 16 long
+        const long long c = c0 + 16 * threadIdx.x;
+        cs[threadIdx.x] = c < cols ? (ACROSS ? jb.compander((long long)b * L, c)
+                                             : jb.compander(c, (long long)b * L))
+                                   : T(0);
+    }
+    __syncthreads();
+    const T c = cs[V * lane / 16];
+    const long long col = c0 + V * lane;
+    const int left = (int)max(0LL, min((long long)V, cols - col));
+    const long long vbase = (long long)b * L, vlim = min(vbase + L, len);
+    for (int u0 = 0; u0 < JW; u0 += UB) {
+        T d[UB][W][V];
+#pragma unroll
+        for (int u = 0; u < UB; ++u)
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                const int j = j0 + warp + 8 * (u0 + u);
+                const long long v = vbase + (long long)W * j + i;
+                const bool in = u0 + u < JW && j < P && v < vlim;
+                load_run<T, V>(jb.o->src + v * ld + col, in ? left : 0, jb.vec, d[u][i]);
+            }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int jt = warp + 8 * (u0 + u), j = j0 + jt;
+            if (u0 + u >= JW || jt >= JT || j >= P) break;
+            T acc[V];
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                // (a digit outside is zero, also where c is not finite)
+                const long long v = vbase + (long long)W * j;
+                acc[e] = v + W - 1 < vlim ? quant(d[u][W - 1][e], c, jb.compand) : T(0);
+#pragma unroll
+                for (int i = W - 2; i >= 0; --i)
+                    acc[e] = fma_t(jb.w, acc[e],
+                                   v + i < vlim ? quant(d[u][i][e], c, jb.compand) : T(0));
+            }
+            if constexpr (ACROSS) {
+#pragma unroll
+                for (int e = 0; e < V; ++e) s[(e * 32 + lane) * PITCH + jt] = acc[e];
+            } else {
+                const long long row = (long long)b * P + j;
+                if (row >= jb.row_end) break;
+                T *dst = jb.out + row * jb.ldo + col;
+                if (jb.vec_out && left == V) {
+                    vstore(dst, acc);
                 } else {
 #pragma unroll
-                    for (int e = 0; e < VEC; ++e) d[e] = (x + e < S.X) ? src[e] : T(0);
+                    for (int e = 0; e < V; ++e)
+                        if (e < left) dst[e] = acc[e];
                 }
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) d[e] = quant(d[e], c, compand);
-            } else {
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) d[e] = T(0);
             }
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) acc[e] = (i == W - 1) ? d[e] : fma_t(w, acc[e], d[e]);
-        }
-        T *dst = out + row * ldo + x;
-        if (full) {
-            vstore(dst, acc);
-        } else {
-#pragma unroll
-            for (int e = 0; e < VEC; ++e)
-                if (x + e < S.X) dst[e] = acc[e];
         }
     }
-}
-
-template <typename T, int W>
-__global__ void __launch_bounds__(256) pack_k_xc_kernel(Src<T> S, int P, const DevPlan *plan,
-                                                        int expectW, int wsign, T *out,
-                                                        long long ldo, long long rows_out,
-                                                        int vec_ok) {
-    pdl_entry();
-    if (expectW > 0 && plan->W != expectW) return;
-    const T w = W > 1 ? pack_weight<T>(plan, wsign) : T(1);
-    pack_k_xc_body<T, W>(S, P, w, out, ldo, rows_out, vec_ok, blockIdx.x, gridDim.x);
-}
-
-// ------------------------------------------------------------------ pack along k,
-// k contiguous in the input: x-rows per tile of pack_k_kc_kernel (shared by
-// the kernel and its launch), each tile TILE packed columns wide
-template <typename T, int W>
-constexpr int kc_tile() { return (sizeof(T) == 4 && W <= 2) ? 64 : 32; }
-
-template <typename T, int W>
-__device__ __forceinline__ void pack_k_kc_body(const Src<T> &S, int P, T w, T *out, long long ldo,
-                                               long long rows_out, int vec_ok, long long vb,
-                                               long long vg) {
-    constexpr int VEC = VecT<T>::n;
-    // fp32 with W <= 2: 64 x-rows per tile (a 33 KB tile, four times the
-    // work per pass of the loop's fixed costs); else 32
-    constexpr int TILE = kc_tile<T, W>();
-    constexpr int NK = TILE * W;            // k values per tile row
-    constexpr int PITCH = NK + 1;
-    __shared__ T s[TILE * PITCH];
-    __shared__ T crow[TILE];
-    const bool compand = S.c != nullptr;
-    const int L = S.L;
-    const int jt = (P + TILE - 1) / TILE;
-    const long long xt = (S.X + TILE - 1) / TILE;
-    const int nK = (int)((S.K + L - 1) / L);
-    const long long tiles = xt * nK * jt;
-    for (long long t = vb; t < tiles; t += vg) {
-        const long long xtile = t % xt;
-        const long long r = t / xt;
-        const int l = (int)(r / jt), j0 = (int)(r % jt) * TILE;
-        const long long x0 = xtile * TILE;
-        const long long kslab = (long long)l * L;
-        const long long k0 = kslab + (long long)W * j0;
-        const long long klim = min(kslab + L, S.K);
-        __syncthreads();   // previous tile's readers are done with s / crow
-        if (threadIdx.x < TILE) {
-            const long long x = x0 + threadIdx.x;
-            crow[threadIdx.x] = (compand && x < S.X) ? S.c[(x / L) * S.cx + (long long)l * S.cl] : T(1);
-        }
+    if constexpr (ACROSS) {
         __syncthreads();
-        constexpr int CH = NK / VEC;
-        for (int e = threadIdx.x; e < TILE * CH; e += blockDim.x) {
-            const int xr = e / CH, kc = (e % CH) * VEC;
-            const long long x = x0 + xr, k = k0 + kc;
-            T d[VEC];
-            if (x < S.X && vec_ok && k + VEC <= klim) {
-                vload(S.p + x * S.sx + k, d);
-            } else {
-#pragma unroll
-                for (int q = 0; q < VEC; ++q)
-                    d[q] = (x < S.X && k + q < klim) ? S.p[x * S.sx + k + q] : T(0);
-            }
-            const T c = crow[xr];
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                const bool valid = x < S.X && k + q < klim;
-                s[xr * PITCH + kc + q] = valid ? quant(d[q], c, compand) : T(0);
-            }
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < TILE * TILE; e += blockDim.x) {
-            const int jr = e / TILE, xr = e % TILE;
-            const int j = j0 + jr;
-            const long long x = x0 + xr;
-            const long long row = (long long)l * P + j;
-            if (j >= P || x >= S.X || row >= rows_out) continue;
-            const T *d = s + xr * PITCH + jr * W;
-            T acc = d[W - 1];
-#pragma unroll
-            for (int i = W - 2; i >= 0; --i) acc = fma_t(w, acc, d[i]);
-            out[row * ldo + x] = acc;
+#pragma unroll 4
+        for (int e = threadIdx.x; e < CT * JT; e += NT) {
+            const int k = e / JT, j = e % JT;
+            if (j0 + j >= P || c0 + k >= cols) continue;
+            jb.out[(c0 + k) * jb.ldo + (long long)b * P + j0 + j] =
+                s[(k % V * 32 + k / V) * PITCH + j];
         }
     }
 }
 
-template <typename T, int W>
-__global__ void __launch_bounds__(256) pack_k_kc_kernel(Src<T> S, int P, const DevPlan *plan,
-                                                        int expectW, int wsign, T *out,
-                                                        long long ldo, long long rows_out,
-                                                        int vec_ok) {
-    pdl_entry();
-    if (expectW > 0 && plan->W != expectW) return;
-    const T w = W > 1 ? pack_weight<T>(plan, wsign) : T(1);
-    pack_k_kc_body<T, W>(S, P, w, out, ldo, rows_out, vec_ok, blockIdx.x, gridDim.x);
-}
-
-// Both operands of the symmetric form in one launch, A k-contiguous (eq. 6)
-// and B x-contiguous (eq. 7), the layouts of C = A B with row-major A and B:
-// the first 2 m CTAs alternate between the two (m = the smaller CTA count),
-// the rest go to the operand with more, so every SM runs both kinds at once
-// (the A pack is issue-bound, the B pack latency-bound).
-template <typename T, int W>
-__global__ void __launch_bounds__(256) pack_k_pair_kernel(Src<T> SA, Src<T> SB, int P,
-                                                          const DevPlan *plan, int expectW,
-                                                          T *outA, long long ldoA,
-                                                          long long rowsA, int vecA, T *outB,
-                                                          long long ldoB, long long rowsB,
-                                                          int vecB, long long gA, long long gB) {
-    pdl_entry();
-    if (expectW > 0 && plan->W != expectW) return;
-    const long long b = blockIdx.x, m = min(gA, gB);
-    bool isA;
-    long long vb;
-    if (b < 2 * m) {
-        isA = (b & 1) != 0;
-        vb = b >> 1;
-    } else {
-        isA = gA > gB;
-        vb = m + (b - 2 * m);
-    }
-    if (isA) {
-        const T w = W > 1 ? pack_weight<T>(plan, -1) : T(1);
-        pack_k_kc_body<T, W>(SA, P, w, outA, ldoA, rowsA, vecA, vb, gA);
-    } else {
-        const T w = W > 1 ? pack_weight<T>(plan, +1) : T(1);
-        pack_k_xc_body<T, W>(SB, P, w, outB, ldoB, rowsB, vecB, vb, gB);
-    }
-}
-
-// ------------------------------------------------------------------ plain k-major copy
-// out[k][x] = in[x][k] of a k-contiguous operand without companding (the
-// plain product's operands): 64 x 64 tiles through shared memory (s[x][k],
-// pitch 65), 16-byte loads along k issued before any is used, 16-byte stores
-// along x.  256 threads per CTA.
+// Tiles of one operand: t = (other-dimension tile) + count * (block chunk)
 template <typename T>
-__global__ void __launch_bounds__(256) transpose_copy_kernel(Src<T> S, const DevPlan *plan,
-                                                             int expectW, T *out, long long ldo,
-                                                             int vec_ok) {
-    pdl_entry();
-    if (expectW > 0 && plan->W != expectW) return;
-    constexpr int VEC = VecT<T>::n;
-    constexpr int TT = 64, PITCH = TT + 1;
-    constexpr int NV = TT * TT / VEC / 256;     // vectors per thread and phase
-    __shared__ T s[TT * PITCH];
-    const long long xt = (S.X + TT - 1) / TT, kt = (S.K + TT - 1) / TT;
-    for (long long t = blockIdx.x; t < xt * kt; t += gridDim.x) {
-        const long long x0 = (t % xt) * TT, k0 = (t / xt) * TT;
-        T v[NV][VEC];
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            const int e = threadIdx.x + u * 256;
-            const int xr = e / (TT / VEC), kc = (e % (TT / VEC)) * VEC;
-            const long long x = x0 + xr, k = k0 + kc;
-            if (x < S.X && vec_ok && k + VEC <= S.K) {
-                vload(S.p + x * S.sx + k, v[u]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < VEC; ++q)
-                    v[u][q] = (x < S.X && k + q < S.K) ? S.p[x * S.sx + k + q] : T(0);
-            }
-        }
-        __syncthreads();   // the previous tile's readers are done with s
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            const int e = threadIdx.x + u * 256;
-            const int xr = e / (TT / VEC), kc = (e % (TT / VEC)) * VEC;
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) s[xr * PITCH + kc + q] = v[u][q];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            const int e = threadIdx.x + u * 256;
-            const int kr = e / (TT / VEC), xc = (e % (TT / VEC)) * VEC;
-            const long long k = k0 + kr, x = x0 + xc;
-            if (k >= S.K || x >= S.X) continue;
-            T w[VEC];
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) w[q] = s[(xc + q) * PITCH + kr];
-            T *dst = out + k * ldo + x;
-            if (vec_ok && x + VEC <= S.X) {
-                vstore(dst, w);
-            } else {
-#pragma unroll
-                for (int q = 0; q < VEC; ++q)
-                    if (x + q < S.X) dst[q] = w[q];
-            }
-        }
-    }
-}
-
-// ------------------------------------------------------------------ pack along x
-// out[k][i*P + j] for j in [j0, j0 + 32) of row block i, k in [k0, k0 + 32)
+struct TileGrid {
+    unsigned int other, chunks, nblk;      // other-dimension tiles, chunks per block, blocks
+    int jt, span;                          // numbers and other-dimension values per tile
+    __device__ inline unsigned int tiles() const { return other * chunks * nblk; }
+};
 template <typename T, int W>
-__global__ void __launch_bounds__(256) pack_x_kernel(Src<T> S, int P, const DevPlan *plan,
-                                                     int expectW, int wsign, T *out,
-                                                     long long ldo) {
-    pdl_entry();
-    if (expectW > 0 && plan->W != expectW) return;
-    constexpr int NX = TILE * W;
-    constexpr int PITCH = TILE + 1;
-    __shared__ T s[NX * PITCH];
-    __shared__ T ccol[TILE];
-    const T w = W > 1 ? pack_weight<T>(plan, wsign) : T(1);
-    const bool compand = S.c != nullptr;
-    const int L = S.L;
-    const int jt = (P + TILE - 1) / TILE;
-    const int nM = (int)((S.X + L - 1) / L);
-    const long long kt = (S.K + TILE - 1) / TILE;
-    const long long tiles = (long long)nM * jt * kt;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const long long ktile = t % kt;
-        const long long r = t / kt;
-        const int i = (int)(r / jt), j0 = (int)(r % jt) * TILE;
-        const long long k0 = ktile * TILE;
-        const long long xblk0 = (long long)i * L;
-        const long long xlim = min(xblk0 + L, S.X);
-        const long long x0 = xblk0 + (long long)W * j0;
-        __syncthreads();
-        if (threadIdx.x < TILE) {
-            const long long k = k0 + threadIdx.x;
-            ccol[threadIdx.x] = (compand && k < S.K) ? S.c[(long long)i * S.cx + (k / L) * S.cl] : T(1);
-        }
-        __syncthreads();
-        if (S.sk == 1) {
-            for (int e = threadIdx.x; e < NX * TILE; e += blockDim.x) {
-                const int xr = e / TILE, kc = e % TILE;
-                const long long x = x0 + xr, k = k0 + kc;
-                const bool valid = x < xlim && k < S.K;
-                s[xr * PITCH + kc] = valid ? quant(S.p[x * S.sx + k], ccol[kc], compand) : T(0);
-            }
-        } else {
-            for (int e = threadIdx.x; e < NX * TILE; e += blockDim.x) {
-                const int kc = e / NX, xr = e % NX;
-                const long long x = x0 + xr, k = k0 + kc;
-                const bool valid = x < xlim && k < S.K;
-                s[xr * PITCH + kc] = valid ? quant(S.p[x + k * S.sk], ccol[kc], compand) : T(0);
-            }
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < TILE * TILE; e += blockDim.x) {
-            const int kr = e / TILE, jr = e % TILE;
-            const int j = j0 + jr;
-            const long long k = k0 + kr;
-            if (j >= P || k >= S.K) continue;
-            const T *d = s + (jr * W) * PITCH + kr;
-            T acc = d[(W - 1) * PITCH];
-#pragma unroll
-            for (int ii = W - 2; ii >= 0; --ii) acc = fma_t(w, acc, d[ii * PITCH]);
-            out[k * ldo + (long long)i * P + j] = acc;
-        }
-    }
+__device__ inline TileGrid<T> tile_grid(const PackOperand<T> &o, bool along_k, int L, int P) {
+    const bool contig = along_k ? o.sk == 1 && o.sx != 1 : o.sx == 1;
+    const bool across = along_k == contig;
+    TileGrid<T> g;
+    const long long oth = along_k ? o.X : o.K, len = along_k ? o.K : o.X;
+    g.span = contig ? (across ? (sizeof(T) == 4 ? 64 : 32) : 32) : 32 * VecT<T>::n;
+    g.jt = !contig && across ? 32 : jspan<T, W>();
+    g.other = (unsigned int)((oth + g.span - 1) / g.span);
+    g.chunks = (unsigned int)((P + g.jt - 1) / g.jt);
+    g.nblk = (unsigned int)((len + L - 1) / L);
+    return g;
 }
 
-template <typename T>
-Src<T> make_src(const PackOperand<T> &o) {
-    Src<T> S;
-    S.p = o.src; S.sx = o.sx; S.sk = o.sk; S.X = o.X; S.K = o.K;
-    S.c = o.c; S.cx = o.cx; S.cl = o.cl; S.L = o.L;
-    return S;
-}
-
-int capped(long long n) { return (int)max(1LL, min(n, (long long)MAX_CTAS)); }
-
-// Grid of at most `waves` full waves of resident CTAs for `kern` (occupancy
-// x SMs, cached per device and kernel under a lock, since host threads may
-// launch concurrently), so a grid-stride kernel never ends on a partial wave
-// of long-running CTAs and an early exit costs few CTAs.
-int resident_grid(const void *kern, long long n, int waves) {
-    struct Entry { const void *k; int dev, ctas; };
-    static Entry cache[128];
-    static int ncache = 0;
-    static std::mutex mu;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int ctas = 0;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        for (int i = 0; i < ncache; ++i)
-            if (cache[i].k == kern && cache[i].dev == dev) ctas = cache[i].ctas;
-    }
-    if (!ctas) {
-        int sms = 0, per = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 256, 0) != cudaSuccess || per < 1)
-            per = 1;
-        ctas = per * sms;
-        std::lock_guard<std::mutex> lock(mu);
-        if (ncache < 128) cache[ncache++] = {kern, dev, ctas};
-    }
-    return (int)max(1LL, min(n, (long long)ctas * waves));
-}
-
-template <typename T, int W>
-cudaError_t launch_pack_k_w(const PackOperand<T> &o, const DevPlan *plan, int expectW, int wsign,
-                            T *out, long long ldo, long long rows_out, cudaStream_t st) {
-    constexpr int VEC = VecT<T>::n;
-    Src<T> S = make_src(o);
-    const int P = (o.L + W - 1) / W;
-    const bool aligned_in = ((uintptr_t)o.src % 16 == 0);
-    const bool aligned_out = ((uintptr_t)out % 16 == 0) && (ldo % VEC == 0);
-    if (o.sx == 1) {
-        const int vec_ok = aligned_in && aligned_out && (o.sk % VEC == 0);
-        const long long items = rows_out * ((o.X + VEC - 1) / VEC);
-        return launch_pdl(pack_k_xc_kernel<T, W>,
-                          dim3(resident_grid((const void *)pack_k_xc_kernel<T, W>,
-                                             (items + 255) / 256, 4)),
-                          dim3(256), 0, st, S, P, plan, expectW, wsign, out, ldo, rows_out,
-                          vec_ok);
-    } else if (W == 1 && o.c == nullptr && o.sk == 1 && rows_out == o.K) {
-        // plain copy: a straight transpose
-        const int vec_ok = aligned_in && aligned_out && (o.sx % VEC == 0);
-        const long long tiles = ((o.X + 63) / 64) * ((o.K + 63) / 64);
-        return launch_pdl(transpose_copy_kernel<T>, dim3(capped(tiles)), dim3(256), 0, st, S, plan,
-                          expectW, out, ldo, vec_ok);
+template <typename T, int W, bool ALONG_K>
+__device__ __forceinline__ void pack_tile(const Job<T> &jb, const TileGrid<T> &g, unsigned int t,
+                                          T *s, T *cs) {
+    const PackOperand<T> &o = *jb.o;
+    const unsigned int r = t / g.other, b = r / g.chunks;
+    const long long base = (long long)(t - r * g.other) * g.span;
+    const int j0 = (int)(r - b * g.chunks) * g.jt;
+    // contiguous dimension: k when sk = 1 (and x is not), else x
+    if constexpr (ALONG_K) {
+        if (o.sk == 1 && o.sx != 1) pack_contig<T, W, true>(jb, base, o.X, o.sx, (int)b, j0, o.K, s, cs);
+        else pack_rows<T, W, false>(jb, base, o.X, o.sk, (int)b, j0, o.K, s, cs);
     } else {
-        const int vec_ok = aligned_in && (o.sx % VEC == 0) && o.sk == 1;
-        constexpr int TK = kc_tile<T, W>();
-        const long long tiles = ((o.X + TK - 1) / TK) * ((o.K + o.L - 1) / o.L) *
-                                ((P + TK - 1) / TK);
-        return launch_pdl(pack_k_kc_kernel<T, W>,
-                          dim3(resident_grid((const void *)pack_k_kc_kernel<T, W>, tiles, 4)),
-                          dim3(256), 0, st, S, P, plan, expectW, wsign, out, ldo, rows_out,
-                          vec_ok);
+        if (o.sx == 1) pack_contig<T, W, false>(jb, base, o.K, o.sk, (int)b, j0, o.X, s, cs);
+        else pack_rows<T, W, true>(jb, base, o.K, o.sx, (int)b, j0, o.X, s, cs);
     }
-    return cudaGetLastError();
 }
 
-template <typename T, int W>
-cudaError_t launch_pack_x_w(const PackOperand<T> &o, const DevPlan *plan, int expectW, int wsign,
-                            T *out, long long ldo, cudaStream_t st) {
-    Src<T> S = make_src(o);
-    const int P = (o.L + W - 1) / W;
-    const long long tiles = ((o.X + o.L - 1) / o.L) * ((P + TILE - 1) / TILE) *
-                            ((o.K + TILE - 1) / TILE);
-    return launch_pdl(pack_x_kernel<T, W>, dim3(capped(tiles)), dim3(256), 0, st, S, P, plan,
-                      expectW, wsign, out, ldo);
-    return cudaGetLastError();
+// the de-companding factors (T)(s_A,il s_B,lj), s = 1/c in fp64, of one slab and
+// a PAIR_TILE x PAIR_TILE tile of block pairs
+template <typename T>
+__device__ __forceinline__ void pair_tile(const PackArgs<T> &a, const DevPlan *plan, unsigned int t,
+                                          double *s) {
+    const unsigned int tn = (unsigned int)((a.nN + PAIR_TILE - 1) / PAIR_TILE);
+    const unsigned int tm = (unsigned int)((a.nM + PAIR_TILE - 1) / PAIR_TILE);
+    const unsigned int l = t / (tm * tn), r = t % (tm * tn);
+    const int i0 = (int)(r / tn) * PAIR_TILE, j0 = (int)(r % tn) * PAIR_TILE;
+    if (threadIdx.x < 2 * PAIR_TILE) {
+        const bool isA = threadIdx.x < PAIR_TILE;
+        const int e = isA ? i0 + threadIdx.x : j0 + threadIdx.x - PAIR_TILE;
+        double v = 0.0;
+        if (e < (isA ? a.nM : a.nN)) {
+            const PackOperand<T> &o = isA ? a.A : a.B;
+            double c;
+            if (a.manual) {
+                c = isA ? a.manual_cA : a.manual_cB;
+            } else {
+                const double m = __ldg(&o.mx[e * o.cx + l * o.cl]);
+                c = m > 0.0 ? __ddiv_rn((double)(isA ? plan->gA : plan->gB), m) : 0.0;
+            }
+            v = c > 0.0 ? __ddiv_rn(1.0, c) : 0.0;
+        }
+        s[threadIdx.x] = v;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < PAIR_TILE * PAIR_TILE; e += NT) {
+        const int i = e / PAIR_TILE, j = e % PAIR_TILE;
+        if (i0 + i < a.nM && j0 + j < a.nN)
+            a.pair[((long long)l * a.nM + i0 + i) * a.nN + j0 + j] =
+                (T)__dmul_rn(s[i], s[PAIR_TILE + j]);
+    }
+    __syncthreads();
+}
+
+// The CTAs take the factor tiles first, then tiles of A and B in turn (A's
+// transposing pack is bound by issue, B's by latency, in the row-major case),
+// last tiles first: the statistics read op(A) and then op(B) front to back, so
+// the ends are in L2.
+template <typename T, int WA, int WB, bool A_ALONG_K>
+__device__ __forceinline__ void pack_both(const PackArgs<T> &a, const DevPlan *plan, bool compand,
+                                          T *s, T *cs) {
+    const int q = plan->q;
+    auto job = [&](const PackOperand<T> &o, T *out, long long ldo, int W, bool isA) {
+        Job<T> j;
+        j.o = &o;
+        j.out = out;
+        j.ldo = ldo;
+        j.L = compand ? a.L : KSPAN;         // plain copies: any block length will do
+        j.P = (j.L + W - 1) / W;
+        j.w = W > 1 ? pow2_of<T>(isA ? -q : q) : T(1);
+        j.compand = compand;
+        j.manual = a.manual != 0;
+        // unpacked rows end with k; packed slabs are read to their last number
+        j.row_end = A_ALONG_K && compand ? LLONG_MAX : o.K;
+        j.gamma = a.manual ? (isA ? a.manual_cA : a.manual_cB) : (double)(isA ? plan->gA : plan->gB);
+        constexpr int V = VecT<T>::n;
+        j.vec = (reinterpret_cast<uintptr_t>(o.src) & 15) == 0 && (o.sk == 1 ? o.sx : o.sk) % V == 0;
+        j.vec_out = (reinterpret_cast<uintptr_t>(out) & 15) == 0 && ldo % V == 0;
+        return j;
+    };
+    const Job<T> ja = job(a.A, a.outA, a.ldoA[compand ? WA : 0], WA, true);
+    const Job<T> jbb = job(a.B, a.outB, a.ldoB, WB, false);
+    TileGrid<T> ga = tile_grid<T, WA>(a.A, A_ALONG_K, ja.L, ja.P);
+    TileGrid<T> gb = tile_grid<T, WB>(a.B, true, jbb.L, jbb.P);
+    const bool skipA = a.skipA || (!compand && a.directA), skipB = a.skipB || (!compand && a.directB);
+    const unsigned int nA = skipA ? 0u : ga.tiles(), nB = skipB ? 0u : gb.tiles();
+    const unsigned int np = compand ? (unsigned int)a.pair_tiles : 0u, both = 2 * min(nA, nB);
+    for (unsigned int t = blockIdx.x; t < np + nA + nB; t += gridDim.x) {
+        if (t < np) {
+            pair_tile(a, plan, t, reinterpret_cast<double *>(s));
+            continue;
+        }
+        const unsigned int v = t - np;
+        const bool isA = v < both ? (v & 1) != 0 : nA > nB;
+        const unsigned int w = v < both ? v >> 1 : v - both / 2;
+        if (isA) pack_tile<T, WA, A_ALONG_K>(ja, ga, nA - 1 - w, s, cs);
+        else pack_tile<T, WB, true>(jbb, gb, nB - 1 - w, s, cs);
+    }
+}
+
+template <typename T, bool ASYM>
+__global__ void __launch_bounds__(NT, 4) pack_kernel(const __grid_constant__ PackArgs<T> a,
+                                                     const DevPlan *plan) {
+    pdl_entry();
+    // staging: the largest tile is 64 (fp32) or 32 (fp64) rows of KSPAN numbers
+    __shared__ __align__(16) unsigned char raw[(sizeof(T) == 4 ? 64 : 32) * (KSPAN + 1) * sizeof(T)];
+    __shared__ T cs[64];
+    T *s = reinterpret_cast<T *>(raw);
+    const int W = a.plain ? 1 : plan->W;
+    // W = 1 from the planner of a distortion target is the conventional product
+    if (a.plain || (W == 1 && a.target)) {
+        pack_both<T, 1, 1, true>(a, plan, false, s, cs);
+        return;
+    }
+    if (a.plain_only) return;         // (pair-exact tiles are packed by the product itself)
+    if constexpr (ASYM) {
+        switch (W) {
+            case 1: pack_both<T, 1, 1, false>(a, plan, true, s, cs); break;
+            case 2: pack_both<T, 2, 1, false>(a, plan, true, s, cs); break;
+            case 3: pack_both<T, 3, 1, false>(a, plan, true, s, cs); break;
+            case 4: pack_both<T, 4, 1, false>(a, plan, true, s, cs); break;
+        }
+    } else {
+        switch (W) {
+            case 1: pack_both<T, 1, 1, true>(a, plan, true, s, cs); break;
+            case 2: pack_both<T, 2, 2, true>(a, plan, true, s, cs); break;
+            case 3: pack_both<T, 3, 3, true>(a, plan, true, s, cs); break;
+            case 4: pack_both<T, 4, 4, true>(a, plan, true, s, cs); break;
+        }
+    }
 }
 
 }  // namespace
 
-// The symmetric form's two packs (A with wsign -1, B with +1): one launch of
-// pack_k_pair_kernel when A is k-contiguous and B x-contiguous, else B's pack
-// and then A's.
-template <typename T, int W>
-cudaError_t launch_pack_k_pair_w(const PackOperand<T> &a, const PackOperand<T> &b,
-                                 const DevPlan *plan, int expectW, T *outA, long long ldoA,
-                                 long long rowsA, T *outB, long long ldoB, long long rowsB,
-                                 cudaStream_t st) {
-    constexpr int VEC = VecT<T>::n;
-    const bool a_copy = W == 1 && a.c == nullptr && a.sk == 1 && rowsA == a.K;
-    if (a.sx == 1 || a_copy || b.sx != 1) {
-        cudaError_t e = launch_pack_k_w<T, W>(b, plan, expectW, +1, outB, ldoB, rowsB, st);
-        if (e != cudaSuccess) return e;
-        return launch_pack_k_w<T, W>(a, plan, expectW, -1, outA, ldoA, rowsA, st);
-    }
-    Src<T> SA = make_src(a), SB = make_src(b);
-    const int P = (a.L + W - 1) / W;
-    const int vecA = ((uintptr_t)a.src % 16 == 0) && (a.sx % VEC == 0) && a.sk == 1;
-    const int vecB = ((uintptr_t)b.src % 16 == 0) && ((uintptr_t)outB % 16 == 0) &&
-                     (ldoB % VEC == 0) && (b.sk % VEC == 0);
-    constexpr int TK = kc_tile<T, W>();
-    const long long tilesA = ((a.X + TK - 1) / TK) * ((a.K + a.L - 1) / a.L) * ((P + TK - 1) / TK);
-    const long long blocksB = (rowsB * ((b.X + VEC - 1) / VEC) + 255) / 256;
-    const void *kern = (const void *)pack_k_pair_kernel<T, W>;
-    const long long gA = resident_grid(kern, tilesA, 2);
-    const long long gB = resident_grid(kern, blocksB, 2);
-    return launch_pdl(pack_k_pair_kernel<T, W>, dim3((unsigned)(gA + gB)), dim3(256), 0, st, SA,
-                      SB, P, plan, expectW, outA, ldoA, rowsA, vecA, outB, ldoB, rowsB, vecB,
-                      gA, gB);
-}
-
 template <typename T>
-cudaError_t launch_pack_k_pair(const PackOperand<T> &a, const PackOperand<T> &b, int W,
-                               const DevPlan *plan, int expectW, T *outA, long long ldoA,
-                               long long rowsA, T *outB, long long ldoB, long long rowsB,
-                               cudaStream_t st) {
-    switch (W) {
-        case 1: return launch_pack_k_pair_w<T, 1>(a, b, plan, expectW, outA, ldoA, rowsA, outB, ldoB, rowsB, st);
-        case 2: return launch_pack_k_pair_w<T, 2>(a, b, plan, expectW, outA, ldoA, rowsA, outB, ldoB, rowsB, st);
-        case 3: return launch_pack_k_pair_w<T, 3>(a, b, plan, expectW, outA, ldoA, rowsA, outB, ldoB, rowsB, st);
-        case 4: return launch_pack_k_pair_w<T, 4>(a, b, plan, expectW, outA, ldoA, rowsA, outB, ldoB, rowsB, st);
-    }
-    return cudaErrorInvalidValue;
+cudaError_t launch_pack(bool asym, const PackArgs<T> &a0, const DevPlan *plan, cudaStream_t st) {
+    PackArgs<T> a = a0;
+    const long long tm = (a.nM + PAIR_TILE - 1) / PAIR_TILE, tn = (a.nN + PAIR_TILE - 1) / PAIR_TILE;
+    const long long np = a.pair ? tm * tn * a.nK : 0;
+    // an upper bound of the tiles over every packing (32 values by 16 numbers)
+    auto bound = [&](const PackOperand<T> &o) {
+        return ((o.X + 31) / 32) * ((o.K + std::min(a.L, KSPAN) - 1) / std::min(a.L, KSPAN) + 1) +
+               ((o.K + 31) / 32) * ((o.X + 31) / 32 + 1);
+    };
+    if (np > 0x3fffffffLL || bound(a.A) > 0x3fffffffLL || bound(a.B) > 0x3fffffffLL)
+        return cudaErrorInvalidConfiguration;
+    a.pair_tiles = (int)np;
+    // a resident wave (four CTAs fit an SM), or less for small operands
+    const long long want = np + (a.skipA ? 0 : bound(a.A)) + (a.skipB ? 0 : bound(a.B));
+    const unsigned int grid = (unsigned int)std::max(1LL, std::min(want, 4LL * device_sms()));
+    return asym ? launch_pdl(pack_kernel<T, true>, dim3(grid), dim3(NT), 0, st, a, plan)
+                : launch_pdl(pack_kernel<T, false>, dim3(grid), dim3(NT), 0, st, a, plan);
 }
 
-template <typename T>
-cudaError_t launch_pack_k(const PackOperand<T> &o, int W, const DevPlan *plan, int expectW,
-                          int wsign, T *out, long long ldo, long long rows_out, cudaStream_t st) {
-    switch (W) {
-        case 1: return launch_pack_k_w<T, 1>(o, plan, expectW, wsign, out, ldo, rows_out, st);
-        case 2: return launch_pack_k_w<T, 2>(o, plan, expectW, wsign, out, ldo, rows_out, st);
-        case 3: return launch_pack_k_w<T, 3>(o, plan, expectW, wsign, out, ldo, rows_out, st);
-        case 4: return launch_pack_k_w<T, 4>(o, plan, expectW, wsign, out, ldo, rows_out, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
-template <typename T>
-cudaError_t launch_pack_x(const PackOperand<T> &o, int W, const DevPlan *plan, int expectW,
-                          int wsign, T *out, long long ldo, cudaStream_t st) {
-    switch (W) {
-        case 1: return launch_pack_x_w<T, 1>(o, plan, expectW, wsign, out, ldo, st);
-        case 2: return launch_pack_x_w<T, 2>(o, plan, expectW, wsign, out, ldo, st);
-        case 3: return launch_pack_x_w<T, 3>(o, plan, expectW, wsign, out, ldo, st);
-        case 4: return launch_pack_x_w<T, 4>(o, plan, expectW, wsign, out, ldo, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
-template cudaError_t launch_pack_k_pair<float>(const PackOperand<float> &, const PackOperand<float> &,
-                                               int, const DevPlan *, int, float *, long long,
-                                               long long, float *, long long, long long,
-                                               cudaStream_t);
-template cudaError_t launch_pack_k_pair<double>(const PackOperand<double> &,
-                                                const PackOperand<double> &, int,
-                                                const DevPlan *, int, double *, long long,
-                                                long long, double *, long long, long long,
-                                                cudaStream_t);
-template cudaError_t launch_pack_k<float>(const PackOperand<float> &, int, const DevPlan *, int, int,
-                                          float *, long long, long long, cudaStream_t);
-template cudaError_t launch_pack_k<double>(const PackOperand<double> &, int, const DevPlan *, int,
-                                           int, double *, long long, long long, cudaStream_t);
-template cudaError_t launch_pack_x<float>(const PackOperand<float> &, int, const DevPlan *, int, int,
-                                          float *, long long, cudaStream_t);
-template cudaError_t launch_pack_x<double>(const PackOperand<double> &, int, const DevPlan *, int,
-                                           int, double *, long long, cudaStream_t);
+template cudaError_t launch_pack<float>(bool, const PackArgs<float> &, const DevPlan *, cudaStream_t);
+template cudaError_t launch_pack<double>(bool, const PackArgs<double> &, const DevPlan *,
+                                         cudaStream_t);
 
 }  // namespace tdg

@@ -1,16 +1,32 @@
-// Launchers of tdg_pack.cu beyond those every translation unit shares.
+// The pack launch: companding, packing and the de-companding factors of a call.
 #pragma once
 
 #include "tdg_internal.h"
 
 namespace tdg {
 
-// The symmetric form's A (eq. 6) and B (eq. 7) packs: one launch where the
-// layouts allow (A k-contiguous, B x-contiguous), else B's pack and then A's.
 template <typename T>
-cudaError_t launch_pack_k_pair(const PackOperand<T> &a, const PackOperand<T> &b, int W,
-                               const DevPlan *plan, int expectW, T *outA, long long ldoA,
-                               long long rowsA, T *outB, long long ldoB, long long rowsB,
-                               cudaStream_t st);
+struct PackArgs {
+    PackOperand<T> A, B;      // op(A)[m][k] and op(B)[k][n] as (x, k), with block maxima
+    T *outA, *outB;
+    // leading dimension of the packed A by W (the asymmetric form's differs),
+    // [0]: of its plain copy
+    long long ldoA[kMaxW + 1], ldoB;
+    T *pair;                  // nullable: [l][i][j] factors
+    int L, nM, nK, nN;
+    int target;               // the plan may have fallen back to the plain product
+    int plain;                // plain copies whatever the plan says
+    int plain_only;           // only the fallback's plain copies
+    int directA, directB;     // the plain product reads this operand in place
+    int skipA, skipB;         // operand kept from an earlier call
+    int manual;
+    double manual_cA, manual_cB;
+    int pair_tiles;           // set by the launcher
+};
+
+// One launch over both operands for whichever W the device plan holds (along k:
+// the symmetric form and plain copies; asym: A along x, B unpacked).
+template <typename T>
+cudaError_t launch_pack(bool asym, const PackArgs<T> &a, const DevPlan *plan, cudaStream_t st);
 
 }  // namespace tdg

@@ -12,8 +12,8 @@
 //   lower level) and keeps the first W whose SNR meets the target.  Otherwise
 //   W = 1 (plain product) with TDG_ALLOW_FALLBACK, else TDG_EUNREACHABLE.
 // * Manual mode: given q and uniform companders (the Sec. 4.B protocol).
-// Then a grid-wide kernel writes c (in T) and s = 1/c (fp64) per block and the
-// de-companding factors (T)(s_A,il s_B,lj) for every (l, i, j).
+// The companders c and the de-companding factors (T)(s_A,il s_B,lj) follow in the
+// pack launch.
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
 #include "tdg_planner.cuh"
@@ -85,45 +85,6 @@ __global__ void __launch_bounds__(32) planner_kernel(PlanParams pp, const double
                                                      DevPlan *plan) {
     pdl_entry();
     decide_plan(pp, stab, nullptr, plan, 0.0, 0.0, 0.0, 0.0, rho_of(0.0, 0.0));
-}
-
-// c = gamma / max|x| (fp64, rounded to T for eq. 3), s = 1/c, per block.
-template <typename T>
-__global__ void scales_kernel(PlanParams pp, const double *__restrict__ mA,
-                              const double *__restrict__ mB, const DevPlan *__restrict__ plan,
-                              T *cA, double *sA, T *cB, double *sB) {
-    pdl_entry();
-    const long long nAblk = (long long)pp.nM * pp.nK, nBblk = (long long)pp.nK * pp.nN;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const DevPlan a = *plan;
-    if (!needs_companders(pp, a)) return;  // plain product: nothing to compand
-    for (long long k = idx; k < nAblk + nBblk; k += (long long)gridDim.x * blockDim.x) {
-        const bool isA = k < nAblk;
-        const long long b = isA ? k : k - nAblk;
-        double m = isA ? mA[b] : mB[b];
-        double c;
-        if (pp.mode == MODE_MANUAL) c = isA ? pp.manual_cA : pp.manual_cB;
-        else c = m > 0.0 ? __ddiv_rn((double)(isA ? a.gA : a.gB), m) : 0.0;
-        double s = c > 0.0 ? __ddiv_rn(1.0, c) : 0.0;
-        if (isA) { cA[b] = (T)c; sA[b] = s; }
-        else { cB[b] = (T)c; sB[b] = s; }
-    }
-}
-
-// (T)(s_A,il * s_B,lj) for every (l, i, j), layout [l][i][j]
-template <typename T>
-__global__ void pairs_kernel(PlanParams pp, const double *__restrict__ sA,
-                             const double *__restrict__ sB, const DevPlan *__restrict__ plan,
-                             T *pair) {
-    pdl_entry();
-    if (!needs_companders(pp, *plan)) return;
-    const long long n = (long long)pp.nK * pp.nM * pp.nN;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        long long j = k % pp.nN, r = k / pp.nN;
-        long long i = r % pp.nM, l = r / pp.nM;
-        pair[k] = (T)__dmul_rn(sA[i * pp.nK + l], sB[l * pp.nN + j]);
-    }
 }
 
 // ---- Sec. 6: per inner kernel R_ij, predicted S_ij / N_ij with the call's
@@ -293,42 +254,20 @@ cudaError_t launch_kernel_control(const PlanParams &pp, const double *mA, const 
                       0, st, T, mode, thr, k, F, fw, plan, (const double *)ratio, mask);
 }
 
-template <typename T>
-cudaError_t launch_planner(const PlanParams &pp, const double *mA, const double *eA,
-                           const double *mB, const double *eB, const double *stab,
-                           DevPlan *plan, double *agg, T *cA, double *sA, T *cB, double *sB,
-                           T *pair, cudaStream_t st) {
-    // agg: 4 nK per-slab aggregates, then one record per candidate (W, level)
-    LevelRec *res = reinterpret_cast<LevelRec *>(agg + 4 * (long long)pp.nK);
-    cudaError_t e = cudaSuccess;
+cudaError_t launch_planner(const PlanParams &pp, const double *stab, DevPlan *plan, double *agg,
+                           cudaStream_t st) {
     if (pp.mode == MODE_TARGET && (pp.form == TDG_SYM || pp.form == TDG_ASYM)) {
         // every candidate level, the plan decided by the last CTA to finish
+        LevelRec *res = reinterpret_cast<LevelRec *>(agg + 4 * (long long)pp.nK);
         int t_lo = 0;
         while (r_level(t_lo) < pp.L) ++t_lo;
         const int nlev = (pp.p == 24 ? 4 * 24 : 4 * 40) - t_lo + 1;
         const int ctas = max(1, (pp.Wreq - 1) * ((nlev + 31) / 32));
-        e = launch_pdl(level_kernel, dim3(ctas), dim3(32), 0, st, pp, stab, res, plan);
-    } else if (pp.form == TDG_PLAIN || pp.mode == MODE_MANUAL) {
-        e = launch_pdl(planner_kernel, dim3(1), dim3(32), 0, st, pp, stab, plan);
-    }   // else decided by the statistics kernel
-    if (e != cudaSuccess) return e;
-    const long long nblk = (long long)pp.nM * pp.nK + (long long)pp.nK * pp.nN;
-    e = launch_pdl(scales_kernel<T>, dim3((unsigned)min((nblk + 255) / 256, 4096LL)), dim3(256), 0,
-                   st, pp, mA, mB, (const DevPlan *)plan, cA, sA, cB, sB);
-    if (e != cudaSuccess) return e;
-    long long np = (long long)pp.nK * pp.nM * pp.nN;
-    int g = (int)min((np + 255) / 256, 8192LL);
-    return launch_pdl(pairs_kernel<T>, dim3(g), dim3(256), 0, st, pp, (const double *)sA,
-                      (const double *)sB, (const DevPlan *)plan, pair);
+        return launch_pdl(level_kernel, dim3(ctas), dim3(32), 0, st, pp, stab, res, plan);
+    }
+    if (pp.form == TDG_PLAIN || pp.mode == MODE_MANUAL)
+        return launch_pdl(planner_kernel, dim3(1), dim3(32), 0, st, pp, stab, plan);
+    return cudaSuccess;      // decided by the statistics kernel
 }
-
-template cudaError_t launch_planner<float>(const PlanParams &, const double *, const double *,
-                                           const double *, const double *, const double *,
-                                           DevPlan *, double *, float *, double *, float *,
-                                           double *, float *, cudaStream_t);
-template cudaError_t launch_planner<double>(const PlanParams &, const double *, const double *,
-                                            const double *, const double *, const double *,
-                                            DevPlan *, double *, double *, double *, double *,
-                                            double *, double *, cudaStream_t);
 
 }  // namespace tdg

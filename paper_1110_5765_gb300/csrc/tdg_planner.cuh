@@ -9,15 +9,6 @@
 
 namespace tdg {
 
-// The plain product (form PLAIN, or the W = 1 fallback of target mode for the
-// packed forms) uses no companders.
-__device__ inline bool needs_companders(const PlanParams &pp, const DevPlan &a) {
-    if (pp.form == TDG_PLAIN) return false;
-    if ((pp.form == TDG_SYM || pp.form == TDG_ASYM) && pp.mode == MODE_TARGET && a.W == 1)
-        return false;
-    return true;
-}
-
 __device__ inline int t_max_for(int p) { return p == 24 ? 4 * 24 : 4 * 40; }
 
 

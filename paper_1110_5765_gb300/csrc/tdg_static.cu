@@ -37,6 +37,7 @@
 
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
+#include "tdg_pack.h"
 #include "tdg_planner.cuh"
 #include "tdgemm.h"
 
@@ -111,8 +112,6 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
         take(((size_t)4 * nK + (size_t)kLevelRecDoubles * (kMaxW - 1) * kMaxLevels) * 8);
     const size_t o_mA = take(nA_blk * 8), o_eA = take(nA_blk * 8);
     const size_t o_mB = take(nB_blk * 8), o_eB = take(nB_blk * 8);
-    const size_t o_sA = take(nA_blk * 8), o_sB = take(nB_blk * 8);
-    const size_t o_cA = take(nA_blk * sizeof(T)), o_cB = take(nB_blk * sizeof(T));
     const size_t o_pair = take((size_t)nK * nM * nN * sizeof(T));
     const size_t o_A = take((size_t)(a_rows * a_ld) * sizeof(T));
     const size_t o_B = take((size_t)(b_rows * b_ld) * sizeof(T));
@@ -128,8 +127,7 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     double *agg = (double *)(ws + o_agg);
     double *mA = (double *)(ws + o_mA), *eA = (double *)(ws + o_eA);
     double *mB = (double *)(ws + o_mB), *eB = (double *)(ws + o_eB);
-    double *sA = (double *)(ws + o_sA), *sB = (double *)(ws + o_sB);
-    T *cA = (T *)(ws + o_cA), *cB = (T *)(ws + o_cB), *pair = (T *)(ws + o_pair);
+    T *pair = (T *)(ws + o_pair);
     T *Abuf = (T *)(ws + o_A), *Bbuf = (T *)(ws + o_B);
 
     // the plan record and the slab counters start at zero (the array holds
@@ -146,19 +144,17 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     ST_TRY(launch_block_stats<T>(A, nA ? M : K, nA ? K : M, lda, nA ? 0 : 1, nK, mA, eA, B,
                                  nB ? K : N, nB ? N : K, ldb, nB ? 0 : 1, nN, mB, eB, L, dplan,
                                  fin, st));
-    ST_TRY(launch_planner<T>(pp, mA, eA, mB, eB, nullptr, dplan, agg, cA, sA, cB, sB, pair, st));
-    PackOperand<T> oa{}, ob{};
-    oa.src = A; oa.X = M; oa.K = K; oa.L = L; oa.c = cA; oa.cx = nK; oa.cl = 1;
-    if (nA) { oa.sx = lda; oa.sk = 1; } else { oa.sx = 1; oa.sk = lda; }
-    ob.src = B; ob.X = N; ob.K = K; ob.L = L; ob.c = cB; ob.cx = 1; ob.cl = nN;
-    if (nB) { ob.sx = 1; ob.sk = ldb; } else { ob.sx = ldb; ob.sk = 1; }
-    if (form == TDG_SYM) {
-        ST_TRY(launch_pack_k<T>(oa, W, dplan, W, -1, Abuf, a_ld, a_rows, st));
-        ST_TRY(launch_pack_k<T>(ob, W, dplan, W, +1, Bbuf, b_ld, b_rows, st));
-    } else {
-        ST_TRY(launch_pack_x<T>(oa, W, dplan, W, -1, Abuf, a_ld, st));
-        ST_TRY(launch_pack_k<T>(ob, 1, dplan, W, 0, Bbuf, b_ld, b_rows, st));
-    }
+    PackArgs<T> pa{};
+    pa.A.src = A; pa.A.X = M; pa.A.K = K; pa.A.L = L; pa.A.mx = mA; pa.A.cx = nK; pa.A.cl = 1;
+    if (nA) { pa.A.sx = lda; pa.A.sk = 1; } else { pa.A.sx = 1; pa.A.sk = lda; }
+    pa.B.src = B; pa.B.X = N; pa.B.K = K; pa.B.L = L; pa.B.mx = mB; pa.B.cx = 1; pa.B.cl = nN;
+    if (nB) { pa.B.sx = 1; pa.B.sk = ldb; } else { pa.B.sx = ldb; pa.B.sk = 1; }
+    pa.outA = Abuf; pa.outB = Bbuf;
+    for (long long &ld : pa.ldoA) ld = a_ld;
+    pa.ldoB = b_ld;
+    pa.pair = pair;
+    pa.L = L; pa.nM = nM; pa.nK = nK; pa.nN = nN;
+    ST_TRY(launch_pack<T>(form == TDG_ASYM, pa, dplan, st));
     const int gform = form == TDG_SYM ? G_SYM : G_ASYM;
     GemmOperands ops{};
     ops.a = {Abuf, a_cols, a_rows, a_ld};

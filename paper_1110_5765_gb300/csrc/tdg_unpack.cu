@@ -24,10 +24,13 @@ __device__ inline T rint_d(T v) {
     else return rint(v);
 }
 
+constexpr int BATCH = 8;            // slabs whose loads are in flight together
+
 template <typename T, int ASYM>
 __global__ void unpack_kernel(GemmArgs<T> g, int W, int64_t *rint_out) {
     pdl_entry();
-    if (g.plan->W != W) return;            // the planner chose another packing
+    // the planner chose another packing (W = 0: any packing was expected)
+    if (W ? g.plan->W != W : g.plan->W < 2) return;
     const long long total = g.M * g.N;
     const int q = g.plan->q;
     const T z = sizeof(T) == 4 ? (T)scalbnf(1.0f, -q) : (T)scalbn(1.0, -q);
@@ -46,41 +49,56 @@ __global__ void unpack_kernel(GemmArgs<T> g, int W, int64_t *rint_out) {
             xr = m;
         }
         T c = T(0);
-        for (int l = 0; l < g.nK; ++l) {
-            const T rbar = g.Rbar[((long long)l * g.Mrows + xr) * g.N + n];
-            T rt;
-            if constexpr (sizeof(T) == 8) {
-                // digits in integer arithmetic, as the fused epilogue takes them
-                if constexpr (ASYM) {
-                    double dg[kMaxW];
-                    asym_digits<kMaxW>(rbar, q, dg);
-                    rt = d == 0 ? dg[0] : d == 1 ? dg[1] : d == 2 ? dg[2] : dg[3];
-                } else {
-                    rt = sym_digit<false>(rbar, q);
-                }
-            } else if (ASYM) {
-                T x = rbar;
-                rt = rint_d(x);
-                for (int k = 0; k < d; ++k) {
-                    if constexpr (sizeof(T) == 4) x = __fmul_rn(Q, __fsub_rn(x, rt));
-                    else x = __dmul_rn(Q, __dsub_rn(x, rt));
-                    rt = rint_d(x);
-                }
-            } else {
-                const T u = rint_d(rbar);
-                T t;
-                if constexpr (sizeof(T) == 4) {
-                    t = rintf(__fmul_rn(z, u));
-                    rt = __fmaf_rn(-Q, t, u);
-                } else {
-                    t = rint(__dmul_rn(z, u));
-                    rt = __fma_rn(-Q, t, u);
-                }
+        const T *src = g.Rbar + xr * g.N + n;
+        const T *pair = g.pair + i * g.nN + jn;
+        const long long rs = g.Mrows * g.N, ps = (long long)g.nM * g.nN;
+        for (int l0 = 0; l0 < g.nK; l0 += BATCH) {
+            // the loads of BATCH slabs issued before any is used: the sum over
+            // slabs is one chain per output, and few outputs leave few warps
+            T rb[BATCH], pr[BATCH];
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) {
+                const int l = min(l0 + u, g.nK - 1);
+                rb[u] = __ldcs(src + l * rs);
+                pr[u] = __ldg(pair + l * ps);
             }
-            const T pr = g.pair[((long long)l * g.nM + i) * g.nN + jn];
-            if constexpr (sizeof(T) == 4) c = __fmaf_rn(rt, pr, c);
-            else c = __fma_rn(rt, pr, c);
-            if (rint_out) rint_out[e * g.nK + l] = (int64_t)rt;
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) {
+                if (l0 + u >= g.nK) break;
+                const T rbar = rb[u];
+                T rt;
+                if constexpr (sizeof(T) == 8) {
+                    // digits in integer arithmetic, as the fused epilogue takes them
+                    if constexpr (ASYM) {
+                        double dg[kMaxW];
+                        asym_digits<kMaxW>(rbar, q, dg);
+                        rt = d == 0 ? dg[0] : d == 1 ? dg[1] : d == 2 ? dg[2] : dg[3];
+                    } else {
+                        rt = sym_digit<false>(rbar, q);
+                    }
+                } else if (ASYM) {
+                    T x = rbar;
+                    rt = rint_d(x);
+                    for (int k = 0; k < d; ++k) {
+                        if constexpr (sizeof(T) == 4) x = __fmul_rn(Q, __fsub_rn(x, rt));
+                        else x = __dmul_rn(Q, __dsub_rn(x, rt));
+                        rt = rint_d(x);
+                    }
+                } else {
+                    const T u = rint_d(rbar);
+                    T t;
+                    if constexpr (sizeof(T) == 4) {
+                        t = rintf(__fmul_rn(z, u));
+                        rt = __fmaf_rn(-Q, t, u);
+                    } else {
+                        t = rint(__dmul_rn(z, u));
+                        rt = __fma_rn(-Q, t, u);
+                    }
+                }
+                if constexpr (sizeof(T) == 4) c = __fmaf_rn(rt, pr[u], c);
+                else c = __fma_rn(rt, pr[u], c);
+                if (rint_out) rint_out[e * g.nK + l0 + u] = (int64_t)rt;
+            }
         }
         if (g.C) {
             // the GEMM epilogue: C = alpha c (beta == 0) or alpha c + beta C

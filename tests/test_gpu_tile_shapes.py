@@ -31,3 +31,48 @@ def test_f64_tiles(orc, shape, form, W):
         p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C, 0.75, -1.5)
         assert p.info()["device_status"] == 0
         assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
+
+
+# fp32: one ragged 64-tile, 64-tiles, 128 x 64 tiles (r = 1, 2), 128 x 128 tiles,
+# slabs split over CTAs
+F32 = [(60, 50, 130), (700, 690, 130), (1000, 777, 130), (1500, 1300, 130), (2000, 1900, 66),
+       (129, 70, 1400)]
+
+
+@pytest.mark.parametrize("shape", F32)
+@pytest.mark.parametrize("form,W", [("sym", 1), ("sym", 2), ("sym", 3), ("asym", 2), ("asym", 4)])
+def test_f32_tiles(orc, shape, form, W):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1110_5765_gb300 as tdg
+    M, N, K = shape
+    A, B = synth.laplace((M, K), 64, np.float32), synth.gaussian((K, N), 65, np.float32)
+    C0 = synth.gaussian((M, N), 66, np.float32)
+    kw = dict(L=64, W=W, dtype="f32", form=form, bits=6)
+    ref = orc.tdgemm(A, B, alpha=0.75, beta=-1.5, C_in=C0, **kw)
+    with tdg.Plan(M, N, K, **kw) as p:
+        C = torch.from_numpy(C0.copy()).cuda()
+        p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C, 0.75, -1.5)
+        assert p.info()["device_status"] == 0
+        assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
+
+
+@pytest.mark.parametrize("shape", F32)
+@pytest.mark.parametrize("form,W,target,used", [("sym", 2, 20.0, 2), ("sym", 2, 60.0, 1),
+                                                ("sym", 4, 20.0, None), ("asym", 2, 20.0, 2),
+                                                ("asym", 2, 60.0, 1)])
+def test_f32_target_launches(orc, shape, form, W, target, used):
+    """Targets met by packing and missed (plain fallback), in the launches that hold
+    several candidates: the plan and C of the oracle."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1110_5765_gb300 as tdg
+    M, N, K = shape
+    A, B = synth.uniform((M, K), 67, np.float32), synth.uniform((K, N), 68, np.float32)
+    kw = dict(L=64, W=W, dtype="f32", form=form)
+    ref = orc.tdgemm(A, B, target_db=target, s_table=orc.load_s_table(), **kw)
+    assert used is None or ref.plan.W == used
+    with tdg.Plan(M, N, K, target_snr_db=target, **kw) as p:
+        C = p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda())
+        assert p.info()["W_used"] == ref.plan.W
+        assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
