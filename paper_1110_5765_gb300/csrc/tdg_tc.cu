@@ -31,7 +31,8 @@
 //               two TMEM accumulators, a fresh accumulation per slab, and
 //               commits to mbarriers in both CTAs that free ring stages and
 //               hand a full slab to the epilogue;
-//   warps 2..17 epilogue: each thread owns one output row and 64 columns;
+//   warps 2..17 epilogue: each thread owns one output row and 64 columns (32 of
+//               a half tile);
 //               per slab it reads its TMEM lane (tcgen05.ld), applies
 //               C_acc = fma(r, s_A s_B, C_acc) in fp32 and releases the
 //               accumulator to the even CTA's MMA issuer, so the
@@ -44,6 +45,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
@@ -85,24 +87,28 @@ __device__ inline uint64_t desc_sw128(uint32_t saddr) {
 }
 
 // instruction descriptor: D fp32, A/B fp16 (or E4M3 under kind::f8f6f4,
-// whose format code is also 0), both K-major, N = 256, M = 256 (the pair)
-constexpr uint32_t IDESC = (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                           ((uint32_t)((2 * BM) >> 4) << 24);
+// whose format code is also 0), both K-major, N = 256 (128 for a half tile),
+// M = 256 (the pair)
+constexpr uint32_t idesc(int n) {
+    return (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)((2 * BM) >> 4) << 24);
+}
 
 // the pair's MMA, issued by the even CTA: A rows 0..127 and B~ rows 0..127
 // from its shared memory, rows 128..255 of both from the peer's (same offsets)
 template <int FP8>
-__device__ inline void mma2(uint32_t dtmem, uint64_t ad, uint64_t bd, int accumulate) {
+__device__ inline void mma2(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t desc,
+                            int accumulate) {
     if constexpr (FP8) {
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
             "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(ad), "l"(bd), "r"(IDESC), "r"(accumulate));
+            "l"(ad), "l"(bd), "r"(desc), "r"(accumulate));
     } else {
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
             "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(ad), "l"(bd), "r"(IDESC), "r"(accumulate));
+            "l"(ad), "l"(bd), "r"(desc), "r"(accumulate));
     }
 }
 
@@ -207,11 +213,13 @@ __device__ inline bool tc_wait_epilogue(uint64_t *bar, uint32_t parity) {
 // The plain-store path of the epilogue (beta != 0, or C rows that cannot be
 // mapped for TMA): 32 rows x 16 columns of C_acc from the warp's staging tile
 // (16-byte unit u of row r at u ^ ((r >> 1) & 3)), each store instruction
-// writing 8 rows x 64 contiguous bytes.  Kept out of line: inlined, its
-// address arithmetic made the promotion loop spill registers.
-__device__ __noinline__ void store_staged_plain(const TcArgs &g, const unsigned char *stg, int lane,
+// writing 8 rows x 64 contiguous bytes.  Inlined and not unrolled: a call, even one
+// never taken, cost the whole kernel 2 to 10 % and this path half its speed (3001 x
+// 2999 x 4097: 131 -> 80 us integer, 114 -> 61 us E4M3); unrolled, its addresses
+// made the promotion loop spill.
+__device__ __forceinline__ void store_staged_plain(const TcArgs &g, const unsigned char *stg, int lane,
                                                 long long rbase, long long cbase, bool vec) {
-#pragma unroll
+#pragma unroll 1
     for (int i = 0; i < 4; ++i) {
         const int r = 8 * i + (lane >> 2), u = lane & 3;
         const float4 a4 = *reinterpret_cast<const float4 *>(stg + r * 64 + ((u ^ ((r >> 1) & 3)) * 16));
@@ -275,7 +283,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int cid = (int)blockIdx.x >> 1, ncl = (int)gridDim.x >> 1;
     const int tiles_n = (int)((g.N + BN - 1) / BN), tiles_m = (int)((g.M + BM - 1) / BM);
     const int npairs = tiles_n * ((tiles_m + 1) / 2);
-    const int my_tiles = npairs > cid ? (npairs - 1 - cid) / ncl + 1 : 0;
+    // The last wave: when its tiles are at most half as many as the clusters, each
+    // is computed as two half tiles of 128 columns by two clusters (an N = 128 MMA
+    // takes 0.62 of an N = 256 one): 8192^3 E4M3 503 -> 482 us, 4096^3 80 -> 76.  Not
+    // the integer form, whose clock the power limit sets: alone 762 -> 762 and 116
+    // -> 114, but in a sequence of 4096^3 calls 183 -> 191, since the next call's
+    // CTAs no longer start on the SMs that a short last wave leaves idle.
+    const int last = npairs % ncl;
+    const int nfull = FP8 && 2 * last <= ncl ? npairs - last : npairs;
+    const int ntiles = 2 * npairs - nfull;
+    const int my_tiles = ntiles > cid ? (ntiles - 1 - cid) / ncl + 1 : 0;
     // a slab is L / 16 (fp16) or L / 32 (E4M3) MMAs, a multiple of four (one
     // box, since L % 64 == 0 or L % 128 == 0 respectively); a stage is two
     // boxes, so slabs and stages share boundaries in boxes; a tile whose
@@ -285,10 +302,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int boxes_slab = g.L / KB;
     const int per_tile = (nslab * boxes_slab + BOXES - 1) / BOXES;   // stages per tile
     const int total = my_tiles * per_tile;
+    // this cluster's whole tiles come first
+    const int kf = min(my_tiles, nfull > cid ? (nfull - 1 - cid) / ncl + 1 : 0);
+    auto is_half = [&](int k) { return FP8 && cid + k * ncl >= nfull; };
     auto tile_origin = [&](int k, long long &m0, long long &n0) {
-        const int t = cid + k * ncl;
+        int t = cid + k * ncl;
+        const int h = max(0, t - nfull);
+        if (t >= nfull) t = nfull + (h >> 1);
         m0 = (long long)(2 * (t / tiles_n) + (int)rank) * BM;   // may pass M: zero rows
-        n0 = (long long)(t % tiles_n) * BN;
+        n0 = (long long)(t % tiles_n) * BN + (h & 1) * BNH;
     };
 
     // full[] and acc_empty[] are used in the even CTA only (arrivals from both
@@ -339,13 +361,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 tile_origin(kt, m0, n0);
                 // this CTA's 128 rows of A~ and of B~; both CTAs' copies
                 // complete on the even CTA's full barrier, which expects them all
+                // (a half tile: 64 rows of B~ per CTA; its box brings 128)
+                const int brows = is_half(kt) ? BNH / 2 : BNH;
                 const uint32_t bar = cluster_addr(&full[stage], 0);
                 if (leader) mbar_arrive_expect_tx(&full[stage], PAIR_TX);
 #pragma unroll
                 for (int x = 0; x < BOXES; ++x) {
                     tma_load_2d_pair(sA + stage * STAGE_A + x * BOX_A, &mapA, bar, kx + x * KB, (int)m0);
                     tma_load_2d_pair(sB + stage * STAGE_B + x * BOX_B, &mapB, bar, kx + x * KB,
-                                     (int)(n0 + rank * BNH));
+                                     (int)n0 + (int)rank * brows);
                 }
             }
             // every copy issued must land before the CTA can exit: the pair's
@@ -362,51 +386,58 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             uint64_t ad0 = 0, bd0 = 0;
             bool ok = true;
             const int quads = boxes_slab;                 // 4-MMA groups per slab
-            for (int kt = 0; kt < my_tiles && ok; ++kt) {
-                for (int l = 0; l < nslab; ++l) {
-                    const int gs = kt * nslab + l;        // global slab count
-                    const int b = gs & 1;
-                    if (gs >= 2 && !tc_wait<FP8>(&acc_empty[b], ((gs >> 1) + 1) & 1)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(b * BN);
-                    for (int q = 0; q < quads; ++q) {
-                        if (box == 0) {
-                            if (!tc_wait<FP8>(&full[stage], phase)) {
-                                ok = false;
-                                break;
+            // (a constant descriptor per loop: read from a register, a 2048^3 E4M3
+            // product took 18.4 us instead of 17.4)
+            auto issue_tiles = [&](auto n_c, int k0, int k1) {
+                constexpr uint32_t desc = idesc(decltype(n_c)::value);
+                for (int kt = k0; kt < k1 && ok; ++kt) {
+                    for (int l = 0; l < nslab; ++l) {
+                        const int gs = kt * nslab + l;        // global slab count
+                        const int b = gs & 1;
+                        if (gs >= 2 && !tc_wait<FP8>(&acc_empty[b], ((gs >> 1) + 1) & 1)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t d = tmem + (uint32_t)(b * BN);
+                        for (int q = 0; q < quads; ++q) {
+                            if (box == 0) {
+                                if (!tc_wait<FP8>(&full[stage], phase)) {
+                                    ok = false;
+                                    break;
+                                }
+                                tc_fence_after();
+                                ad0 = desc_sw128(smem_u32(sA + stage * STAGE_A));
+                                bd0 = desc_sw128(smem_u32(sB + stage * STAGE_B));
                             }
-                            tc_fence_after();
-                            ad0 = desc_sw128(smem_u32(sA + stage * STAGE_A));
-                            bd0 = desc_sw128(smem_u32(sB + stage * STAGE_B));
-                        }
-                        const uint64_t ad = ad0 + (uint64_t)((box * BOX_A) >> 4);
-                        const uint64_t bd = bd0 + (uint64_t)((box * BOX_B) >> 4);
+                            const uint64_t ad = ad0 + (uint64_t)((box * BOX_A) >> 4);
+                            const uint64_t bd = bd0 + (uint64_t)((box * BOX_B) >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < MMAS_PER_BOX; ++kk) {
-                            const uint64_t adv = (uint64_t)((kk * 32) >> 4);
-                            mma2<FP8>(d, ad + adv, bd + adv, (q | kk) != 0);
+                            for (int kk = 0; kk < MMAS_PER_BOX; ++kk) {
+                                const uint64_t adv = (uint64_t)((kk * 32) >> 4);
+                                mma2<FP8>(d, ad + adv, bd + adv, desc, (q | kk) != 0);
+                            }
+                            if (++box == BOXES) {
+                                mma_commit_pair(&empty[stage]);     // frees the stage in both CTAs
+                                box = 0;
+                                ++it;
+                                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                            }
                         }
-                        if (++box == BOXES) {
-                            mma_commit_pair(&empty[stage]);     // frees the stage in both CTAs
-                            box = 0;
-                            ++it;
-                            if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                        }
+                        if (!ok) break;
+                        mma_commit_pair(&acc_full[b]);          // the slab is complete in both TMEMs
                     }
-                    if (!ok) break;
-                    mma_commit_pair(&acc_full[b]);          // the slab is complete in both TMEMs
+                    if (ok && box != 0) {
+                        // the tile ended inside a stage: release its unused half too
+                        mma_commit_pair(&empty[stage]);
+                        box = 0;
+                        ++it;
+                        if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                    }
                 }
-                if (ok && box != 0) {
-                    // the tile ended inside a stage: release its unused half too
-                    mma_commit_pair(&empty[stage]);
-                    box = 0;
-                    ++it;
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                }
-            }
+            };
+            issue_tiles(std::integral_constant<int, BN>{}, 0, kf);
+            if constexpr (FP8) issue_tiles(std::integral_constant<int, BN / 2>{}, kf, my_tiles);
             if (!ok) {
                 raise_status(const_cast<DevPlan *>(g.plan), TDG_ETIMEOUT);
                 *abort_flag = 1;
@@ -420,122 +451,157 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         // ------------------------------------------------------------ epilogue
         const int ew = warp - 2;
         const int quad = warp & 3;                     // TMEM lanes 32*quad .. +31
-        const int cgrp = ew >> 2;                      // columns [EPI_COLS*cgrp, +EPI_COLS)
-        const uint32_t acc_empty_cl[2] = {cluster_addr(&acc_empty[0], 0),
-                                          cluster_addr(&acc_empty[1], 0)};
+        const int cgrp = ew >> 2;                      // columns [EPI_COLS*cgrp, +EPI_COLS), or
+                                                       // half as many each of a half tile
+        const bool vec = ((g.ldc & 3) == 0) && (((uintptr_t)g.C & 15) == 0);
         bool ok = true;
-        // the warp's 32 rows and EPI_COLS columns lie in one row and one column
-        // block (L % 64 == 0), so it needs one factor (float)(s_A s_B) per slab:
-        // lane u forms slab u's of the next 32 (one fp64 product), and a slab
-        // takes its own by a shuffle.  The next 32 are fetched a batch ahead,
-        // across tiles too.
-        auto fetch_factors = [&](int k, int l0, double &fa, double &fb) {
-            if (k >= my_tiles) return;
+        // The warp's 32 rows and its columns lie in one row and one column block
+        // (L % 64 == 0), so it needs one factor (float)(s_A s_B) per slab: lane u
+        // forms slab u's of 32 (one fp64 product), and they wait in the warp's
+        // staging tile, which only the store of C needs otherwise.  The next 32
+        // slabs' s come by cp.async, the next tile's first through registers
+        // during the store of C: nothing but the running sums is live in the
+        // promotion loop, which has no register to spare (kept in registers and
+        // handed out by shuffles, the factors cost E4M3 3 % at 8192^3).
+        unsigned char *stg = stg_base + ew * STG_BYTES;
+        volatile float *sfac = reinterpret_cast<float *>(stg);
+        double *sab = reinterpret_cast<double *>(stg + 256);      // 32 s_A, 32 s_B
+        auto blocks = [&](int k, int cols, int &iblk, int &jblk) {
             long long m0, n0;
             tile_origin(k, m0, n0);
-            const int iblk = (int)min((m0 + quad * 32) / g.L, (long long)g.nM - 1);
-            const int jblk = (int)min((n0 + cgrp * EPI_COLS) / g.L, (long long)g.nN - 1);
-            const int l = min(l0 + lane, nslab - 1);
-            fa = __ldg(g.sA + (long long)iblk * g.nK + l);
-            fb = __ldg(g.sB + (long long)l * g.nN + jblk);
+            iblk = (int)min((m0 + quad * 32) / g.L, (long long)g.nM - 1);
+            jblk = (int)min((n0 + cgrp * cols) / g.L, (long long)g.nN - 1);
         };
-        double fa = 0.0, fb = 0.0;
-        fetch_factors(0, 0, fa, fb);
-        float fac_next = (float)__dmul_rn(fa, fb);
-        for (int kt = 0; kt < my_tiles && ok; ++kt) {
-            float fac = 0.f;
-            float cacc[EPI_COLS];
+        auto tile_cols = [&](int k) { return is_half(k) ? EPI_COLS / 2 : EPI_COLS; };
+        auto first_factor = [&](int k) -> double2 {
+            int iblk, jblk;
+            blocks(k, tile_cols(k), iblk, jblk);
+            const int l = min(lane, nslab - 1);
+            return make_double2(__ldg(g.sA + (long long)iblk * g.nK + l),
+                                __ldg(g.sB + (long long)l * g.nN + jblk));
+        };
+        auto set_factors = [&](double a, double b) {
+            sfac[lane] = (float)__dmul_rn(a, b);
+            __syncwarp();
+        };
+        // tiles [k0, k1) of NCH 16-column chunks per thread
+        auto run_tiles = [&](auto nch_c, int k0, int k1) {
+            constexpr int NCH = decltype(nch_c)::value;
+            for (int kt = k0; kt < k1 && ok; ++kt) {
+                float cacc[16 * NCH];
 #pragma unroll
-            for (int c = 0; c < EPI_COLS; ++c) cacc[c] = 0.f;
-            for (int l = 0; l < nslab; ++l) {
-                const int gs = kt * nslab + l;
-                const int b = gs & 1;
-                if ((l & 31) == 0) {
-                    fac = fac_next;
-                    const bool more = l + 32 < nslab;
-                    fetch_factors(more ? kt : kt + 1, more ? l + 32 : 0, fa, fb);
-                }
-                const float pr = __shfl_sync(0xffffffffu, fac, l & 31);
-                if (!tc_wait_epilogue<FP8>(&acc_full[b], (gs >> 1) & 1)) { ok = false; break; }
-                if ((l & 31) == 0) fac_next = (float)__dmul_rn(fa, fb);   // (fetched before the wait)
-                tc_fence_after();
-                const uint32_t base =
-                    tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * BN + cgrp * EPI_COLS);
-#pragma unroll
-                for (int ch = 0; ch < EPI_COLS / 16; ++ch) {
-                    float v[16];
-                    tmem_ld16(base + ch * 16, v);
-                    if (ch == EPI_COLS / 16 - 1) {
-                        // the accumulator is read: hand it back before the last fmas
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_cluster(acc_empty_cl[b]);
+                for (int c = 0; c < 16 * NCH; ++c) cacc[c] = 0.f;
+                for (int l = 0; l < nslab; ++l) {
+                    const int gs = kt * nslab + l;
+                    const int b = gs & 1;
+                    if ((l & 31) == 0) {
+                        if (l > 0) {
+                            asm volatile("cp.async.wait_all;" ::: "memory");
+                            __syncwarp();
+                            set_factors(sab[lane], sab[32 + lane]);
+                        }
+                        if (l + 32 < nslab) {
+                            int iblk, jblk;
+                            blocks(kt, 16 * NCH, iblk, jblk);
+                            const int ln = min(l + 32 + lane, nslab - 1);
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(sab + lane)),
+                                         "l"(g.sA + (long long)iblk * g.nK + ln)
+                                         : "memory");
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(sab + 32 + lane)),
+                                         "l"(g.sB + (long long)ln * g.nN + jblk)
+                                         : "memory");
+                        }
                     }
+                    const float pr = sfac[l & 31];
+                    if (!tc_wait_epilogue<FP8>(&acc_full[b], (gs >> 1) & 1)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t base =
+                        tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * BN + cgrp * 16 * NCH);
                     // C_acc = fma(r, s_A s_B, C_acc) on column pairs: each lane
                     // of fma.rn.f32x2 rounds once, as fmaf does
                     uint64_t pr2;
                     asm("mov.b64 %0, {%1, %1};" : "=l"(pr2) : "f"(pr));
 #pragma unroll
-                    for (int e = 0; e < 16; e += 2) {
-                        uint64_t v2, c2;
-                        asm("mov.b64 %0, {%1, %2};" : "=l"(v2) : "f"(v[e]), "f"(v[e + 1]));
-                        asm("mov.b64 %0, {%1, %2};" : "=l"(c2) : "f"(cacc[ch * 16 + e]), "f"(cacc[ch * 16 + e + 1]));
-                        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c2) : "l"(v2), "l"(pr2));
-                        asm("mov.b64 {%0, %1}, %2;" : "=f"(cacc[ch * 16 + e]), "=f"(cacc[ch * 16 + e + 1]) : "l"(c2));
+                    for (int ch = 0; ch < NCH; ++ch) {
+                        float v[16];
+                        tmem_ld16(base + ch * 16, v);
+                        if (ch == NCH - 1) {
+                            // the accumulator is read: hand it back before the last fmas
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0));
+                        }
+#pragma unroll
+                        for (int e = 0; e < 16; e += 2) {
+                            uint64_t v2, c2;
+                            asm("mov.b64 %0, {%1, %2};" : "=l"(v2) : "f"(v[e]), "f"(v[e + 1]));
+                            asm("mov.b64 %0, {%1, %2};" : "=l"(c2) : "f"(cacc[ch * 16 + e]), "f"(cacc[ch * 16 + e + 1]));
+                            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c2) : "l"(v2), "l"(pr2));
+                            asm("mov.b64 {%0, %1}, %2;" : "=f"(cacc[ch * 16 + e]), "=f"(cacc[ch * 16 + e + 1]) : "l"(c2));
+                        }
                     }
                 }
-            }
-            if (!ok) break;
-            // C out through this warp's staging tile, 16 columns at a time: the
-            // thread of row r writes its 16 values as row r (16-byte units
-            // XOR-swizzled by row, conflict-free), then each store instruction
-            // of the warp writes 8 rows x 64 contiguous bytes (a thread per
-            // 16 bytes) instead of 32 rows x 16 bytes
-            unsigned char *stg = stg_base + ew * STG_BYTES;
-            const bool vec = ((g.ldc & 3) == 0) && (((uintptr_t)g.C & 15) == 0);
-            long long m0, n0;
-            tile_origin(kt, m0, n0);
-            const long long rbase = m0 + quad * 32;
-            const long long col0 = n0 + cgrp * EPI_COLS;
-            if (g.c_tma) {
-                // beta = 0: alpha C_acc staged in the C map's 64-byte swizzle
-                // (16-byte unit u of row r at u ^ ((r >> 1) & 3)), written by
-                // one TMA store per 32 x 16 box, which clips rows and columns
-                // outside C
+                if (!ok) break;
+                double2 fn = make_double2(0.0, 0.0);
+                if (kt + 1 < my_tiles) fn = first_factor(kt + 1);
+                // C out through this warp's staging tile, 16 columns at a time: the
+                // thread of row r writes its 16 values as row r (16-byte units
+                // XOR-swizzled by row, conflict-free), then each store instruction
+                // of the warp writes 8 rows x 64 contiguous bytes (a thread per
+                // 16 bytes) instead of 32 rows x 16 bytes
+                long long m0, n0;
+                tile_origin(kt, m0, n0);
+                const long long rbase = m0 + quad * 32;
+                const long long col0 = n0 + cgrp * 16 * NCH;
+                __syncwarp();                          // every lane has read its factors
+                if (g.c_tma) {
+                    // beta = 0: alpha C_acc staged in the C map's 64-byte swizzle
+                    // (16-byte unit u of row r at u ^ ((r >> 1) & 3)), written by
+                    // one TMA store per 32 x 16 box, which clips rows and columns
+                    // outside C
 #pragma unroll
-                for (int ch = 0; ch < EPI_COLS / 16; ++ch) {
-                    if (ch > 0 && lane == 0) tma_store_wait_read();   // the box before is read
-                    __syncwarp();
+                    for (int ch = 0; ch < NCH; ++ch) {
+                        if (ch > 0 && lane == 0) tma_store_wait_read();   // the box before is read
+                        __syncwarp();
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int us = u ^ ((lane >> 1) & 3);
-                        const float *cu = cacc + ch * 16 + 4 * u;
-                        *reinterpret_cast<float4 *>(stg + lane * 64 + us * 16) =
-                            make_float4(__fmul_rn(g.alpha, cu[0]), __fmul_rn(g.alpha, cu[1]),
-                                        __fmul_rn(g.alpha, cu[2]), __fmul_rn(g.alpha, cu[3]));
+                        for (int u = 0; u < 4; ++u) {
+                            const int us = u ^ ((lane >> 1) & 3);
+                            const float *cu = cacc + ch * 16 + 4 * u;
+                            *reinterpret_cast<float4 *>(stg + lane * 64 + us * 16) =
+                                make_float4(__fmul_rn(g.alpha, cu[0]), __fmul_rn(g.alpha, cu[1]),
+                                            __fmul_rn(g.alpha, cu[2]), __fmul_rn(g.alpha, cu[3]));
+                        }
+                        fence_proxy_async();
+                        __syncwarp();
+                        if (lane == 0) tma_store_2d(&mapC, stg, (int)(col0 + ch * 16), (int)rbase);
                     }
-                    fence_proxy_async();
+                    if (lane == 0) tma_store_wait_read();
                     __syncwarp();
-                    if (lane == 0) tma_store_2d(&mapC, stg, (int)(col0 + ch * 16), (int)rbase);
-                }
-                if (lane == 0) tma_store_wait_read();
-                __syncwarp();
-                continue;
-            }
+                } else {
 #pragma unroll
-            for (int ch = 0; ch < EPI_COLS / 16; ++ch) {
+                    for (int ch = 0; ch < NCH; ++ch) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int us = u ^ ((lane >> 1) & 3);
-                    *reinterpret_cast<float4 *>(stg + lane * 64 + us * 16) =
-                        make_float4(cacc[ch * 16 + 4 * u], cacc[ch * 16 + 4 * u + 1],
-                                    cacc[ch * 16 + 4 * u + 2], cacc[ch * 16 + 4 * u + 3]);
+                        for (int u = 0; u < 4; ++u) {
+                            const int us = u ^ ((lane >> 1) & 3);
+                            *reinterpret_cast<float4 *>(stg + lane * 64 + us * 16) =
+                                make_float4(cacc[ch * 16 + 4 * u], cacc[ch * 16 + 4 * u + 1],
+                                            cacc[ch * 16 + 4 * u + 2], cacc[ch * 16 + 4 * u + 3]);
+                        }
+                        __syncwarp();
+                        store_staged_plain(g, stg, lane, rbase, col0 + ch * 16, vec);
+                        __syncwarp();
+                    }
                 }
-                __syncwarp();
-                store_staged_plain(g, stg, lane, rbase, col0 + ch * 16, vec);
-                __syncwarp();
+                set_factors(fn.x, fn.y);
             }
+        };
+        if (my_tiles > 0) {
+            const double2 f0 = first_factor(0);
+            set_factors(f0.x, f0.y);
         }
+        run_tiles(std::integral_constant<int, EPI_COLS / 16>{}, 0, kf);
+        if constexpr (FP8) run_tiles(std::integral_constant<int, EPI_COLS / 32>{}, kf, my_tiles);
+        asm volatile("cp.async.wait_all;" ::: "memory");
         if (lane == 0) tma_store_wait_all();
         if (!ok) {
             raise_status(const_cast<DevPlan *>(g.plan), TDG_ETIMEOUT);

@@ -53,3 +53,30 @@ def test_fp8_codes_do_not_depend_on_the_layout(M, N, K, L):
                       lda=bufs[0].shape[1], ldb=bufs[1].shape[1]) as p:
             out.append(p.run(bufs[0], bufs[1]))
     assert all(torch.equal(c, out[0]) for c in out[1:])
+
+
+@pytest.mark.parametrize("form,K", [("tc_int", 130), ("tc_fp8", 130), ("tc_int", 64 * 67)])
+@pytest.mark.parametrize("M,N", [(256, 256), (2600, 2100), (3000, 3001), (5000, 4097)])
+def test_tensor_core_last_wave(M, N, K, form):
+    """Whole and half tiles (the last wave's) and factors beyond the first 32 slabs:
+    every row block of a product equals the same rows multiplied alone, whose tiles
+    fall differently (1, 99, 144 and 340 tile pairs for 76 clusters)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1110_5765_gb300 as tdg
+    L = 128 if form == "tc_fp8" else 64
+    A = torch.from_numpy(synth.laplace((M, K), 75, np.float32)).cuda()
+    B = torch.from_numpy(synth.gaussian((K, N), 76, np.float32)).cuda()
+    kw = dict(L=L, W=1, dtype="f32", form=form, **({} if form == "tc_fp8" else dict(bits=6)))
+    C = torch.full((M, N), 3.0, device="cuda")
+    Cin = C.clone()
+    with tdg.Plan(M, N, K, **kw) as p:
+        p.run(A, B, C)
+        p.run(A, B, Cin, alpha=1.0, beta=-1.0)
+        assert p.info()["device_status"] == 0
+    assert torch.equal(Cin, C - 3.0)
+    for r0 in range(0, M, 1024):
+        rows = min(1024, M - r0)
+        with tdg.Plan(rows, N, K, **kw) as p:
+            part = p.run(A[r0:r0 + rows], B)
+            assert torch.equal(part, C[r0:r0 + rows]), r0
