@@ -294,7 +294,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
                     p->split_groups = (int)std::min<long long>(p->nK, (2 * sms + ntiles - 1) / ntiles);
             } else {
                 p->split_groups = f32_tile(mrows, N, p->nK, form == TDG_SYM ? Pof(L, W) : L,
-                                           form == TDG_SYM, true).groups;
+                                           form == TDG_SYM, p->mode == MODE_TARGET, true).groups;
             }
         }
         for (int w : candidates(p)) {

@@ -200,7 +200,9 @@ struct GemmCfg {
     static constexpr int NC = NCACC * TM * TN;         // sums per thread
     static constexpr int TMEM_COLS = pow2_at_least(2 * NC);
     // fp64: two CTAs per SM, so one's slab end overlaps the other's fma chains
-    static constexpr int MIN_CTAS = (TMEMC || (sizeof(T) == 8 && NC <= 16)) ? 2 : 1;
+    // fp32 64 x 64 tiles: three
+    static constexpr int MIN_CTAS = TMEMC && TM * TN == 16 && NCACC == 1 ? 3
+                                    : (TMEMC || (sizeof(T) == 8 && NC <= 16)) ? 2 : 1;
     static constexpr size_t STAGE_A = (size_t)BK * BM * sizeof(T);
     static constexpr size_t STAGE_B = (size_t)BK * BN * sizeof(T);
     static constexpr size_t RING = STAGES * (STAGE_A + STAGE_B) + STAGES * sizeof(uint64_t) + 16;
@@ -236,7 +238,8 @@ struct SlabWalk {
 // chain over all of K from the plain operands, no slab epilogue) instead of
 // the packed one.  Tiles never straddle inner kernels (L is a multiple of the
 // tile), and the block scheduler balances the two kinds of tile.
-// Wp: the packing that runs; P: its packed numbers per block.
+// Wp: the packing that runs; P: its packed numbers per block (the asymmetric form
+// reads g.P, the same: held in a register it cost 5 % of a 4096^3 product).
 template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, int RND>
 __device__ __forceinline__ void packed_gemm_tile(const CUtensorMap &mapA, const CUtensorMap &mapB,
                                                  const CUtensorMap &mapPA, const CUtensorMap &mapPB,
@@ -350,7 +353,7 @@ __device__ __forceinline__ void packed_gemm_tile(const CUtensorMap &mapA, const 
 #pragma unroll
         for (int e = 0; e < GR; ++e) {
             long long xr = x0 + gi * (BM / RG) + ty * GR + e;
-            long long ib = FORM == G_ASYM ? xr / P : xr / g.L;
+            long long ib = FORM == G_ASYM ? xr / g.P : xr / g.L;
             iblk[gi * GR + e] = (int)min(ib, (long long)g.nM - 1);
         }
 #pragma unroll
@@ -363,7 +366,7 @@ __device__ __forceinline__ void packed_gemm_tile(const CUtensorMap &mapA, const 
     auto out_row = [&](int i, int d) -> long long {
         const long long xr = x0 + (i / GR) * (BM / RG) + ty * GR + (i % GR);
         if (FORM == G_ASYM) {
-            const long long ib = xr / P, jr = xr % P;
+            const long long ib = xr / g.P, jr = xr % g.P;
             const long long inblk = jr * W + d;
             if (inblk >= g.L) return -1;
             return ib * g.L + inblk;
@@ -687,19 +690,11 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W
 
 // A distortion target's product in one launch: the packing, and whether the
 // target was met at all, are known on the device only.  The packed product
-// (symmetric: of any W, only the operand rows differ) is inlined, the plain
-// fallback (tile CP, arguments gp) called, which keeps their registers apart.
-// As launches of their own, the ones not chosen took 2 to 7 us each to return at
-// entry.  Not for the unsplit fp32 product in 8 x 8 thread tiles, which has no
+// (symmetric: of any W, only the operand rows differ) and the plain fallback (tile
+// CP, arguments gp) are one kernel.  As launches of their own, the ones not chosen
+// took 2 to 7 us each to return at entry.  Not for the unsplit fp32 product in 8 x 8 thread tiles, which has no
 // register to spare (1.155 ms instead of 1.106 at 4096^3): there both rounding
 // variants and the fallback are queued.
-template <typename T, typename CP>
-static __device__ __noinline__ void plain_gemm_apart(const CUtensorMap &mapA,
-                                                     const CUtensorMap &mapB,
-                                                     const GemmArgs<T> &g) {
-    packed_gemm_tile<T, G_PLAIN, 1, CP, false, false, 0>(mapA, mapB, mapA, mapB, g, 1, 0);
-}
-
 template <typename T, int FORM, int W, typename C, typename CP, bool KEEP>
 __global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W, C>::MIN_CTAS)
     target_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
@@ -711,7 +706,8 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W
     pdl_entry();
     const int Wp = g.plan->W;
     if (Wp == 1) {
-        if (g.fallback) plain_gemm_apart<T, CP>(mapPA, mapPB, gp);
+        if (g.fallback)
+            packed_gemm_tile<T, G_PLAIN, 1, CP, false, false, 0>(mapPA, mapPB, mapPA, mapPB, gp, 1, 0);
         return;
     }
     if (FORM == G_ASYM && Wp != g.W) return;

@@ -18,62 +18,71 @@ static bool small_plain(long long M, long long N) {
 // How a packed fp32 product over `slabs` slabs of `depth` k-rows is tiled.  A tile
 // costs clocks per k-row of its SM, measured with the symmetric kernel (K = 1024
 // to 4096; one tile on an SM / several): 128 x 128 202 / 177, 128 x 64 104 / 96,
-// 64 x 64 70 / 61.  The SM with the most tiles sets the time.  Splitting the slabs
-// of 128 x 128 tiles over all SMs runs 85 fma per clock and SM and moves every
-// slab's packed results out and in again (2.9 TB/s, and the second kernel's 8 us).
+// 64 x 64 70 / 61.  The SM with the most tiles sets the time.  Where even the
+// smallest tiles leave SMs idle, groups of slabs go to CTAs of their own (two to
+// an SM, so that they all run at once); that moves every slab's packed results out
+// (2.9 TB/s) and, in a second kernel (5 us), in again (4 TB/s).
 //   1024 x 1024 x 4096  split 187 us, 128 x 64 110, 64 x 64 128
 //   1000 x 777 x 1531   split  71 us, 128 x 64  46, 64 x 64  52
 //    700 x 700 x 3000   split  74 us, 128 x 64  84, 64 x 64  57
 //    512 x 512 x 4096   split  50 us, 128 x 64 110, 64 x 64  74
-F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, bool wide,
-                 bool may_split) {
-    const double sms = device_sms(), rows = (double)slabs * depth, mhz = 1940.0;
-    auto count = [&](long long bm, long long bn) {
-        return (double)(((mrows + bm - 1) / bm) * ((ncols + bn - 1) / bn));
-    };
-    auto cost = [&](long long bm, long long bn, double one, double more) {
-        const double r = ceil(count(bm, bn) / sms);
-        return rows * (r <= 1 ? one : r * more);
-    };
+F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, bool sym,
+                 bool target, bool may_split) {
+    const double sms = device_sms(), mhz = 1940.0;
+    struct Shape { int tile; long long bm, bn; double one, more; };
+    static const Shape shapes[] = {{F32_TILE_128, 128, 128, 202, 177},
+                                   {F32_TILE_MID, 128, 64, 104, 96},
+                                   {F32_TILE_SMALL, 64, 64, 70, 61}};
     F32Tile best{F32_TILE_128, 1};
-    double t = 0.97 * cost(128, 128, 202, 177);       // the default unless clearly slower
-    const double mid = cost(128, 64, 104, 96), small = cost(64, 64, 70, 61);
-    if (wide && mid < t) { best = {F32_TILE_MID, 1}; t = mid; }
-    if (small < t) { best = {F32_TILE_SMALL, 1}; t = small; }
-    const double tiles = count(128, 128);
-    if (may_split && slabs >= 4 && 2 * tiles <= sms) {
-        const double rbar = 4.0 * slabs * mrows * ncols;
-        const double split = 8.0 * mhz + rows * tiles * 128 * 128 / (sms * 85) +
-                             2 * rbar / 2.9e6 * mhz;
-        if (split < t)
-            best = {F32_TILE_128, (int)std::min<double>((double)slabs, (2 * sms + tiles - 1) / tiles)};
+    double least = INFINITY;
+    for (const Shape &s : shapes) {
+        if (s.tile == F32_TILE_MID && !sym) continue;
+        const double tiles = (double)((mrows + s.bm - 1) / s.bm) * ((ncols + s.bn - 1) / s.bn);
+        auto clocks = [&](double ctas, double rows) {
+            const double r = ceil(ctas / sms);
+            return rows * (r <= 1 ? s.one : r * s.more);
+        };
+        double t = clocks(tiles, (double)slabs * depth);
+        // the default unless clearly slower; a target's two other launches cost 6.6 us
+        if (s.tile == F32_TILE_128) t = 0.97 * t + (target ? 6.6 * mhz : 0.0);
+        if (t < least) { least = t; best = {s.tile, 1}; }
+        if (!may_split || s.tile == F32_TILE_MID || slabs < 4 || 2 * tiles > sms) continue;
+        const double spg = ceil(slabs / std::min<double>((double)slabs, floor(2 * sms / tiles)));
+        const double groups = ceil(slabs / spg), rbar = 4.0 * slabs * mrows * ncols;
+        t = clocks(tiles * groups, spg * depth) +
+            (rbar / 2.9e6 + rbar / 4e6 + 5.0) * mhz;
+        if (groups > 1 && t < least) { least = t; best = {s.tile, (int)groups}; }
     }
     return best;
 }
 
-// C: the packed tile; the plain fallback's by its own rule
+// C: the packed tile; the plain fallback's by its own rule, but for 64 x 64 tiles,
+// whose registers (three CTAs per SM) hold no larger one
 template <int FORM, int W, typename C>
 static cudaError_t go(const GemmArgs<float> &g, const GemmOperands &ops, cudaStream_t st) {
-    if (g.target && g.fallback && small_plain(g.M, g.N))
-        return launch_cfg<float, FORM, W, C, TilesF32Small>(g, ops, st);
-    return launch_cfg<float, FORM, W, C, TilesF32>(g, ops, st);
+    if constexpr (C::TM * C::TN > 16) {
+        if (!(g.target && g.fallback && small_plain(g.M, g.N)))
+            return launch_cfg<float, FORM, W, C, TilesF32>(g, ops, st);
+    }
+    return launch_cfg<float, FORM, W, C, TilesF32Small>(g, ops, st);
 }
 
-// Mixed tiles (Sec. 6) keep the tile that the tile order was made for, kept or
-// split slab results the 128 x 128 ones.
-static int tile_of(int form, int W, const GemmArgs<float> &g) {
-    if (g.kmask || g.Rbar) return F32_TILE_128;
-    return f32_tile(g.Mrows, g.N, g.nK, form == G_SYM ? (g.L + W - 1) / W : g.L, form == G_SYM, false)
+// Mixed tiles (Sec. 6) keep the tile that the tile order was made for, kept slab
+// results the 128 x 128 ones.
+static int tile_of(int form, int W, const GemmArgs<float> &g, bool target) {
+    if (g.kmask || (g.Rbar && g.groups <= 1)) return F32_TILE_128;
+    return f32_tile(g.Mrows, g.N, g.nK, form == G_SYM ? (g.L + W - 1) / W : g.L, form == G_SYM,
+                    target, g.groups > 1)
         .tile;
 }
 
 bool f32_target_in_one_launch(int form, int W, const GemmArgs<float> &g) {
-    return g.Rbar || tile_of(form, W, g) != F32_TILE_128;
+    return g.Rbar || tile_of(form, W, g, true) != F32_TILE_128;
 }
 
 template <int W, typename Big>
 static cudaError_t go_asym(const GemmArgs<float> &g, const GemmOperands &ops, cudaStream_t st) {
-    if (tile_of(G_ASYM, W, g) == F32_TILE_SMALL) return go<G_ASYM, W, TilesF32Small>(g, ops, st);
+    if (tile_of(G_ASYM, W, g, g.small_t < 0) == F32_TILE_SMALL) return go<G_ASYM, W, TilesF32Small>(g, ops, st);
     return go<G_ASYM, W, Big>(g, ops, st);
 }
 
@@ -90,7 +99,7 @@ cudaError_t launch_packed_gemm<float>(int form, int W, const GemmArgs<float> &g0
     }
     if (form == G_SYM) {
         // the symmetric kernel is the same for every W
-        switch (tile_of(form, W, g)) {
+        switch (tile_of(form, W, g, g.small_t < 0)) {
             case F32_TILE_MID: return go<G_SYM, 1, TilesF32Mid>(g, ops, st);
             case F32_TILE_SMALL: return go<G_SYM, 1, TilesF32Small>(g, ops, st);
             default: return go<G_SYM, 1, TilesF32>(g, ops, st);

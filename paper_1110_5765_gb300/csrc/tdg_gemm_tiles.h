@@ -17,7 +17,7 @@ using TilesF32 = Tiles<128, 128, 8, 8, 32, 3>;
 // fp32 products with few 128 x 128 tiles: half and quarter tiles, so that two or
 // four times as many SMs share the work (f32_tile)
 using TilesF32Mid = Tiles<128, 64, 8, 4, 32, 3>;
-using TilesF32Small = Tiles<64, 64, 4, 4, 32, 4>;
+using TilesF32Small = Tiles<64, 64, 4, 4, 32, 4>;       // 64 KB of ring: three CTAs per SM
 // fp32 asymmetric: 64 packed rows (W result rows each) x 128 columns
 using TilesF32Asym = Tiles<64, 128, 4, 8, 16, 6>;     // W >= 3: W x 32 running sums per thread
 using TilesF32AsymW2 = Tiles<128, 128, 8, 8, 32, 3>;  // W <= 2: W x 64 sums fit TMEM, 2.6 % faster

@@ -164,13 +164,13 @@ cudaError_t launch_px_gemm(int W, const GemmArgs<T> &g, const GemmOperands &ops,
 // edge of the others).
 int f64_tile_edge(long long mrows, long long ncols);
 // fp32 packed products: the tile, and how many groups the slabs are split into
-// (1: not split); wide: 128 x 64 tiles are among the choices (symmetric form)
+// (1: not split)
 enum { F32_TILE_128 = 0, F32_TILE_MID = 1, F32_TILE_SMALL = 2 };
 struct F32Tile {
     int tile, groups;
 };
-F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, bool wide,
-                 bool may_split);
+F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, bool sym,
+                 bool target, bool may_split);
 // whether a distortion target's product needs one launch only (symmetric: for
 // every W; with the plain fallback)
 bool f32_target_in_one_launch(int form, int W, const GemmArgs<float> &g);
