@@ -261,7 +261,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     size_t o_plan = off; off += up(sizeof(DevPlan));
     size_t o_done = off; off += up((size_t)p->nK * sizeof(unsigned int));
     size_t o_agg = off;
-    off += up(((size_t)4 * p->nK + (size_t)kLevelRecDoubles * (kMaxW - 1) * kMaxLevels) * 8);
+    off += up((size_t)4 * p->nK * 8);
     size_t o_mA = off; off += up(nAblk * 8);
     size_t o_eA = off; off += up(nAblk * 8);
     size_t o_mB = off; off += up(nBblk * 8);
@@ -473,6 +473,7 @@ static PlanParams params_of(const tdgemm_plan_s *p) {
     pp.allow_fallback = (p->flags & TDG_ALLOW_FALLBACK) ? 1 : 0;
     pp.noise_rms = (p->flags & TDG_NOISE_UNIFORM) ? 0 : 1;
     pp.target_db = p->target;
+    pp.target_ratio = p->mode == MODE_TARGET ? pow(10.0, p->target / 10.0) : 0.0;
     pp.manual_q = p->manual_q; pp.manual_cA = p->manual_cA; pp.manual_cB = p->manual_cB;
     pp.nM = p->nM; pp.nK = p->nK; pp.nN = p->nN;
     pp.M = p->M; pp.N = p->N; pp.K = p->K;
@@ -534,7 +535,7 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
                                      nB ? p->N : p->K, p->ldb, nB ? 0 : 1, p->nN, p->mB, p->eB,
                                      p->L, p->dplan, fin, st));
     }
-    CU_TRY(launch_planner(pp, stab, p->dplan, p->agg, st));
+    CU_TRY(launch_planner(pp, stab, p->dplan, st));
     const bool px = (p->flags & TDG_PAIR_EXACT) != 0;
     if (px)
         CU_TRY(launch_px_scales<T>(pp, p->mA, p->eA, p->mB, p->eB, p->dplan, (T *)p->cApx,

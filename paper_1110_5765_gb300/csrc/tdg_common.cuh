@@ -12,7 +12,6 @@ namespace tdg {
 constexpr int kUSafe = 50;             // Prop. 1: u_safe = 50
 constexpr int kMaxW = 4;               // packings built: W in 1..4
 constexpr int kMaxLevels = 192;        // R_max candidate levels t in [0, 192)
-constexpr int kLevelRecDoubles = 6;    // workspace per planner candidate (W, level)
 constexpr double kTcIntExact = 16777215.0;  // per-slab |sum| that fp32 holds exactly
 constexpr int kTcIntMaxGamma = 2048;        // integers exactly representable in fp16
 constexpr double kFp8Max = 448.0;           // largest finite E4M3 value
@@ -31,10 +30,11 @@ struct DevPlan {
     int status;        // tdg_status raised on the device (0 = ok)
     int nonfinite;     // NaN or Inf among the inputs of the last pack
     double pred_snr;   // model SNR (dB), NaN if not modelled
+    double ratio;      // target mode: S / N, whose 10 log10 the pack launch writes to
+    int log_pending;   // pred_snr when this is set
     double s_rep;      // representation-noise RMSE the model used (0 if none)
     double S, T1, T2, T3;  // noise-model aggregates
     // zero between calls (the decision, which writes the record, leaves them so)
-    unsigned int levels_done;  // candidate-level CTAs finished (the last one decides)
     unsigned int slabs_done;   // slabs whose aggregates are written
     int nonfinite_seen;        // set by the statistics kernels
     // target mode, written by the statistics' last warp: the slab sums S, T1,
@@ -87,7 +87,7 @@ struct PlanParams {
     int bits;          // fixed-bit mode
     int allow_fallback;
     int noise_rms;     // representation noise scaled by crest factors
-    double target_db;
+    double target_db, target_ratio;    // ratio: 10^(target_db / 10)
     int manual_q;
     double manual_cA, manual_cB;
     int nM, nK, nN;    // block counts

@@ -38,10 +38,8 @@ cudaError_t launch_block_stats(const T *A, long long rows_a, long long cols_a, l
                                const SlabFinish &fin, cudaStream_t st);
 
 // Planner, where the statistics did not decide the plan: target mode's
-// candidates (agg: 4 nK + kLevelRecDoubles (kMaxW - 1) kMaxLevels doubles of
-// workspace, the per-slab aggregates and one record per candidate (W, level)),
-// and calls without statistics.
-cudaError_t launch_planner(const PlanParams &pp, const double *stab, DevPlan *plan, double *agg,
+// candidates, and calls without statistics.
+cudaError_t launch_planner(const PlanParams &pp, const double *stab, DevPlan *plan,
                            cudaStream_t st);
 
 // Launch order of the tiles of a mixed (Sec. 6) launch: the tiles of

@@ -393,7 +393,7 @@ __device__ __forceinline__ void pack_both(const PackArgs<T> &a, const DevPlan *p
     const bool skipA = a.skipA || (!compand && a.directA), skipB = a.skipB || (!compand && a.directB);
     const unsigned int nA = skipA ? 0u : ga.tiles(), nB = skipB ? 0u : gb.tiles();
     const unsigned int np = compand ? (unsigned int)a.pair_tiles : 0u, both = 2 * min(nA, nB);
-    for (unsigned int t = blockIdx.x; t < np + nA + nB; t += gridDim.x) {
+    for (unsigned int t = blockIdx.x; t < np + nA + nB; t += a.log_cta) {
         if (t < np) {
             pair_tile(a, plan, t, reinterpret_cast<double *>(s));
             continue;
@@ -408,12 +408,17 @@ __device__ __forceinline__ void pack_both(const PackArgs<T> &a, const DevPlan *p
 
 template <typename T, bool ASYM>
 __global__ void __launch_bounds__(NT, 4) pack_kernel(const __grid_constant__ PackArgs<T> a,
-                                                     const DevPlan *plan) {
+                                                     DevPlan *plan) {
     pdl_entry();
     // staging: the largest tile is 64 (fp32) or 32 (fp64) rows of KSPAN numbers
     __shared__ __align__(16) unsigned char raw[(sizeof(T) == 4 ? 64 : 32) * (KSPAN + 1) * sizeof(T)];
     __shared__ T cs[64];
     T *s = reinterpret_cast<T *>(raw);
+    if (blockIdx.x == a.log_cta) {
+        // the predicted SNR of a target's plan, which only the host reads
+        if (threadIdx.x == 0 && plan->log_pending) plan->pred_snr = 10.0 * log10(plan->ratio);
+        return;
+    }
     const int W = a.plain ? 1 : plan->W;
     // W = 1 from the planner of a distortion target is the conventional product
     if (a.plain || (W == 1 && a.target)) {
@@ -441,7 +446,7 @@ __global__ void __launch_bounds__(NT, 4) pack_kernel(const __grid_constant__ Pac
 }  // namespace
 
 template <typename T>
-cudaError_t launch_pack(bool asym, const PackArgs<T> &a0, const DevPlan *plan, cudaStream_t st) {
+cudaError_t launch_pack(bool asym, const PackArgs<T> &a0, DevPlan *plan, cudaStream_t st) {
     PackArgs<T> a = a0;
     const long long tm = (a.nM + PAIR_TILE - 1) / PAIR_TILE, tn = (a.nN + PAIR_TILE - 1) / PAIR_TILE;
     const long long np = a.pair ? tm * tn * a.nK : 0;
@@ -455,13 +460,13 @@ cudaError_t launch_pack(bool asym, const PackArgs<T> &a0, const DevPlan *plan, c
     a.pair_tiles = (int)np;
     // a resident wave (four CTAs fit an SM), or less for small operands
     const long long want = np + (a.skipA ? 0 : bound(a.A)) + (a.skipB ? 0 : bound(a.B));
-    const unsigned int grid = (unsigned int)std::max(1LL, std::min(want, 4LL * device_sms()));
+    a.log_cta = (unsigned int)std::max(1LL, std::min(want, 4LL * device_sms()));
+    const unsigned int grid = a.log_cta + (a.target && !a.plain ? 1 : 0);
     return asym ? launch_pdl(pack_kernel<T, true>, dim3(grid), dim3(NT), 0, st, a, plan)
                 : launch_pdl(pack_kernel<T, false>, dim3(grid), dim3(NT), 0, st, a, plan);
 }
 
-template cudaError_t launch_pack<float>(bool, const PackArgs<float> &, const DevPlan *, cudaStream_t);
-template cudaError_t launch_pack<double>(bool, const PackArgs<double> &, const DevPlan *,
-                                         cudaStream_t);
+template cudaError_t launch_pack<float>(bool, const PackArgs<float> &, DevPlan *, cudaStream_t);
+template cudaError_t launch_pack<double>(bool, const PackArgs<double> &, DevPlan *, cudaStream_t);
 
 }  // namespace tdg

@@ -21,12 +21,15 @@ struct PackArgs {
     int skipA, skipB;         // operand kept from an earlier call
     int manual;
     double manual_cA, manual_cB;
-    int pair_tiles;           // set by the launcher
+    // set by the launcher: tiles of factors; CTAs that pack, and the index of the
+    // one after them (targets only)
+    int pair_tiles;
+    unsigned int log_cta;
 };
 
 // One launch over both operands for whichever W the device plan holds (along k:
 // the symmetric form and plain copies; asym: A along x, B unpacked).
 template <typename T>
-cudaError_t launch_pack(bool asym, const PackArgs<T> &a, const DevPlan *plan, cudaStream_t st);
+cudaError_t launch_pack(bool asym, const PackArgs<T> &a, DevPlan *plan, cudaStream_t st);
 
 }  // namespace tdg

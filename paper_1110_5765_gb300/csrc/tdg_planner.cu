@@ -7,8 +7,7 @@
 //   into four per-slab aggregates, so every candidate R_max level costs O(1):
 //     N = L T1 / (12 gB^2) + L T2 / (12 gA^2) + T3 (L/144 + s^2) / (gA gB)^2,
 //     S = L sum_l (sum_i sigma_A^2)(sum_j sigma_B^2).
-//   For each W from the request down to 2 the CTA evaluates every level in
-//   parallel, takes the argmin of N (eq. 27's argmax of the SNR; ties go to the
+//   For each W from the request down to 2 a CTA evaluates every level, takes the argmin of N (eq. 27's argmax of the SNR; ties go to the
 //   lower level) and keeps the first W whose SNR meets the target.  Otherwise
 //   W = 1 (plain product) with TDG_ALLOW_FALLBACK, else TDG_EUNREACHABLE.
 // * Manual mode: given q and uniform companders (the Sec. 4.B protocol).
@@ -23,60 +22,161 @@ namespace tdg {
 namespace {
 
 
-// Target mode, packed forms: each lane evaluates one candidate (W, R_max
-// level t) in full -- companders, z, representation noise, model noise and
-// SNR -- 32 candidates per CTA spread over SMs (fp64 divisions, square roots
-// and logarithms are slow on GB300 and would serialise on one SM).  The last
-// CTA to finish (a counter in the plan, no waiting) then decides the plan
-// from all records.  n < 0 marks a level without usable companders or
-// representation-noise value.
-__global__ void __launch_bounds__(32) level_kernel(PlanParams pp,
-                                                   const double *__restrict__ stab,
-                                                   LevelRec *res, DevPlan *plan) {
+// Target mode, packed forms: for W from the request down to 2 the R_max level of
+// least model noise (eq. 27's argmax of the SNR; ties to the lower level), the
+// first W whose SNR meets the target; else the plain product (fallback) or
+// TDG_EUNREACHABLE.
+//
+// An fp64 warp instruction takes 64 clocks of its SM sub-partition (2 lanes per
+// clock and SM), and a candidate is some 170 of them, so what counts is how many
+// follow one another.  One CTA: a warp per 32 levels forms the companders, then
+// four warps, one on each sub-partition, the four quotients of eq. 21 side by
+// side; the uniform quotients come from a fourth warp meanwhile.  The logarithm of
+// the SNR is left to the pack launch, where it delays nothing: the target is met
+// where S / N exceeds 10^(target / 10), and only within 1e-9 of that the logarithm
+// decides.  (A candidate per lane with every operation in sequence, 32 per CTA,
+// records in memory and the last CTA deciding, took 12 us.)
+constexpr int kGroups = 3, kTermWarps = 4 * kGroups;
+
+__global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
+                                                                const double *__restrict__ stab,
+                                                                DevPlan *plan) {
     pdl_entry();
-    const int L = pp.L;
-    const int lane = threadIdx.x;
+    __shared__ double term[4][32 * kGroups], rep[kMaxLevels], uni[2];
+    __shared__ int gam[2][kMaxLevels];
+    __shared__ unsigned long long best_n[kGroups];
+    __shared__ int best_t[kGroups];
+    __shared__ int met;
+    const int L = pp.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the slab sums and rho that the statistics' last warp wrote
+    const double S = (double)L * plan->tS, T1 = plan->tT1, T2 = plan->tT2, T3 = plan->tT3;
+    const double rho = plan->trho;
     int t_lo = 0;
     while (r_level(t_lo) < L) ++t_lo;
     const int t_hi = t_max_for(pp.p);
-    const int nlev = t_hi - t_lo + 1;
-    const int per_w = (nlev + 31) / 32;                 // CTAs per W
-    const int W = pp.Wreq - (int)blockIdx.x / per_w;
-    const int t = t_lo + ((int)blockIdx.x % per_w) * 32 + lane;
-    // the slab sums and rho that the statistics' last warp wrote
-    const double S = plan->tS, T1 = plan->tT1, T2 = plan->tT2, T3 = plan->tT3, rho = plan->trho;
-    if (W >= 2 && t <= t_hi) {
-        DevPlan a{};
-        a.S = (double)L * S; a.T1 = T1; a.T2 = T2; a.T3 = T3;
-        LevelRec r{};
-        r.n = -1.0;
-        const long long Rt = r_level(t);
-        r.q = q_for(Rt);
-        split_gammas(Rt, L, rho, r.gA, r.gB);
-        if (r.gA >= 1) {
-            r.R = (long long)L * r.gA * r.gB;
-            r.Wef = w_ef(r.R, r.q, pp.p);
-            double sv = -1.0;
-            if (W <= r.Wef) sv = 0.0;
-            else if (stab && t >= pp.t0 && t < pp.t0 + pp.nt) sv = stab[(W - 2) * pp.nt + (t - pp.t0)];
-            if (sv >= 0.0) {
-                r.n = model_noise(a, L, r.gA, r.gB, sv, pp.noise_rms);
-                r.pred = snr_db(a.S, r.n);
-                r.s = sv > 0.0 ? sv : 0.0;
+
+    // representation noise of level t for W with R = L gA gB (s < 0: not usable)
+    auto rep_noise = [&](int W, int t, int gA, int gB) -> double {
+        if (gA < 1) return -1.0;
+        if (W <= w_ef((long long)L * gA * gB, q_for(r_level(t)), pp.p)) return 0.0;
+        if (stab && t >= pp.t0 && t < pp.t0 + pp.nt) return __ldg(&stab[(W - 2) * pp.nt + (t - pp.t0)]);
+        return -1.0;
+    };
+    // quotient k of eq. 21 (model_noise), operation for operation
+    auto quotient = [&](int k, double gA, double gB, double s) -> double {
+        if (k == 0) return __ddiv_rn(__dmul_rn((double)L, T1), __dmul_rn(__dmul_rn(12.0, gB), gB));
+        if (k == 1) return __ddiv_rn(__dmul_rn((double)L, T2), __dmul_rn(__dmul_rn(12.0, gA), gA));
+        const double g2 = __dmul_rn(__dmul_rn(__dmul_rn(gA, gA), gB), gB);
+        if (k == 2)
+            return __ddiv_rn(__dmul_rn(T3, pp.noise_rms ? uni[0] : __dadd_rn(uni[0], __dmul_rn(s, s))), g2);
+        return __ddiv_rn(__dmul_rn(__dmul_rn(9.0, uni[1]), __dmul_rn(s, s)), g2);
+    };
+
+    DevPlan a{}, first{};
+    bool chosen = false, have_first = false;
+    for (int W = pp.Wreq; W >= 2 && !chosen; --W) {
+        unsigned long long bn = ~0ull;
+        int bt = -1;
+        for (int t0 = t_lo; t0 <= t_hi; t0 += 32 * kGroups) {
+            __syncthreads();
+            if (warp < kGroups) {
+                const int t = t0 + 32 * warp + lane;
+                if (t <= t_hi) {
+                    int gA, gB;
+                    split_gammas(r_level(t), L, rho, gA, gB);
+                    rep[t] = rep_noise(W, t, gA, gB);
+                    gam[0][t] = max(gA, 1);
+                    gam[1][t] = max(gB, 1);
+                }
+            } else if (warp == kGroups) {
+                const double l144 = __ddiv_rn((double)L, 144.0), sl = __ddiv_rn(S, (double)L);
+                if (lane == 0) {
+                    uni[0] = l144;
+                    uni[1] = sl;
+                }
+            }
+            __syncthreads();
+            {
+                // the warps of one sub-partition (warp % 4) take different quotients
+                const int g = warp >> 2, k = (warp + g) & 3, e = 32 * g + lane, t = t0 + e;
+                if (t <= t_hi && (k < 3 || pp.noise_rms))
+                    term[k][e] = quotient(k, (double)gam[0][t], (double)gam[1][t], rep[t]);
+            }
+            __syncthreads();
+            if (warp < kGroups) {
+                const int e = 32 * warp + lane;
+                if (t0 + e <= t_hi && rep[t0 + e] >= 0.0) {
+                    double n = __dadd_rn(__dadd_rn(term[0][e], term[1][e]), term[2][e]);
+                    if (pp.noise_rms) n = __dadd_rn(n, term[3][e]);
+                    // N >= 0: its bit pattern orders like its value
+                    const unsigned long long nb = (unsigned long long)__double_as_longlong(n);
+                    if (nb < bn) { bn = nb; bt = t0 + e; }           // levels ascend
+                }
             }
         }
-        res[(W - 2) * kMaxLevels + t] = r;
+        auto take = [&](unsigned long long n2, int t2) {
+            if (t2 >= 0 && (bt < 0 || n2 < bn || (n2 == bn && t2 < bt))) { bn = n2; bt = t2; }
+        };
+        if (warp < kGroups) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const unsigned long long n2 = __shfl_xor_sync(0xffffffffu, bn, off);
+                const int t2 = __shfl_xor_sync(0xffffffffu, bt, off);
+                take(n2, t2);
+            }
+            if (lane == 0) { best_n[warp] = bn; best_t[warp] = bt; }
+        }
+        __syncthreads();
+        bn = ~0ull;
+        bt = -1;
+        for (int g = 0; g < kGroups; ++g) take(best_n[g], best_t[g]);
+        if (bt < 0) continue;                          // the same in every thread
+        if (warp == 0) {                               // (fp64 once, not once per warp)
+            const double N = __longlong_as_double((long long)bn);
+            DevPlan c{};
+            c.W = W;
+            c.level = bt;
+            c.gA = gam[0][bt];
+            c.gB = gam[1][bt];
+            c.q = q_for(r_level(bt));
+            c.R = (long long)L * c.gA * c.gB;
+            c.Wef = w_ef(c.R, c.q, pp.p);
+            c.s_rep = rep[bt] > 0.0 ? rep[bt] : 0.0;
+            c.ratio = N <= 0.0 ? INFINITY : __ddiv_rn(S, N);
+            c.log_pending = 1;
+            if (!have_first) { first = c; have_first = true; }
+            bool ok = c.ratio > pp.target_ratio;
+            if (!(fabs(c.ratio - pp.target_ratio) > 1e-9 * pp.target_ratio))
+                ok = snr_db(S, N) >= pp.target_db;
+            if (ok) a = c;
+            if (lane == 0) met = ok;
+        }
+        __syncthreads();
+        chosen = met != 0;
     }
-    // the records of this CTA are written: count it; the last one decides
-    __threadfence();
-    __syncwarp();
-    unsigned int prev = 0;
-    if (lane == 0) prev = atomicAdd(&plan->levels_done, 1u);
-    prev = __shfl_sync(0xffffffffu, prev, 0);
-    if (prev + 1 == gridDim.x) {
-        __threadfence();
-        decide_plan(pp, stab, res, plan, S, T1, T2, T3, rho);
+    if (threadIdx.x != 0) return;
+    if (!chosen) {
+        if (pp.allow_fallback) {
+            a = DevPlan{};
+            a.W = 1;
+            a.level = -1;
+            a.pred_snr = INFINITY;
+        } else if (have_first) {
+            a = first;
+            a.status = TDG_EUNREACHABLE;
+        } else {
+            a = DevPlan{};
+            a.W = pp.Wreq; a.q = q_for(L); a.gA = a.gB = 1; a.R = L;
+            a.level = -1;
+            a.pred_snr = NAN;
+            a.status = TDG_EUNREACHABLE;
+        }
     }
+    a.S = S;
+    a.T1 = T1;
+    a.T2 = T2;
+    a.T3 = T3;
+    write_plan(a, plan);
 }
 
 // The plan of calls that take no statistics: the conventional product and
@@ -84,7 +184,7 @@ __global__ void __launch_bounds__(32) level_kernel(PlanParams pp,
 __global__ void __launch_bounds__(32) planner_kernel(PlanParams pp, const double *__restrict__ stab,
                                                      DevPlan *plan) {
     pdl_entry();
-    decide_plan(pp, stab, nullptr, plan, 0.0, 0.0, 0.0, 0.0, rho_of(0.0, 0.0));
+    decide_plan(pp, stab, plan, 0.0, 0.0, 0.0, 0.0, rho_of(0.0, 0.0));
 }
 
 // ---- Sec. 6: per inner kernel R_ij, predicted S_ij / N_ij with the call's
@@ -254,17 +354,10 @@ cudaError_t launch_kernel_control(const PlanParams &pp, const double *mA, const 
                       0, st, T, mode, thr, k, F, fw, plan, (const double *)ratio, mask);
 }
 
-cudaError_t launch_planner(const PlanParams &pp, const double *stab, DevPlan *plan, double *agg,
+cudaError_t launch_planner(const PlanParams &pp, const double *stab, DevPlan *plan,
                            cudaStream_t st) {
-    if (pp.mode == MODE_TARGET && (pp.form == TDG_SYM || pp.form == TDG_ASYM)) {
-        // every candidate level, the plan decided by the last CTA to finish
-        LevelRec *res = reinterpret_cast<LevelRec *>(agg + 4 * (long long)pp.nK);
-        int t_lo = 0;
-        while (r_level(t_lo) < pp.L) ++t_lo;
-        const int nlev = (pp.p == 24 ? 4 * 24 : 4 * 40) - t_lo + 1;
-        const int ctas = max(1, (pp.Wreq - 1) * ((nlev + 31) / 32));
-        return launch_pdl(level_kernel, dim3(ctas), dim3(32), 0, st, pp, stab, res, plan);
-    }
+    if (pp.mode == MODE_TARGET && (pp.form == TDG_SYM || pp.form == TDG_ASYM))
+        return launch_pdl(level_kernel, dim3(1), dim3(32 * kTermWarps), 0, st, pp, stab, plan);
     if (pp.form == TDG_PLAIN || pp.mode == MODE_MANUAL)
         return launch_pdl(planner_kernel, dim3(1), dim3(32), 0, st, pp, stab, plan);
     return cudaSuccess;      // decided by the statistics kernel

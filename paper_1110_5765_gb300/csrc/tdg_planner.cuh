@@ -63,42 +63,21 @@ __device__ inline double rho_of(double T1, double T2) {
     return (T1 <= 0.0 || T2 <= 0.0) ? 1.0 : sqrt(T2 / T1);
 }
 
-// Target mode, packed forms: every candidate (W, R_max level t) evaluated in
-// full by one lane (companders, z, representation noise, model noise and
-// SNR), 32 candidates per CTA spread over SMs: fp64 divisions, square roots
-// and logarithms are slow on GB300 and would serialise on one SM.  n < 0
-// marks a level without usable companders or representation-noise value.
-struct LevelRec {
-    double n, pred, s;
-    long long R;
-    int gA, gB, q, Wef;
-};
-static_assert(sizeof(LevelRec) == kLevelRecDoubles * sizeof(double), "planner workspace record");
-
-// a candidate record written by another CTA of the same grid: read from L2
-__device__ inline LevelRec load_rec(const LevelRec *p) {
-    LevelRec r;
-    r.n = __ldcg(&p->n);
-    r.pred = __ldcg(&p->pred);
-    r.s = __ldcg(&p->s);
-    r.R = __ldcg(&p->R);
-    r.gA = __ldcg(&p->gA);
-    r.gB = __ldcg(&p->gB);
-    r.q = __ldcg(&p->q);
-    r.Wef = __ldcg(&p->Wef);
-    return r;
+// The decided plan into the record (one thread).  The record's counters and the
+// statistics' flag return to zero here, for the next call's kernels.
+__device__ inline void write_plan(DevPlan a, DevPlan *plan) {
+    const int nf = __ldcg(&plan->nonfinite_seen);
+    a.nonfinite = nf;
+    if (nf && a.status == 0) a.status = TDG_ENONFINITE;
+    *plan = a;
 }
 
-// The plan, decided by one full warp: fixed bits, manual parameters, the
-// tensor-core forms, or (target mode, packed forms) the choice among the
-// candidate records res: for W from the request down to 2 the level of least
-// model noise (eq. 27's argmax of the SNR; ties to the lower level), the first
-// W whose SNR meets the target; else the plain product (fallback) or
-// TDG_EUNREACHABLE.  Lane 0 writes the plan.
+// The plan, decided by one full warp: fixed bits, manual parameters and the
+// tensor-core forms (a distortion target's choice of packing: level_kernel).
 static __device__ __forceinline__ void decide_plan(const PlanParams &pp,
-                                                const double *__restrict__ stab,
-                                                const LevelRec *res, DevPlan *plan, double S,
-                                                double T1, double T2, double T3, double rho) {
+                                                const double *__restrict__ stab, DevPlan *plan,
+                                                double S, double T1, double T2, double T3,
+                                                double rho) {
     const int lane = threadIdx.x & 31;
     const int L = pp.L;
     DevPlan a{};
@@ -148,78 +127,8 @@ static __device__ __forceinline__ void decide_plan(const PlanParams &pp,
             a.pred_snr = snr_db(a.S, model_noise(a, L, g, g, s, pp.noise_rms));
             a.s_rep = s;
         }
-    } else {  // MODE_TARGET, packed forms
-        int t_lo = 0;
-        while (r_level(t_lo) < L) ++t_lo;
-        const int t_hi = t_max_for(pp.p);
-        bool chosen = false;
-        DevPlan first{};
-        bool have_first = false;
-        for (int W = pp.Wreq; W >= 2 && !chosen; --W) {
-            // argmin of N over the levels (ties to the lower level); N >= 0,
-            // so its bit pattern orders like its value (integer compares)
-            // every load of the lane's levels issued before any is used
-            constexpr int kPerLane = (kMaxLevels + 31) / 32;
-            double nv[kPerLane];
-#pragma unroll
-            for (int u = 0; u < kPerLane; ++u) {
-                const int t = t_lo + lane + 32 * u;
-                nv[u] = t <= t_hi ? __ldcg(&res[(W - 2) * kMaxLevels + t].n) : -1.0;
-            }
-            unsigned long long bn = ~0ull;
-            int bt = -1;
-#pragma unroll
-            for (int u = 0; u < kPerLane; ++u) {     // lanes scan ascending t
-                if (nv[u] < 0.0) continue;
-                const unsigned long long nb = (unsigned long long)__double_as_longlong(nv[u]);
-                if (nb < bn) { bn = nb; bt = t_lo + lane + 32 * u; }
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const unsigned long long n2 = __shfl_xor_sync(0xffffffffu, bn, off);
-                const int t2 = __shfl_xor_sync(0xffffffffu, bt, off);
-                if (t2 >= 0 && (bt < 0 || n2 < bn || (n2 == bn && t2 < bt))) {
-                    bn = n2;
-                    bt = t2;
-                }
-            }
-            const int t = bt;                          // the same in every lane
-            if (t < 0) continue;
-            const LevelRec r = load_rec(&res[(W - 2) * kMaxLevels + t]);
-            DevPlan c = a;
-            c.W = W;
-            c.q = r.q;
-            c.gA = r.gA;
-            c.gB = r.gB;
-            c.R = r.R;
-            c.Wef = r.Wef;
-            c.level = t;
-            c.pred_snr = r.pred;
-            c.s_rep = r.s;
-            if (!have_first) { first = c; have_first = true; }
-            if (c.pred_snr >= pp.target_db) { a = c; chosen = true; }
-        }
-        if (!chosen) {
-            if (pp.allow_fallback) {
-                a.W = 1; a.q = 0; a.gA = a.gB = 0; a.R = 0; a.Wef = 0; a.level = -1;
-                a.pred_snr = INFINITY;
-            } else if (have_first) {
-                a = first;
-                a.status = TDG_EUNREACHABLE;
-            } else {
-                a.W = pp.Wreq; a.q = q_for(L); a.gA = a.gB = 1; a.R = L; a.Wef = 0;
-                a.status = TDG_EUNREACHABLE;
-            }
-        }
     }
-    if (lane == 0) {
-        // the record's counters and the statistics' flag return to zero here,
-        // for the next call's kernels
-        const int nf = __ldcg(&plan->nonfinite_seen);
-        a.nonfinite = nf;
-        if (nf && a.status == 0) a.status = TDG_ENONFINITE;
-        *plan = a;
-    }
+    if (lane == 0) write_plan(a, plan);
 }
 
 // Called by one full warp of a statistics CTA once its block of slab l is
@@ -231,7 +140,7 @@ static __device__ __forceinline__ void decide_plan(const PlanParams &pp,
 // its own for the aggregates, and one for the decision, took 7-9 and 2.5-8 us
 // of a call.  Inlined: as a call it cost the statistics and code kernels 1 to 3 us.
 // A target's candidates stay a kernel of their own: evaluated by this warp, three
-// rounds of fp64 latency, a 4096^3 fp32 call took 1217 us instead of 1204.)
+// rounds of fp64 work, a 4096^3 fp32 call took 1217 us instead of 1204.)
 struct SlabFinish {
     PlanParams pp;
     const double *mA, *vA, *mB, *vB;   // block maxima and variances of op(A), op(B)
@@ -274,7 +183,7 @@ static __device__ __forceinline__ void slab_finish(const SlabFinish &f, int l, D
             plan->slabs_done = 0;
         }
     } else {
-        decide_plan(f.pp, f.stab, nullptr, plan, S, T1, T2, T3, rho);
+        decide_plan(f.pp, f.stab, plan, S, T1, T2, T3, rho);
     }
 }
 

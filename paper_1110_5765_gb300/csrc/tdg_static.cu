@@ -109,7 +109,7 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     const size_t o_done = take((size_t)nK * sizeof(unsigned int));
     const size_t cleared = off;
     const size_t o_agg =
-        take(((size_t)4 * nK + (size_t)kLevelRecDoubles * (kMaxW - 1) * kMaxLevels) * 8);
+        take((size_t)4 * nK * 8);
     const size_t o_mA = take(nA_blk * 8), o_eA = take(nA_blk * 8);
     const size_t o_mB = take(nB_blk * 8), o_eB = take(nB_blk * 8);
     const size_t o_pair = take((size_t)nK * nM * nN * sizeof(T));
