@@ -150,26 +150,31 @@ struct SlabFinish {
     unsigned int blocks;               // arrivals per slab
 };
 
+// One arrival on a counter, ordered after this thread's (and, behind a barrier,
+// its CTA's) writes and before what it reads next; lighter than __threadfence()
+// around a relaxed atomic, which orders sequentially consistently.
+__device__ inline unsigned int arrive_acq_rel(unsigned int *p) {
+    unsigned int v;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 static __device__ __forceinline__ void slab_finish(const SlabFinish &f, int l, DevPlan *plan) {
     const int lane = threadIdx.x & 31;
     unsigned int prev = 0;
-    if (lane == 0) {
-        __threadfence();
-        prev = atomicAdd(&f.slab_done[l], 1u);
-    }
+    if (lane == 0) prev = arrive_acq_rel(&f.slab_done[l]);
     prev = __shfl_sync(0xffffffffu, prev, 0);
     if (prev + 1 != f.blocks) return;
-    __threadfence();
+    __syncwarp();
     const bool modelled = f.pp.form != TDG_TC_FP8;      // E4M3 has no noise model
     if (modelled) slab_aggregate_warp(l, f.pp.nM, f.pp.nK, f.pp.nN, f.mA, f.vA, f.mB, f.vB, f.agg);
     if (lane == 0) {
         f.slab_done[l] = 0;
-        __threadfence();
-        prev = atomicAdd(&plan->slabs_done, 1u);
+        prev = arrive_acq_rel(&plan->slabs_done);
     }
     prev = __shfl_sync(0xffffffffu, prev, 0);
     if (prev + 1 != (unsigned int)f.pp.nK) return;
-    __threadfence();
+    __syncwarp();
     double S = 0.0, T1 = 0.0, T2 = 0.0, T3 = 0.0;
     if (modelled) slab_totals(f.pp, f.agg, S, T1, T2, T3);
     const double rho = rho_of(T1, T2);
