@@ -323,15 +323,15 @@ def run_reference(args):
 # ---------------------------------------------------------------------------
 def launches_per_step(plan) -> int:
     """Kernels this library queues per tdgemm_run for a target-mode symmetric
-    fp32 plan with fallback, inputs 'N'/'N': block statistics of A and B (one
-    launch), planner (per-slab aggregates; every candidate level, the last CTA
-    deciding the plan), companders and de-companding factors, the packs of A
-    and B for W = 2 (one launch), plain copy of A for the W = 1 fallback (B is
-    used in place), the packed GEMM for W = 2 in both rounding variants of
-    eq. 10 (the add-subtract one when the planned q allows it, the rintf one
-    otherwise) and the plain GEMM for the fallback (kernels not chosen by the
-    planner exit at entry).  Counted from the ncu launch list of one step."""
-    return 1 + 2 + 2 + 1 + 1 + 3
+    fp32 plan with fallback at the benchmark's size, inputs 'N'/'N': block
+    statistics of A and B with the sums over them (one launch), the candidate
+    levels and the plan, the packs with companders and factors (one launch for
+    whatever W was planned, or the plain copies), the packed GEMM for W = 2 in
+    both rounding variants of eq. 10 (the add-subtract one when the planned q
+    allows it, the rintf one otherwise) and the plain GEMM for the fallback
+    (kernels not chosen by the planner exit at entry).  Counted from the ncu
+    launch list of one step."""
+    return 1 + 1 + 1 + 3
 
 
 def run_gpu(args):
