@@ -94,7 +94,7 @@ struct tdgemm_plan_s {
     double *mA, *eA, *mB, *eB, *sA, *sB, *stab, *agg;
     unsigned int *slab_done = nullptr;    // [nK], zero between calls
     bool clear_record = false;            // a pack failed half-way: counters to zero first
-    void *cA, *cB, *pair;
+    void *pair;
     void *Abuf, *Bbuf, *Rbar;
     void *cApx = nullptr, *cBpx = nullptr, *pairpx = nullptr;   // TDG_PAIR_EXACT
     size_t Abuf_bytes, Bbuf_bytes;
@@ -268,8 +268,6 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     size_t o_eB = off; off += up(nBblk * 8);
     size_t o_sA = off; off += up(nAblk * 8);
     size_t o_sB = off; off += up(nBblk * 8);
-    size_t o_cA = off; off += up(nAblk * p->esz);
-    size_t o_cB = off; off += up(nBblk * p->esz);
     size_t o_pair = off; off += up((size_t)p->nK * p->nM * p->nN * p->esz);
     size_t o_stab = off; off += up((size_t)(kMaxW - 1) * kMaxLevels * 8);
     const size_t npx = (flags & TDG_PAIR_EXACT) ? (size_t)p->nM * p->nK * p->nN : 0;
@@ -333,7 +331,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     p->mA = (double *)(p->ws + o_mA); p->eA = (double *)(p->ws + o_eA);
     p->mB = (double *)(p->ws + o_mB); p->eB = (double *)(p->ws + o_eB);
     p->sA = (double *)(p->ws + o_sA); p->sB = (double *)(p->ws + o_sB);
-    p->cA = p->ws + o_cA; p->cB = p->ws + o_cB; p->pair = p->ws + o_pair;
+    p->pair = p->ws + o_pair;
     p->stab = (double *)(p->ws + o_stab);
     if (npx) {
         p->cApx = p->ws + o_px;
