@@ -33,7 +33,11 @@
  *   - Argument errors are returned at once and leave the plan unchanged.
  *     Conditions found on the device (non-finite input, unreachable target)
  *     are written to a device status word that tdgemm_plan_info reads.
- *   - A plan is not thread-safe; distinct plans are independent.
+ *   - A plan is not thread-safe; distinct plans are independent.  The device
+ *     work of one plan's calls shares the plan's buffers, so it must not
+ *     overlap: queue the calls on one stream, or order the streams by events.
+ *     Calls that overlap all the same leave their own results undefined, but
+ *     not those of later calls.
  *   - Every failing call records a message readable with tdgemm_last_error()
  *     (thread-local).
  */

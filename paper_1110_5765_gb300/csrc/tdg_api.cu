@@ -92,8 +92,7 @@ struct tdgemm_plan_s {
     size_t ws_bytes = 0;
     DevPlan *dplan = nullptr;
     double *mA, *eA, *mB, *eB, *sA, *sB, *stab, *agg;
-    unsigned int *slab_done = nullptr;    // [nK], zero between calls
-    bool clear_record = false;            // a pack failed half-way: counters to zero first
+    unsigned int *slab_count = nullptr;   // the statistics' counters, zero between calls
     void *pair;
     void *Abuf, *Bbuf, *Rbar;
     void *cApx = nullptr, *cBpx = nullptr, *pairpx = nullptr;   // TDG_PAIR_EXACT
@@ -259,7 +258,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     const size_t nAblk = (size_t)p->nM * p->nK, nBblk = (size_t)p->nK * p->nN;
     size_t off = 0;
     size_t o_plan = off; off += up(sizeof(DevPlan));
-    size_t o_done = off; off += up((size_t)p->nK * sizeof(unsigned int));
+    size_t o_count = off; off += up(slab_count_bytes(p->nK));
     size_t o_agg = off;
     off += up((size_t)4 * p->nK * 8);
     size_t o_mA = off; off += up(nAblk * 8);
@@ -326,7 +325,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
         return fail(TDG_ECUDA, "cudaMemset: %s", cudaGetErrorString(e));
     }
     p->dplan = (DevPlan *)(p->ws + o_plan);
-    p->slab_done = (unsigned int *)(p->ws + o_done);
+    p->slab_count = (unsigned int *)(p->ws + o_count);
     p->agg = (double *)(p->ws + o_agg);
     p->mA = (double *)(p->ws + o_mA); p->eA = (double *)(p->ws + o_eA);
     p->mB = (double *)(p->ws + o_mB); p->eB = (double *)(p->ws + o_eB);
@@ -502,14 +501,6 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
                             bool reuse_b = false) {
     // reuse_b: B, its statistics, companders and packed copy are those of the
     // previous pack (the caller keeps B unchanged); only A is processed
-    // the record and its counters are zero where they must be after every
-    // complete call (and at the plan's creation), so a call clears them only
-    // when the one before it failed between its launches
-    if (p->clear_record) {
-        CU_TRY(cudaMemsetAsync(p->dplan, 0, sizeof(DevPlan), st));
-        CU_TRY(cudaMemsetAsync(p->slab_done, 0, (size_t)p->nK * sizeof(unsigned int), st));
-    }
-    p->clear_record = true;               // until every launch below is queued
     if (p->stab_dirty) {
         CU_TRY(cudaMemcpyAsync(p->stab, p->stab_host.data(), p->stab_host.size() * 8,
                                cudaMemcpyHostToDevice, st));
@@ -518,8 +509,8 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
     const bool nA = p->tA == 'N', nB = p->tB == 'N';
     PlanParams pp = params_of(p);
     const double *stab = p->have_table ? p->stab : nullptr;
-    const SlabFinish fin{pp, p->mA, p->eA, p->mB, p->eB, stab, p->agg, p->slab_done,
-                         (unsigned int)(p->nM + (reuse_b ? 0 : p->nN))};
+    SlabFinish fin{pp, p->mA, p->eA, p->mB, p->eB, stab, p->agg};
+    set_slab_counters(fin, p->slab_count, reuse_b);
     // tensor-core forms whose compander is gamma / max|x| of the block alone:
     // statistics, companders and codes in one pass over each input
     const bool tc_fused = is_tc_form(p->form) && p->mode == MODE_FIXED &&
@@ -592,7 +583,6 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
                 CU_TRY(launch_pack<T>(false, a, p->dplan, st));
         }
     }
-    p->clear_record = false;
     p->A_user = A;
     p->B_user = B;
     p->packed = true;

@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(THREADS, TS == 128 ? 1 : 2)
                         const int bkn = (int)min((long long)TS, o.K - k0);
                         o.var[idx] = ((double)h + (double)l) / ((double)bxn * (double)bkn);
                     }
-                    if (mb >= 0x7f800000u) atomicExch(&plan->nonfinite_seen, 1);
+                    if (mb >= 0x7f800000u) atomicExch(fin.nonfinite, 1);
                 }
             }
         } else {

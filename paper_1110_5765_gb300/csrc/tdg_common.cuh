@@ -34,12 +34,10 @@ struct DevPlan {
     int log_pending;   // pred_snr when this is set
     double s_rep;      // representation-noise RMSE the model used (0 if none)
     double S, T1, T2, T3;  // noise-model aggregates
-    // zero between calls (the decision, which writes the record, leaves them so)
-    unsigned int slabs_done;   // slabs whose aggregates are written
-    int nonfinite_seen;        // set by the statistics kernels
     // target mode, written by the statistics' last warp: the slab sums S, T1,
-    // T2, T3 (unscaled) and rho = sqrt(T2 / T1)
+    // T2, T3 (unscaled), rho = sqrt(T2 / T1), and whether NaN or Inf was seen
     double tS, tT1, tT2, tT3, trho;
+    int tnonfinite;
 };
 
 // Per-slab aggregates X_l = sum_i sigma_A,il^2, MA_l = sum_i m_A,il^2,

@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
     a.T1 = T1;
     a.T2 = T2;
     a.T3 = T3;
-    write_plan(a, plan);
+    write_plan(a, plan->tnonfinite, plan);
 }
 
 // The plan of calls that take no statistics: the conventional product and
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
 __global__ void __launch_bounds__(32) planner_kernel(PlanParams pp, const double *__restrict__ stab,
                                                      DevPlan *plan) {
     pdl_entry();
-    decide_plan(pp, stab, plan, 0.0, 0.0, 0.0, 0.0, rho_of(0.0, 0.0));
+    decide_plan(pp, stab, plan, 0.0, 0.0, 0.0, 0.0, rho_of(0.0, 0.0), 0);
 }
 
 // ---- Sec. 6: per inner kernel R_ij, predicted S_ij / N_ij with the call's

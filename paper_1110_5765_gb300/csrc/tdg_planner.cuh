@@ -63,10 +63,8 @@ __device__ inline double rho_of(double T1, double T2) {
     return (T1 <= 0.0 || T2 <= 0.0) ? 1.0 : sqrt(T2 / T1);
 }
 
-// The decided plan into the record (one thread).  The record's counters and the
-// statistics' flag return to zero here, for the next call's kernels.
-__device__ inline void write_plan(DevPlan a, DevPlan *plan) {
-    const int nf = __ldcg(&plan->nonfinite_seen);
+// The decided plan into the record (one thread); nf: NaN or Inf was seen.
+__device__ inline void write_plan(DevPlan a, int nf, DevPlan *plan) {
     a.nonfinite = nf;
     if (nf && a.status == 0) a.status = TDG_ENONFINITE;
     *plan = a;
@@ -77,7 +75,7 @@ __device__ inline void write_plan(DevPlan a, DevPlan *plan) {
 static __device__ __forceinline__ void decide_plan(const PlanParams &pp,
                                                 const double *__restrict__ stab, DevPlan *plan,
                                                 double S, double T1, double T2, double T3,
-                                                double rho) {
+                                                double rho, int nf) {
     const int lane = threadIdx.x & 31;
     const int L = pp.L;
     DevPlan a{};
@@ -128,7 +126,51 @@ static __device__ __forceinline__ void decide_plan(const PlanParams &pp,
             a.s_rep = s;
         }
     }
-    if (lane == 0) write_plan(a, plan);
+    if (lane == 0) write_plan(a, nf, plan);
+}
+
+// What the blocks of a call count up to, and what the last of them does.  The
+// counters are modulo counters: each wraps to zero with its last arrival in the
+// same atomic, so no store can drop an arrival, and after any number of complete
+// calls they stand at zero, also when two calls overlapped by mistake (their
+// results are then undefined, the next call's are not).  Calls that reuse B count
+// to another number and have counters of their own.
+struct SlabFinish {
+    PlanParams pp;
+    const double *mA, *vA, *mB, *vB;   // block maxima and variances of op(A), op(B)
+    const double *stab;
+    double *agg;
+    unsigned int *count;               // [nK] blocks per slab, [nK]: slabs
+    int *nonfinite;                    // set by the statistics, cleared with the decision
+    unsigned int blocks;               // arrivals per slab
+};
+
+// bytes of the counters and the flag of a plan: a counter set for calls that
+// process both operands, one for calls that reuse B
+constexpr size_t slab_count_bytes(int nK) { return (2 * ((size_t)nK + 1) + 1) * sizeof(unsigned int); }
+inline void set_slab_counters(SlabFinish &f, unsigned int *counters, bool reuse_b) {
+    const size_t set = (size_t)f.pp.nK + 1;
+    f.count = counters + (reuse_b ? set : 0);
+    f.nonfinite = reinterpret_cast<int *>(counters + 2 * set);
+    f.blocks = (unsigned int)(f.pp.nM + (reuse_b ? 0 : f.pp.nN));
+}
+
+// One arrival on a modulo-n counter, ordered after this thread's (and, behind a
+// barrier, its CTA's) writes and before what it reads next; lighter than
+// __threadfence() around a relaxed atomic, which orders sequentially consistently.
+// True for the last of n.
+__device__ inline bool last_arrival(unsigned int *p, unsigned int n) {
+#ifdef __CUDA_ARCH__
+    unsigned int v;
+    asm volatile("atom.inc.acq_rel.gpu.global.u32 %0, [%1], %2;"
+                 : "=r"(v)
+                 : "l"(p), "r"(n - 1)
+                 : "memory");
+#else
+    const unsigned int v = *p;
+    *p = v + 1 < n ? v + 1 : 0;
+#endif
+    return v == n - 1;
 }
 
 // Called by one full warp of a statistics CTA once its block of slab l is
@@ -136,48 +178,26 @@ static __device__ __forceinline__ void decide_plan(const PlanParams &pp,
 // (lanes over the blocks, as slab_aggregate_warp orders them), the last slab
 // the sums over slabs and rho -- and decides the plan, except for the packed
 // forms' target mode, whose candidates need a kernel of their own.  Counters
-// only, no waiting; each returns to zero with its last arrival.  (A kernel of
-// its own for the aggregates, and one for the decision, took 7-9 and 2.5-8 us
-// of a call.  Inlined: as a call it cost the statistics and code kernels 1 to 3 us.
-// A target's candidates stay a kernel of their own: evaluated by this warp, three
-// rounds of fp64 work, a 4096^3 fp32 call took 1217 us instead of 1204.)
-struct SlabFinish {
-    PlanParams pp;
-    const double *mA, *vA, *mB, *vB;   // block maxima and variances of op(A), op(B)
-    const double *stab;
-    double *agg;
-    unsigned int *slab_done;           // [nK], zero between calls
-    unsigned int blocks;               // arrivals per slab
-};
-
-// One arrival on a counter, ordered after this thread's (and, behind a barrier,
-// its CTA's) writes and before what it reads next; lighter than __threadfence()
-// around a relaxed atomic, which orders sequentially consistently.
-__device__ inline unsigned int arrive_acq_rel(unsigned int *p) {
-    unsigned int v;
-    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
+// only, no waiting.  (A kernel of its own for the aggregates, and one for the
+// decision, took 7-9 and 2.5-8 us of a call.  Inlined: as a call it cost the
+// statistics and code kernels 1 to 3 us.  A target's candidates stay a kernel of
+// their own: evaluated by this warp, three rounds of fp64 work, a 4096^3 fp32 call
+// took 1217 us instead of 1204.)
 static __device__ __forceinline__ void slab_finish(const SlabFinish &f, int l, DevPlan *plan) {
     const int lane = threadIdx.x & 31;
-    unsigned int prev = 0;
-    if (lane == 0) prev = arrive_acq_rel(&f.slab_done[l]);
-    prev = __shfl_sync(0xffffffffu, prev, 0);
-    if (prev + 1 != f.blocks) return;
+    int last = 0;
+    if (lane == 0) last = last_arrival(&f.count[l], f.blocks);
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __syncwarp();
     const bool modelled = f.pp.form != TDG_TC_FP8;      // E4M3 has no noise model
     if (modelled) slab_aggregate_warp(l, f.pp.nM, f.pp.nK, f.pp.nN, f.mA, f.vA, f.mB, f.vB, f.agg);
-    if (lane == 0) {
-        f.slab_done[l] = 0;
-        prev = arrive_acq_rel(&plan->slabs_done);
-    }
-    prev = __shfl_sync(0xffffffffu, prev, 0);
-    if (prev + 1 != (unsigned int)f.pp.nK) return;
+    if (lane == 0) last = last_arrival(&f.count[f.pp.nK], (unsigned int)f.pp.nK);
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __syncwarp();
     double S = 0.0, T1 = 0.0, T2 = 0.0, T3 = 0.0;
     if (modelled) slab_totals(f.pp, f.agg, S, T1, T2, T3);
     const double rho = rho_of(T1, T2);
+    const int nf = lane == 0 ? atomicExch(f.nonfinite, 0) : 0;
     if (f.pp.mode == MODE_TARGET && (f.pp.form == TDG_SYM || f.pp.form == TDG_ASYM)) {
         if (lane == 0) {
             plan->tS = S;
@@ -185,12 +205,11 @@ static __device__ __forceinline__ void slab_finish(const SlabFinish &f, int l, D
             plan->tT2 = T2;
             plan->tT3 = T3;
             plan->trho = rho;
-            plan->slabs_done = 0;
+            plan->tnonfinite = nf;
         }
     } else {
-        decide_plan(f.pp, f.stab, plan, S, T1, T2, T3, rho);
+        decide_plan(f.pp, f.stab, plan, S, T1, T2, T3, rho, nf);
     }
 }
 
 }  // namespace tdg
-

@@ -106,7 +106,7 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
     const size_t o_plan = take(sizeof(DevPlan));
-    const size_t o_done = take((size_t)nK * sizeof(unsigned int));
+    const size_t o_count = take(slab_count_bytes(nK));
     const size_t cleared = off;
     const size_t o_agg =
         take((size_t)4 * nK * 8);
@@ -139,8 +139,8 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     pp.allow_fallback = 0; pp.noise_rms = 0; pp.target_db = NAN;
     pp.nM = nM; pp.nK = nK; pp.nN = nN; pp.M = M; pp.N = N; pp.K = K;
     pp.t0 = 0; pp.nt = 0;
-    const SlabFinish fin{pp, mA, eA, mB, eB, nullptr, agg, (unsigned int *)(ws + o_done),
-                         (unsigned int)(nM + nN)};
+    SlabFinish fin{pp, mA, eA, mB, eB, nullptr, agg};
+    set_slab_counters(fin, (unsigned int *)(ws + o_count), false);
     ST_TRY(launch_block_stats<T>(A, nA ? M : K, nA ? K : M, lda, nA ? 0 : 1, nK, mA, eA, B,
                                  nB ? K : N, nB ? N : K, ldb, nB ? 0 : 1, nN, mB, eB, L, dplan,
                                  fin, st));

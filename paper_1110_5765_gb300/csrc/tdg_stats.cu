@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256, 3) block_stats_kernel(StatsOp<T> A, Stats
                                               : (long long)bi * o.nbc_op + bj;
                 o.mx[idx] = m;
                 o.var[idx] = ssum / ((double)rn * (double)cn);   // sigma^2 about zero
-                if (bad) atomicExch(&plan->nonfinite_seen, 1);
+                if (bad) atomicExch(fin.nonfinite, 1);
             }
         }
     }
