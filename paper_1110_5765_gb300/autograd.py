@@ -11,9 +11,14 @@ inputs; each backward product is companded and packed on its own, with
 companders and packing chosen from its own block statistics (Sec. 5, Sec. 6).
 Inside CUDA-graph capture the two adjoints of one product run on two streams.
 
-Plans (device workspace) are cached per shape, layout and options.
+Plans (device workspace) are cached per device, shape, layout and options.  A
+plan's calls must not overlap on the device, so each waits for the plan's last
+stream where that is another one, and two adjoints that share a plan stay on one
+stream.
 """
 from __future__ import annotations
+
+import threading
 
 import torch
 
@@ -46,12 +51,28 @@ def _side_stream(device) -> "torch.cuda.Stream":
     return st
 
 
-def _plan_for(M, N, K, tA, tB, lda, ldb, opts) -> Plan:
-    key = (M, N, K, tA, tB, lda, ldb, tuple(sorted(opts.items())))
+def _key(A, B, opts):
+    """Cache key of the product A B, with the stored operands."""
+    tA, lda, As = _op_layout(A)
+    tB, ldb, Bs = _op_layout(B)
+    return (A.shape[0], B.shape[1], A.shape[1], tA, tB, lda, ldb, A.device.index,
+            tuple(sorted(opts.items()))), As, Bs
+
+
+_creating = threading.Lock()
+
+
+def _plan_for(key, opts) -> Plan:
     p = _plans.get(key)
     if p is None:
-        p = Plan(M, N, K, transA=tA, transB=tB, lda=lda, ldb=ldb, **opts)
-        _plans[key] = p
+        with _creating:
+            p = _plans.get(key)
+            if p is None:
+                M, N, K, tA, tB, lda, ldb = key[:7]
+                p = Plan(M, N, K, transA=tA, transB=tB, lda=lda, ldb=ldb, **opts)
+                # the stream that last used the plan (outside capture)
+                p._lock, p._last = threading.Lock(), None
+                _plans[key] = p
     return p
 
 
@@ -63,13 +84,20 @@ def clear_plan_cache():
 
 def product(A: torch.Tensor, B: torch.Tensor, opts: dict) -> torch.Tensor:
     """C = A B through the library; A, B may be transposed views."""
-    tA, lda, As = _op_layout(A)
-    tB, ldb, Bs = _op_layout(B)
-    M, K = A.shape
-    N = B.shape[1]
-    p = _plan_for(M, N, K, tA, tB, lda, ldb, opts)
-    C = torch.empty((M, N), dtype=A.dtype, device=A.device)
-    p.run(As, Bs, C)
+    key, As, Bs = _key(A, B, opts)
+    C = torch.empty((A.shape[0], B.shape[1]), dtype=A.dtype, device=A.device)
+    p = _plan_for(key, opts)
+    with p._lock:                # (ordering the streams and queueing: one step)
+        st = torch.cuda.current_stream(A.device)
+        last = p._last
+        if last is None or last.cuda_stream != st.cuda_stream:
+            # a capture may not wait for work outside it: it begins with the
+            # device synchronised, and its replays are the caller's to order
+            if not torch.cuda.is_current_stream_capturing():
+                if last is not None:
+                    st.wait_stream(last)
+                p._last = st
+        p.run(As, Bs, C, stream=st)
     return C
 
 
@@ -88,7 +116,9 @@ class TDGemmFn(torch.autograd.Function):
         # two streams only inside CUDA-graph capture: replayed graphs carry no
         # host cost, while in eager mode the extra stream bookkeeping costs
         # more host time than the overlap saves on the device
-        if not (need_a and need_b) or not torch.cuda.is_current_stream_capturing():
+        # (a square layer of two transposed views: both adjoints have one plan)
+        if (not (need_a and need_b) or not torch.cuda.is_current_stream_capturing()
+                or _key(dC, B.t(), ctx.opts)[0] == _key(A.t(), dC, ctx.opts)[0]):
             dA = product(dC, B.t(), ctx.opts) if need_a else None
             dB = product(A.t(), dC, ctx.opts) if need_b else None
             return dA, dB, None
