@@ -93,6 +93,8 @@ struct tdgemm_plan_s {
     DevPlan *dplan = nullptr;
     double *mA, *eA, *mB, *eB, *sA, *sB, *stab, *agg;
     unsigned int *slab_count = nullptr;   // the statistics' counters, zero between calls
+    size_t head_bytes = 0;                // the record and the counters, first in ws
+    bool fresh = true;                    // head not yet cleared
     void *pair;
     void *Abuf, *Bbuf, *Rbar;
     void *cApx = nullptr, *cBpx = nullptr, *pairpx = nullptr;   // TDG_PAIR_EXACT
@@ -259,6 +261,7 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     size_t off = 0;
     size_t o_plan = off; off += up(sizeof(DevPlan));
     size_t o_count = off; off += up(slab_count_bytes(p->nK));
+    p->head_bytes = off;
     size_t o_agg = off;
     off += up((size_t)4 * p->nK * 8);
     size_t o_mA = off; off += up(nAblk * 8);
@@ -317,12 +320,6 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
         delete p;
         return fail(e == cudaErrorMemoryAllocation ? TDG_ENOMEM : TDG_ECUDA,
                     "workspace of %zu bytes: %s", off, cudaGetErrorString(e));
-    }
-    e = cudaMemset(p->ws, 0, off);
-    if (e != cudaSuccess) {
-        cudaFree(p->ws);
-        delete p;
-        return fail(TDG_ECUDA, "cudaMemset: %s", cudaGetErrorString(e));
     }
     p->dplan = (DevPlan *)(p->ws + o_plan);
     p->slab_count = (unsigned int *)(p->ws + o_count);
@@ -413,7 +410,6 @@ extern "C" tdg_status tdgemm_set_kernel_control(tdgemm_plan_t p, int mode, doubl
         p->ktiles_n = (p->N + bn - 1) / bn;
         CU_TRY(cudaMalloc(&p->kratio, (size_t)T * 8));
         CU_TRY(cudaMalloc(&p->kmask, (size_t)T));
-        CU_TRY(cudaMemset(p->kmask, 0, (size_t)T));
         CU_TRY(cudaMalloc(&p->korder, (size_t)(p->ktiles_m * p->ktiles_n) * sizeof(int)));
     }
     if (!p->kA) {
@@ -501,10 +497,20 @@ static tdg_status pack_impl(tdgemm_plan_t p, const T *A, const T *B, cudaStream_
                             bool reuse_b = false) {
     // reuse_b: B, its statistics, companders and packed copy are those of the
     // previous pack (the caller keeps B unchanged); only A is processed
-    if (p->stab_dirty) {
-        CU_TRY(cudaMemcpyAsync(p->stab, p->stab_host.data(), p->stab_host.size() * 8,
-                               cudaMemcpyHostToDevice, st));
-        p->stab_dirty = false;
+    // The record and the counters start at zero; every other byte of the workspace is
+    // written by a call before it is read.  Cleared on the first call's own stream: at
+    // the plan's creation cudaMemset would queue on the legacy default stream and could
+    // run after, or during, calls on a stream that does not wait for that one.  A graph
+    // under capture does both on every replay, and whether it ever runs is not known.
+    if (p->fresh || p->stab_dirty) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CU_TRY(cudaStreamIsCapturing(st, &cap));
+        const bool capturing = cap != cudaStreamCaptureStatusNone;
+        if (p->fresh) CU_TRY(cudaMemsetAsync(p->ws, 0, p->head_bytes, st));
+        if (p->stab_dirty)
+            CU_TRY(cudaMemcpyAsync(p->stab, p->stab_host.data(), p->stab_host.size() * 8,
+                                   cudaMemcpyHostToDevice, st));
+        if (!capturing) p->fresh = p->stab_dirty = false;
     }
     const bool nA = p->tA == 'N', nB = p->tB == 'N';
     PlanParams pp = params_of(p);
