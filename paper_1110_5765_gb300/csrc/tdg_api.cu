@@ -645,18 +645,21 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
     // the plain fallback too (mixed, pair-exact and large fp32 products: apart)
     bool one_launch = p->mode == MODE_TARGET && is_packed_form(p->form) && !p->kctrl_mode &&
                       !(p->flags & TDG_PAIR_EXACT);
-    if constexpr (sizeof(T) == 4) {
-        if (one_launch) {
-            GemmArgs<float> g{};
-            g.M = p->M; g.N = p->N; g.nK = p->nK; g.L = p->L; g.Rbar = (float *)p->Rbar;
-            // (one rule for all candidates: that of W = 2)
-            g.Mrows = op_shape(p, 2).a_cols;
-            one_launch = f32_target_in_one_launch(p->form == TDG_SYM ? G_SYM : G_ASYM, 2, g);
-        }
+    bool fallback_apart = false;
+    if (one_launch) {
+        GemmArgs<T> g{};
+        g.M = p->M; g.N = p->N; g.nK = p->nK; g.L = p->L; g.Rbar = (T *)p->Rbar;
+        g.groups = p->split_groups;
+        // (one rule for all candidates: that of W = 2)
+        g.Mrows = op_shape(p, 2).a_cols;
+        const int form = p->form == TDG_SYM ? G_SYM : G_ASYM;
+        if constexpr (sizeof(T) == 4) one_launch = f32_target_in_one_launch(form, 2, g);
+        fallback_apart = !fallback_keeps_tile(form, 2, g);
     }
     for (int w : candidates(p)) {
         const bool plain = (w == 0 || p->form == TDG_PLAIN);
-        if (one_launch && (w == 0 || (p->form == TDG_SYM && w > 2))) continue;
+        if (one_launch && w == 0 && !fallback_apart) continue;
+        if (one_launch && p->form == TDG_SYM && w > 2) continue;
         const int gform = plain ? G_PLAIN : (p->form == TDG_SYM ? G_SYM : G_ASYM);
         const int Wk = plain ? 1 : w;
         OpShape s = op_shape(p, w);
@@ -681,7 +684,7 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
         g.stall_ns = p->stall_ns;
         if (one_launch) {
             g.target = 1;
-            g.fallback = w == 2 && (p->flags & TDG_ALLOW_FALLBACK);
+            g.fallback = w == 2 && (p->flags & TDG_ALLOW_FALLBACK) && !fallback_apart;
             if (g.fallback) plain_ops(p->Abuf, p->Bbuf, ops.pa, ops.pb);
         }
         if (p->mode == MODE_FIXED) {

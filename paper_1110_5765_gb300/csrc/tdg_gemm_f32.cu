@@ -80,6 +80,10 @@ bool f32_target_in_one_launch(int form, int W, const GemmArgs<float> &g) {
     return g.Rbar || tile_of(form, W, g, true) != F32_TILE_128;
 }
 
+bool fallback_keeps_tile(int form, int W, const GemmArgs<float> &g) {
+    return tile_of(form, W, g, true) != F32_TILE_SMALL || small_plain(g.M, g.N);
+}
+
 template <int W, typename Big>
 static cudaError_t go_asym(const GemmArgs<float> &g, const GemmOperands &ops, cudaStream_t st) {
     if (tile_of(G_ASYM, W, g, g.small_t < 0) == F32_TILE_SMALL) return go<G_ASYM, W, TilesF32Small>(g, ops, st);

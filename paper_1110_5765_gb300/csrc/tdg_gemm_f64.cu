@@ -26,6 +26,10 @@ int f64_tile_edge(long long mrows, long long ncols) {
     return best;
 }
 
+bool fallback_keeps_tile(int, int, const GemmArgs<double> &g) {
+    return f64_tile_edge(g.Mrows, g.N) == f64_tile_edge(g.M, g.N);
+}
+
 template <int FORM, int W>
 static cudaError_t go(const GemmArgs<double> &g, const GemmOperands &ops, cudaStream_t st) {
     // mixed tiles (Sec. 6) keep the tile that the tile order was made for

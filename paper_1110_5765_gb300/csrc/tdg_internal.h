@@ -172,6 +172,14 @@ F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, b
 // whether a distortion target's product needs one launch only (symmetric: for
 // every W; with the plain fallback)
 bool f32_target_in_one_launch(int form, int W, const GemmArgs<float> &g);
+// whether the plain fallback runs in its own tile in such a launch (W = 2).  It has
+// the launch's tile (fp64) or one that fits beside it (fp32), and the asymmetric form
+// has about 1 / W as many packed rows as C has: where that tile is not the plain
+// product's own, the fallback is a launch by itself.  Missed targets, in / apart:
+// 1500 x 1300 x 3000 fp32 398 / 272 us, 2500 x 2500 x 300 142 / 101, 512^3 fp64
+// 299 / 263; met ones pay the launch, 299 / 303 us for the first with W = 3 asked.
+bool fallback_keeps_tile(int form, int W, const GemmArgs<float> &g);
+bool fallback_keeps_tile(int form, int W, const GemmArgs<double> &g);
 void packed_gemm_boxes(int dtype, int form, int W, int *box_x_a, int *box_x_b, int *bk);
 
 template <typename T>

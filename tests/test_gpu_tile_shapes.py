@@ -76,3 +76,28 @@ def test_f32_target_launches(orc, shape, form, W, target, used):
         C = p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda())
         assert p.info()["W_used"] == ref.plan.W
         assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
+
+
+@pytest.mark.parametrize("dtype,shape,W,target,used", [
+    ("f32", (1536, 1500, 130), 2, 20.0, 2), ("f32", (1536, 1500, 130), 2, 90.0, 1),
+    ("f32", (1536, 1500, 130), 4, 90.0, 1), ("f32", (2500, 1200, 66), 3, 90.0, 1),
+    ("f64", (512, 500, 130), 2, 20.0, 2), ("f64", (512, 500, 130), 3, 300.0, 1)])
+def test_fallback_apart(orc, dtype, shape, W, target, used):
+    """Asymmetric targets whose plain fallback has another tile than the packed
+    product, and so a launch by itself: met and missed."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1110_5765_gb300 as tdg
+    npt = np.float32 if dtype == "f32" else np.float64
+    M, N, K = shape
+    A, B = synth.uniform((M, K), 77, npt), synth.uniform((K, N), 78, npt)
+    C0 = synth.gaussian((M, N), 79, npt)
+    kw = dict(L=128, W=W, dtype=dtype, form="asym")
+    ref = orc.tdgemm(A, B, target_db=target, s_table=orc.load_s_table(), alpha=0.75, beta=-1.5,
+                     C_in=C0, **kw)
+    assert ref.plan.W == used
+    with tdg.Plan(M, N, K, target_snr_db=target, **kw) as p:
+        C = torch.from_numpy(C0.copy()).cuda()
+        p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C, 0.75, -1.5)
+        assert p.info()["W_used"] == used
+        assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
