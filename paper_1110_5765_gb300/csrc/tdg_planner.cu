@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
     // the slab sums and rho that the statistics' last warp wrote
     const double S = (double)L * plan->tS, T1 = plan->tT1, T2 = plan->tT2, T3 = plan->tT3;
     const double rho = plan->trho;
+    const int nf = plan->tnonfinite;
     int t_lo = 0;
     while (r_level(t_lo) < L) ++t_lo;
     const int t_hi = t_max_for(pp.p);
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
     a.T1 = T1;
     a.T2 = T2;
     a.T3 = T3;
-    write_plan(a, plan->tnonfinite, plan);
+    write_plan(a, nf, plan);
 }
 
 // The plan of calls that take no statistics: the conventional product and

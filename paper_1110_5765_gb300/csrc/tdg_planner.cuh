@@ -194,10 +194,11 @@ static __device__ __forceinline__ void slab_finish(const SlabFinish &f, int l, D
     if (lane == 0) last = last_arrival(&f.count[f.pp.nK], (unsigned int)f.pp.nK);
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __syncwarp();
+    // (on its way while the sums are taken)
+    const int nf = lane == 0 ? atomicExch(f.nonfinite, 0) : 0;
     double S = 0.0, T1 = 0.0, T2 = 0.0, T3 = 0.0;
     if (modelled) slab_totals(f.pp, f.agg, S, T1, T2, T3);
     const double rho = rho_of(T1, T2);
-    const int nf = lane == 0 ? atomicExch(f.nonfinite, 0) : 0;
     if (f.pp.mode == MODE_TARGET && (f.pp.form == TDG_SYM || f.pp.form == TDG_ASYM)) {
         if (lane == 0) {
             plan->tS = S;
