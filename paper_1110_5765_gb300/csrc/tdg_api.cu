@@ -175,6 +175,16 @@ static OpShape op_shape(const tdgemm_plan_s *p, int W) {
     return s;
 }
 
+// tile and slab groups of the fp32 product packed by w.  A symmetric target's product
+// is one launch for every packing, tiled for W = 2.
+static F32Tile f32_tile_of(const tdgemm_plan_s *p, int w, bool may_split) {
+    if (p->flags & TDG_KEEP_PACKED) return {F32_TILE_BIG, 1};
+    const bool sym = p->form == TDG_SYM, target = p->mode == MODE_TARGET;
+    const int W = sym && target ? 2 : w;
+    const long long mrows = sym ? p->M : (long long)p->nM * Pof(p->L, W);
+    return f32_tile({sym, W, p->L, mrows, p->N, p->nK, target, may_split});
+}
+
 static tdg_status validate(char tA, char tB, long long M, long long N, long long K,
                            long long lda, long long ldb, long long ldc, int L, int W, int dtype,
                            int form, double target, int bits) {
@@ -286,15 +296,15 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
         // the ordered sum over slabs in the unpack kernel; needs the r-bar
         // buffer that TDG_KEEP_PACKED also uses
         if (is_packed_form(form) && !(flags & (TDG_KEEP_PACKED | TDG_PAIR_EXACT)) && p->nK >= 4) {
-            const long long mrows = form == TDG_ASYM ? (long long)p->nM * Pof(L, W) : M;
             if (dtype == TDG_F64) {
+                const long long mrows = form == TDG_ASYM ? (long long)p->nM * Pof(L, W) : M;
                 const long long sms = device_sms(), edge = f64_tile_edge(mrows, N);
                 const long long ntiles = ((mrows + edge - 1) / edge) * ((N + edge - 1) / edge);
                 if (ntiles * 2 <= sms)
                     p->split_groups = (int)std::min<long long>(p->nK, (2 * sms + ntiles - 1) / ntiles);
             } else {
-                p->split_groups = f32_tile(mrows, N, p->nK, form == TDG_SYM ? Pof(L, W) : L,
-                                           form == TDG_SYM, p->mode == MODE_TARGET, true).groups;
+                for (int w : candidates(p))
+                    if (w >= 1) p->split_groups = std::max(p->split_groups, f32_tile_of(p, w, true).groups);
             }
         }
         for (int w : candidates(p)) {
@@ -645,16 +655,21 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
     // the plain fallback too (mixed, pair-exact and large fp32 products: apart)
     bool one_launch = p->mode == MODE_TARGET && is_packed_form(p->form) && !p->kctrl_mode &&
                       !(p->flags & TDG_PAIR_EXACT);
+    // mixed tiles (Sec. 6) keep the tile that the tile order was made for, kept slab
+    // results the big one
+    auto tile_of = [&](int w) -> F32Tile {
+        if (sizeof(T) == 8 || p->kctrl_mode || (p->flags & TDG_PAIR_EXACT)) return {F32_TILE_BIG, 1};
+        return f32_tile_of(p, w, p->split_groups > 1 && p->Rbar);
+    };
     bool fallback_apart = false;
     if (one_launch) {
-        GemmArgs<T> g{};
-        g.M = p->M; g.N = p->N; g.nK = p->nK; g.L = p->L; g.Rbar = (T *)p->Rbar;
-        g.groups = p->split_groups;
         // (one rule for all candidates: that of W = 2)
-        g.Mrows = op_shape(p, 2).a_cols;
-        const int form = p->form == TDG_SYM ? G_SYM : G_ASYM;
-        if constexpr (sizeof(T) == 4) one_launch = f32_target_in_one_launch(form, 2, g);
-        fallback_apart = !fallback_keeps_tile(form, 2, g);
+        const F32Tile t = tile_of(2);
+        GemmArgs<T> g{};
+        g.M = p->M; g.N = p->N; g.Mrows = op_shape(p, 2).a_cols; g.tile = t.tile;
+        if (sizeof(T) == 4)
+            one_launch = (p->flags & TDG_KEEP_PACKED) || t.groups > 1 || t.tile != F32_TILE_BIG;
+        fallback_apart = !fallback_keeps_tile(g);
     }
     for (int w : candidates(p)) {
         const bool plain = (w == 0 || p->form == TDG_PLAIN);
@@ -693,11 +708,16 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
         } else {
             g.small_t = p->mode == MODE_MANUAL ? 0 : -1;
         }
-        const bool split = !plain && p->split_groups > 1 && !p->kctrl_mode && p->Rbar;
-        if (split) {
-            g.Rbar = (T *)p->Rbar;
+        bool split = !plain && p->split_groups > 1 && !p->kctrl_mode && p->Rbar;
+        if (sizeof(T) == 4 && !plain) {
+            const F32Tile t = tile_of(w);
+            g.tile = t.tile;
+            g.groups = t.groups;
+            split = t.groups > 1;
+        } else if (split) {
             g.groups = p->split_groups;
         }
+        if (split) g.Rbar = (T *)p->Rbar;
         if (p->kctrl_mode && !plain) {
             // Sec. 6: the tiles of inner kernels left unaccelerated compute the
             // conventional product from the plain operands, same launch

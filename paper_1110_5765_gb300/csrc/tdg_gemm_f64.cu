@@ -26,7 +26,7 @@ int f64_tile_edge(long long mrows, long long ncols) {
     return best;
 }
 
-bool fallback_keeps_tile(int, int, const GemmArgs<double> &g) {
+bool fallback_keeps_tile(const GemmArgs<double> &g) {
     return f64_tile_edge(g.Mrows, g.N) == f64_tile_edge(g.M, g.N);
 }
 

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "tdg_common.cuh"
+#include "tdg_tile_rule.h"
 
 namespace tdg {
 
@@ -106,6 +107,7 @@ struct GemmArgs {
     // CTA computing one tile over one group and storing its packed slab
     // results; the launcher sets spg (slabs per group) and the final count
     int groups, spg;
+    int tile;               // fp32 packed forms: F32_TILE_* of this launch
     // test of the bounded waits: > 0 makes every CTA's first wait for operand
     // tiles wait on a barrier nothing completes, giving up after this many ns
     long long stall_ns;
@@ -162,24 +164,15 @@ cudaError_t launch_px_gemm(int W, const GemmArgs<T> &g, const GemmOperands &ops,
 // edge of the others).
 int f64_tile_edge(long long mrows, long long ncols);
 // fp32 packed products: the tile, and how many groups the slabs are split into
-// (1: not split)
-enum { F32_TILE_128 = 0, F32_TILE_MID = 1, F32_TILE_SMALL = 2 };
-struct F32Tile {
-    int tile, groups;
-};
-F32Tile f32_tile(long long mrows, long long ncols, long long slabs, int depth, bool sym,
-                 bool target, bool may_split);
-// whether a distortion target's product needs one launch only (symmetric: for
-// every W; with the plain fallback)
-bool f32_target_in_one_launch(int form, int W, const GemmArgs<float> &g);
+F32Tile f32_tile(const F32Product &p);
 // whether the plain fallback runs in its own tile in such a launch (W = 2).  It has
 // the launch's tile (fp64) or one that fits beside it (fp32), and the asymmetric form
 // has about 1 / W as many packed rows as C has: where that tile is not the plain
 // product's own, the fallback is a launch by itself.  Missed targets, in / apart:
 // 1500 x 1300 x 3000 fp32 398 / 272 us, 2500 x 2500 x 300 142 / 101, 512^3 fp64
 // 299 / 263; met ones pay the launch, 299 / 303 us for the first with W = 3 asked.
-bool fallback_keeps_tile(int form, int W, const GemmArgs<float> &g);
-bool fallback_keeps_tile(int form, int W, const GemmArgs<double> &g);
+bool fallback_keeps_tile(const GemmArgs<float> &g);
+bool fallback_keeps_tile(const GemmArgs<double> &g);
 void packed_gemm_boxes(int dtype, int form, int W, int *box_x_a, int *box_x_b, int *bk);
 
 template <typename T>

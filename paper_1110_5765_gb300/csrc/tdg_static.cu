@@ -164,6 +164,7 @@ tdg_status run_static(bool nA, bool nB, long long M, long long N, long long K, l
     g.L = L; g.P = P; g.nM = nM; g.nK = nK; g.nN = nN; g.pair = pair;
     g.C = C; g.ldc = ldc; g.alpha = (T)alpha; g.beta = (T)beta; g.beta_zero = beta == 0.0;
     g.Rbar = nullptr;
+    if (sizeof(T) == 4) g.tile = f32_tile({form == TDG_SYM, W, L, a_cols, N, nK, false, false}).tile;
     {
         const long long gam = (1LL << (bits - 1)) - 1;
         g.small_t = small_round_ok(gform, W, q_for((long long)L * gam * gam), (int)gam) ? 1 : 0;

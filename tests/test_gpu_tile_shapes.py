@@ -101,3 +101,30 @@ def test_fallback_apart(orc, dtype, shape, W, target, used):
         p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C, 0.75, -1.5)
         assert p.info()["W_used"] == used
         assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
+
+
+# asymmetric products in every tile of theirs, with W = 3 and 4 results a number, and
+# symmetric targets whose W is decided on the device
+@pytest.mark.parametrize("form,W,L,shape,kw", [
+    ("asym", 4, 64, (700, 900, 330), dict(bits=4)),         # 64 x 64, not split
+    ("asym", 4, 64, (100, 300, 1400), dict(bits=4)),        # 64 x 128, split
+    ("asym", 3, 64, (64, 40, 2000), dict(bits=4)),          # split, ragged digits
+    ("asym", 4, 64, (2300, 2500, 66), dict(bits=4)),        # 64 x 128, not split
+    ("sym", 4, 64, (130, 200, 2100), dict(target=15.0)),    # split
+    ("asym", 4, 64, (130, 200, 2100), dict(target=15.0)),   # split for some W
+    ("asym", 3, 64, (1300, 900, 260), dict(target=15.0)),
+])
+def test_tiles_by_form_and_packing(orc, form, W, L, shape, kw):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1110_5765_gb300 as tdg
+    M, N, K = shape
+    A, B = synth.uniform((M, K), 84, np.float32), synth.uniform((K, N), 85, np.float32)
+    goal = dict(bits=kw["bits"]) if "bits" in kw else dict(target_snr_db=kw["target"])
+    okw = dict(bits=kw["bits"]) if "bits" in kw else dict(target_db=kw["target"],
+                                                          s_table=orc.load_s_table())
+    ref = orc.tdgemm(A, B, L=L, W=W, dtype="f32", form=form, **okw)
+    with tdg.Plan(M, N, K, L=L, W=W, dtype="f32", form=form, **goal) as p:
+        C = p.run(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda())
+        assert p.info()["W_used"] == ref.plan.W
+        assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
