@@ -7,9 +7,10 @@
 //   into four per-slab aggregates, so every candidate R_max level costs O(1):
 //     N = L T1 / (12 gB^2) + L T2 / (12 gA^2) + T3 (L/144 + s^2) / (gA gB)^2,
 //     S = L sum_l (sum_i sigma_A^2)(sum_j sigma_B^2).
-//   For each W from the request down to 2 a CTA evaluates every level, takes the argmin of N (eq. 27's argmax of the SNR; ties go to the
-//   lower level) and keeps the first W whose SNR meets the target.  Otherwise
-//   W = 1 (plain product) with TDG_ALLOW_FALLBACK, else TDG_EUNREACHABLE.
+//   One CTA evaluates every level for each W from the request down to 2, takes
+//   the argmin of N (eq. 27's argmax of the SNR; ties go to the lower level) and
+//   keeps the first W whose SNR meets the target.  Otherwise W = 1 (plain
+//   product) with TDG_ALLOW_FALLBACK, else TDG_EUNREACHABLE.
 // * Manual mode: given q and uniform companders (the Sec. 4.B protocol).
 // The companders c and the de-companding factors (T)(s_A,il s_B,lj) follow in the
 // pack launch.
@@ -21,7 +22,6 @@ namespace tdg {
 
 namespace {
 
-
 // Target mode, packed forms: for W from the request down to 2 the R_max level of
 // least model noise (eq. 27's argmax of the SNR; ties to the lower level), the
 // first W whose SNR meets the target; else the plain product (fallback) or
@@ -29,24 +29,27 @@ namespace {
 //
 // An fp64 warp instruction takes 64 clocks of its SM sub-partition (2 lanes per
 // clock and SM), and a candidate is some 170 of them, so what counts is how many
-// follow one another.  One CTA: a warp per 32 levels forms the companders, then
-// four warps, one on each sub-partition, the four quotients of eq. 21 side by
-// side; the uniform quotients come from a fourth warp meanwhile.  The logarithm of
-// the SNR is left to the pack launch, where it delays nothing: the target is met
-// where S / N exceeds 10^(target / 10), and only within 1e-9 of that the logarithm
-// decides.  (A candidate per lane with every operation in sequence, 32 per CTA,
-// records in memory and the last CTA deciding, took 12 us.)
-constexpr int kGroups = 3, kTermWarps = 4 * kGroups;
+// follow one another.  One CTA: a warp per 32 levels forms the companders, which no
+// W changes, then the quotients of eq. 21, those that the representation noise
+// enters once per W, are dealt to the four sub-partitions side by side.  The
+// logarithm of the SNR is left to the pack launch, where it delays nothing: the
+// target is met where S / N exceeds 10^(target / 10), and only within 1e-9 of that
+// the logarithm decides.  (A candidate per lane with every operation in sequence, 32
+// per CTA, records in memory and the last CTA deciding, took 12 to 14 us; this kernel
+// with 96 levels and one W at a time 10, but 19 where W = 4 was asked and 2 met the
+// target, and 13 and 20 for the 145 levels of fp64.)
+constexpr int kTermWarps = 12, kGroups = kMaxLevels / 32, kWs = kMaxW - 1;
 
 __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
                                                                 const double *__restrict__ stab,
                                                                 DevPlan *plan) {
     pdl_entry();
-    __shared__ double term[4][32 * kGroups], rep[kMaxLevels], uni[2];
+    // [w]: of W = Wreq - w
+    __shared__ double term[3][kMaxLevels], wterm[kWs][kMaxLevels], rep[kWs][kMaxLevels], uni[2];
     __shared__ int gam[2][kMaxLevels];
-    __shared__ unsigned long long best_n[kGroups];
-    __shared__ int best_t[kGroups];
-    __shared__ int met;
+    __shared__ unsigned long long best_n[kWs][kGroups];
+    __shared__ int best_t[kWs][kGroups], met[kWs];
+    __shared__ DevPlan cand[kWs];
     const int L = pp.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the slab sums and rho that the statistics' last warp wrote
     const double S = (double)L * plan->tS, T1 = plan->tT1, T2 = plan->tT2, T3 = plan->tT3;
@@ -55,6 +58,7 @@ __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
     int t_lo = 0;
     while (r_level(t_lo) < L) ++t_lo;
     const int t_hi = t_max_for(pp.p);
+    const int ng = (t_hi - t_lo) / 32 + 1, nw = pp.Wreq - 1;      // groups of levels, packings
 
     // representation noise of level t for W with R = L gA gB (s < 0: not usable)
     auto rep_noise = [&](int W, int t, int gA, int gB) -> double {
@@ -63,115 +67,119 @@ __global__ void __launch_bounds__(32 * kTermWarps) level_kernel(PlanParams pp,
         if (stab && t >= pp.t0 && t < pp.t0 + pp.nt) return __ldg(&stab[(W - 2) * pp.nt + (t - pp.t0)]);
         return -1.0;
     };
-    // quotient k of eq. 21 (model_noise), operation for operation
-    auto quotient = [&](int k, double gA, double gB, double s) -> double {
-        if (k == 0) return __ddiv_rn(__dmul_rn((double)L, T1), __dmul_rn(__dmul_rn(12.0, gB), gB));
-        if (k == 1) return __ddiv_rn(__dmul_rn((double)L, T2), __dmul_rn(__dmul_rn(12.0, gA), gA));
-        const double g2 = __dmul_rn(__dmul_rn(__dmul_rn(gA, gA), gB), gB);
-        if (k == 2)
-            return __ddiv_rn(__dmul_rn(T3, pp.noise_rms ? uni[0] : __dadd_rn(uni[0], __dmul_rn(s, s))), g2);
-        return __ddiv_rn(__dmul_rn(__dmul_rn(9.0, uni[1]), __dmul_rn(s, s)), g2);
-    };
-
-    DevPlan a{}, first{};
-    bool chosen = false, have_first = false;
-    for (int W = pp.Wreq; W >= 2 && !chosen; --W) {
+    if (warp < ng) {
+        const int t = t_lo + 32 * warp + lane;
+        if (t <= t_hi) {
+            int gA, gB;
+            split_gammas(r_level(t), L, rho, gA, gB);
+            for (int w = 0; w < nw; ++w) rep[w][t] = rep_noise(pp.Wreq - w, t, gA, gB);
+            gam[0][t] = max(gA, 1);
+            gam[1][t] = max(gB, 1);
+        }
+    } else if (warp == ng) {
+        const double l144 = __ddiv_rn((double)L, 144.0), sl = __ddiv_rn(S, (double)L);
+        if (lane == 0) {
+            uni[0] = l144;
+            uni[1] = sl;
+        }
+    }
+    __syncthreads();
+    // the quotients of eq. 21 (model_noise), operation for operation: nb that no W
+    // enters, then one per W.  (Warp i and i + 12 share a sub-partition.)
+    const int nb = pp.noise_rms ? 3 : 2;
+    for (int i = warp; i < (nb + nw) * ng; i += kTermWarps) {
+        const int k = i / ng, t = t_lo + 32 * (i % ng) + lane;
+        if (t > t_hi) continue;
+        const double gA = (double)gam[0][t], gB = (double)gam[1][t];
+        if (k == 0) {
+            term[0][t] = __ddiv_rn(__dmul_rn((double)L, T1), __dmul_rn(__dmul_rn(12.0, gB), gB));
+        } else if (k == 1) {
+            term[1][t] = __ddiv_rn(__dmul_rn((double)L, T2), __dmul_rn(__dmul_rn(12.0, gA), gA));
+        } else {
+            const double g2 = __dmul_rn(__dmul_rn(__dmul_rn(gA, gA), gB), gB);
+            if (k < nb) {
+                term[2][t] = __ddiv_rn(__dmul_rn(T3, uni[0]), g2);
+            } else {
+                const double s = rep[k - nb][t];
+                wterm[k - nb][t] =
+                    __ddiv_rn(pp.noise_rms ? __dmul_rn(__dmul_rn(9.0, uni[1]), __dmul_rn(s, s))
+                                           : __dmul_rn(T3, __dadd_rn(uni[0], __dmul_rn(s, s))),
+                              g2);
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = warp; i < nw * ng; i += kTermWarps) {
+        const int w = i / ng, g = i % ng, t = t_lo + 32 * g + lane;
         unsigned long long bn = ~0ull;
         int bt = -1;
-        for (int t0 = t_lo; t0 <= t_hi; t0 += 32 * kGroups) {
-            __syncthreads();
-            if (warp < kGroups) {
-                const int t = t0 + 32 * warp + lane;
-                if (t <= t_hi) {
-                    int gA, gB;
-                    split_gammas(r_level(t), L, rho, gA, gB);
-                    rep[t] = rep_noise(W, t, gA, gB);
-                    gam[0][t] = max(gA, 1);
-                    gam[1][t] = max(gB, 1);
-                }
-            } else if (warp == kGroups) {
-                const double l144 = __ddiv_rn((double)L, 144.0), sl = __ddiv_rn(S, (double)L);
-                if (lane == 0) {
-                    uni[0] = l144;
-                    uni[1] = sl;
-                }
-            }
-            __syncthreads();
-            {
-                // the warps of one sub-partition (warp % 4) take different quotients
-                const int g = warp >> 2, k = (warp + g) & 3, e = 32 * g + lane, t = t0 + e;
-                if (t <= t_hi && (k < 3 || pp.noise_rms))
-                    term[k][e] = quotient(k, (double)gam[0][t], (double)gam[1][t], rep[t]);
-            }
-            __syncthreads();
-            if (warp < kGroups) {
-                const int e = 32 * warp + lane;
-                if (t0 + e <= t_hi && rep[t0 + e] >= 0.0) {
-                    double n = __dadd_rn(__dadd_rn(term[0][e], term[1][e]), term[2][e]);
-                    if (pp.noise_rms) n = __dadd_rn(n, term[3][e]);
-                    // N >= 0: its bit pattern orders like its value
-                    const unsigned long long nb = (unsigned long long)__double_as_longlong(n);
-                    if (nb < bn) { bn = nb; bt = t0 + e; }           // levels ascend
-                }
-            }
+        if (t <= t_hi && rep[w][t] >= 0.0) {
+            double n = __dadd_rn(term[0][t], term[1][t]);
+            if (pp.noise_rms) n = __dadd_rn(n, term[2][t]);
+            // N >= 0: its bit pattern orders like its value
+            bn = (unsigned long long)__double_as_longlong(__dadd_rn(n, wterm[w][t]));
+            bt = t;
         }
-        auto take = [&](unsigned long long n2, int t2) {
-            if (t2 >= 0 && (bt < 0 || n2 < bn || (n2 == bn && t2 < bt))) { bn = n2; bt = t2; }
-        };
-        if (warp < kGroups) {
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const unsigned long long n2 = __shfl_xor_sync(0xffffffffu, bn, off);
-                const int t2 = __shfl_xor_sync(0xffffffffu, bt, off);
-                take(n2, t2);
-            }
-            if (lane == 0) { best_n[warp] = bn; best_t[warp] = bt; }
+        for (int off = 16; off > 0; off >>= 1) {
+            const unsigned long long n2 = __shfl_xor_sync(0xffffffffu, bn, off);
+            const int t2 = __shfl_xor_sync(0xffffffffu, bt, off);
+            if (t2 >= 0 && (bt < 0 || n2 < bn || (n2 == bn && t2 < bt))) { bn = n2; bt = t2; }
         }
-        __syncthreads();
-        bn = ~0ull;
-        bt = -1;
-        for (int g = 0; g < kGroups; ++g) take(best_n[g], best_t[g]);
-        if (bt < 0) continue;                          // the same in every thread
-        if (warp == 0) {                               // (fp64 once, not once per warp)
+        if (lane == 0) { best_n[w][g] = bn; best_t[w][g] = bt; }
+    }
+    __syncthreads();
+    if (warp < nw) {                                   // W = Wreq - warp
+        unsigned long long bn = ~0ull;
+        int bt = -1;
+        for (int g = 0; g < ng; ++g)                   // levels ascend
+            if (best_t[warp][g] >= 0 && (bt < 0 || best_n[warp][g] < bn)) {
+                bn = best_n[warp][g];
+                bt = best_t[warp][g];
+            }
+        int ok = -1;                                   // no usable level
+        if (bt >= 0) {
             const double N = __longlong_as_double((long long)bn);
             DevPlan c{};
-            c.W = W;
+            c.W = pp.Wreq - warp;
             c.level = bt;
             c.gA = gam[0][bt];
             c.gB = gam[1][bt];
             c.q = q_for(r_level(bt));
             c.R = (long long)L * c.gA * c.gB;
             c.Wef = w_ef(c.R, c.q, pp.p);
-            c.s_rep = rep[bt] > 0.0 ? rep[bt] : 0.0;
+            c.s_rep = rep[warp][bt] > 0.0 ? rep[warp][bt] : 0.0;
             c.ratio = N <= 0.0 ? INFINITY : __ddiv_rn(S, N);
             c.log_pending = 1;
-            if (!have_first) { first = c; have_first = true; }
-            bool ok = c.ratio > pp.target_ratio;
+            ok = c.ratio > pp.target_ratio;
             if (!(fabs(c.ratio - pp.target_ratio) > 1e-9 * pp.target_ratio))
                 ok = snr_db(S, N) >= pp.target_db;
-            if (ok) a = c;
-            if (lane == 0) met = ok;
+            if (lane == 0) cand[warp] = c;
         }
-        __syncthreads();
-        chosen = met != 0;
+        if (lane == 0) met[warp] = ok;
     }
+    __syncthreads();
     if (threadIdx.x != 0) return;
-    if (!chosen) {
-        if (pp.allow_fallback) {
-            a = DevPlan{};
-            a.W = 1;
-            a.level = -1;
-            a.pred_snr = INFINITY;
-        } else if (have_first) {
-            a = first;
-            a.status = TDG_EUNREACHABLE;
-        } else {
-            a = DevPlan{};
-            a.W = pp.Wreq; a.q = q_for(L); a.gA = a.gB = 1; a.R = L;
-            a.level = -1;
-            a.pred_snr = NAN;
-            a.status = TDG_EUNREACHABLE;
-        }
+    int pick = -1, first = -1;
+    for (int w = nw - 1; w >= 0; --w) {
+        if (met[w] >= 0) first = w;
+        if (met[w] > 0) pick = w;
+    }
+    DevPlan a{};
+    if (pick >= 0) {
+        a = cand[pick];
+    } else if (pp.allow_fallback) {
+        a.W = 1;
+        a.level = -1;
+        a.pred_snr = INFINITY;
+    } else if (first >= 0) {
+        a = cand[first];
+        a.status = TDG_EUNREACHABLE;
+    } else {
+        a.W = pp.Wreq; a.q = q_for(L); a.gA = a.gB = 1; a.R = L;
+        a.level = -1;
+        a.pred_snr = NAN;
+        a.status = TDG_EUNREACHABLE;
     }
     a.S = S;
     a.T1 = T1;
