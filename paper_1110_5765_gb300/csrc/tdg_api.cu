@@ -706,7 +706,8 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
             const long long gam = (1LL << (p->bits - 1)) - 1;
             g.small_t = small_round_ok(gform, Wk, q_for((long long)p->L * gam * gam), (int)gam) ? 1 : 0;
         } else {
-            g.small_t = p->mode == MODE_MANUAL ? 0 : -1;
+            // (targets: known on the device, but never for symmetric W > 2)
+            g.small_t = p->mode == MODE_MANUAL || (gform == G_SYM && Wk != 2) ? 0 : -1;
         }
         bool split = !plain && p->split_groups > 1 && !p->kctrl_mode && p->Rbar;
         if (sizeof(T) == 4 && !plain) {
