@@ -129,7 +129,6 @@ struct tdgemm_plan_s {
     bool packed = false, gemm_done = false, b_packed = false;
     int split_groups = 1;   // slab splitting of the packed GEMM (> 1: on)
     long long stall_ns = 0; // test of the bounded waits (tdgemm_set_wait_test)
-    int last_pack_W = 0;
     cudaStream_t last_stream = nullptr;
     int device = 0;
 };
@@ -280,7 +279,8 @@ extern "C" tdg_status tdgemm_plan(tdgemm_plan_t *plan, char transA, char transB,
     size_t o_eB = off; off += up(nBblk * 8);
     size_t o_sA = off; off += up(nAblk * 8);
     size_t o_sB = off; off += up(nBblk * 8);
-    size_t o_pair = off; off += up((size_t)p->nK * p->nM * p->nN * p->esz);
+    // (the tensor-core forms take their factors from s_A and s_B)
+    size_t o_pair = off; off += is_tc_form(form) ? 0 : up((size_t)p->nK * p->nM * p->nN * p->esz);
     size_t o_stab = off; off += up((size_t)(kMaxW - 1) * kMaxLevels * 8);
     const size_t npx = (flags & TDG_PAIR_EXACT) ? (size_t)p->nM * p->nK * p->nN : 0;
     size_t o_px = off; off += up(3 * npx * p->esz);      // c_A, c_B, pair factors per (i, l, j)

@@ -814,7 +814,8 @@ cudaError_t launch_target(const GemmArgs<T> &g0, const GemmOperands &ops, cudaSt
 // that code.  CP: the plain fallback's tile.
 template <typename T, int FORM, int W, typename C, typename CP>
 cudaError_t launch_cfg(const GemmArgs<T> &g, const GemmOperands &ops, cudaStream_t st) {
-    if constexpr (FORM == G_SYM && C::TM >= 4) {
+    // (mixed products keep the largest tile of their type)
+    if constexpr (FORM == G_SYM && C::TM * C::TN == (sizeof(T) == 4 ? 64 : 16)) {
         if (g.kmask) {
             if (g.Rbar || !ops.pa.base || !ops.pb.base) return cudaErrorInvalidValue;
             if constexpr (sizeof(T) == 4)

@@ -36,19 +36,17 @@ __device__ inline double snr_db(double S, double N) {
 // S / L, T1, T2, T3: products of the per-slab aggregates summed over slabs by
 // one warp (lanes over l, then a fixed xor tree); every caller gets the same
 // bits.
-__device__ inline void slab_totals(const PlanParams &pp, const double *__restrict__ agg,
-                                   double &S, double &T1, double &T2, double &T3) {
+__device__ inline void slab_totals(const double *__restrict__ agg, int nK, double &S, double &T1,
+                                   double &T2, double &T3) {
     const int lane = threadIdx.x & 31;
     S = T1 = T2 = T3 = 0.0;
-    if (pp.mode != MODE_MANUAL) {
-        for (int l = lane; l < pp.nK; l += 32) {
-            const double X = __ldcg(&agg[4 * (long long)l]), MA = __ldcg(&agg[4 * (long long)l + 1]);
-            const double Y = __ldcg(&agg[4 * (long long)l + 2]), MB = __ldcg(&agg[4 * (long long)l + 3]);
-            S += X * Y;
-            T1 += X * MB;
-            T2 += Y * MA;
-            T3 += MA * MB;
-        }
+    for (int l = lane; l < nK; l += 32) {
+        const double X = __ldcg(&agg[4 * (long long)l]), MA = __ldcg(&agg[4 * (long long)l + 1]);
+        const double Y = __ldcg(&agg[4 * (long long)l + 2]), MB = __ldcg(&agg[4 * (long long)l + 3]);
+        S += X * Y;
+        T1 += X * MB;
+        T2 += Y * MA;
+        T3 += MA * MB;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -197,7 +195,7 @@ static __device__ __forceinline__ void slab_finish(const SlabFinish &f, int l, D
     // (on its way while the sums are taken)
     const int nf = lane == 0 ? atomicExch(f.nonfinite, 0) : 0;
     double S = 0.0, T1 = 0.0, T2 = 0.0, T3 = 0.0;
-    if (modelled) slab_totals(f.pp, f.agg, S, T1, T2, T3);
+    if (modelled) slab_totals(f.agg, f.pp.nK, S, T1, T2, T3);
     const double rho = rho_of(T1, T2);
     if (f.pp.mode == MODE_TARGET && (f.pp.form == TDG_SYM || f.pp.form == TDG_ASYM)) {
         if (lane == 0) {
