@@ -354,9 +354,14 @@ cudaError_t launch_kernel_control(const PlanParams &pp, const double *mA, const 
                                   int mode, double thr, long long k, double F,
                                   const Speedups &fw, double *ratio, unsigned char *mask,
                                   cudaStream_t st) {
-    const long long T = (long long)pp.nM * pp.nN;
-    cudaError_t e = launch_pdl(kernel_ratio_kernel, dim3((unsigned)((T * 32 + 255) / 256)),
-                               dim3(256), 0, st, pp, mA, vA, mB, vB, plan, ratio);
+    const long long T = (long long)pp.nM * pp.nN, ctas = (T * 32 + 255) / 256;
+    // Behind the statistics' full wave the few CTAs, launched early, pile up on the SMs
+    // that are left first and share their fp64 pipes (fixed bits, 2048^3: the steps up to
+    // the product took 73 us, with a plain launch 58).  A target's decision, one CTA,
+    // leaves them all.
+    const bool pdl = pp.mode == MODE_TARGET || pdl_for_grid(ctas);
+    cudaError_t e = launch_pdl_if(pdl, kernel_ratio_kernel, dim3((unsigned)ctas), dim3(256), 0, st,
+                                  pp, mA, vA, mB, vB, plan, ratio);
     if (e != cudaSuccess) return e;
     return launch_pdl(kernel_mask_kernel,
                       dim3((unsigned)((T + kMaskThreads - 1) / kMaskThreads)), dim3(kMaskThreads),
