@@ -25,6 +25,7 @@
 
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
+#include "tdg_optin.h"
 #include "tdg_planner.cuh"
 
 namespace tdg {
@@ -327,9 +328,8 @@ cudaError_t go(const CodesOp &A, const CodesOp &B, int L, double gamma, long lon
                DevPlan *plan, const SlabFinish &fin, cudaStream_t st) {
     constexpr size_t smem = (size_t)STAGES * TS * TS * sizeof(float);
     auto kern = codes_kernel<FP8, TS, FUSED>;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr != cudaSuccess) return attr;
+    static SmemOptIn smem_ok;
+    if (cudaError_t e = smem_ok.allow(kern, (int)smem)) return e;
     const long long total = (long long)A.tiles + B.tiles;
     const long long grid = std::min<long long>(total, (TS == 128 ? 1LL : 2LL) * device_sms());
     return launch_pdl(kern, dim3((unsigned)grid), dim3(THREADS), smem, st, A, B, L, gamma, ldo,

@@ -38,6 +38,7 @@
 #include "tdg_common.cuh"
 #include "tdg_digits.cuh"
 #include "tdg_internal.h"
+#include "tdg_optin.h"
 
 namespace tdg {
 
@@ -756,9 +757,8 @@ template <typename T, int FORM, int W, typename C, bool KEEP, bool MIX, int RND 
 cudaError_t launch_grid(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStream_t st) {
     using Cfg = GemmCfg<T, FORM, W, C>;
     auto kern = packed_gemm_kernel<T, FORM, W, C, KEEP, MIX, RND>;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCtaSmem);
-    if (attr != cudaSuccess) return attr;
+    static SmemOptIn smem_ok;
+    if (cudaError_t e = smem_ok.allow(kern, kMaxCtaSmem)) return e;
     CUtensorMap ma, mb, mpa, mpb;
     if (!map_operand<T, C>(&ma, ops.a, C::BM) || !map_operand<T, C>(&mb, ops.b, C::BN))
         return cudaErrorInvalidValue;
@@ -784,9 +784,8 @@ cudaError_t launch_target(const GemmArgs<T> &g0, const GemmOperands &ops, cudaSt
     using CfgP = GemmCfg<T, G_PLAIN, 1, CP>;
     static_assert((int)Cfg::NT == (int)CfgP::NT, "one block shape");
     auto kern = target_gemm_kernel<T, FORM, W, C, CP, KEEP>;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCtaSmem);
-    if (attr != cudaSuccess) return attr;
+    static SmemOptIn smem_ok;
+    if (cudaError_t e = smem_ok.allow(kern, kMaxCtaSmem)) return e;
     CUtensorMap ma, mb, mpa, mpb;
     if (!map_operand<T, C>(&ma, ops.a, C::BM) || !map_operand<T, C>(&mb, ops.b, C::BN))
         return cudaErrorInvalidValue;

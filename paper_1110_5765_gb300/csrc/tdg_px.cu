@@ -284,13 +284,8 @@ template <typename T, int W, typename C>
 cudaError_t launch_px_w(const GemmArgs<T> &g0, const GemmOperands &ops, cudaStream_t st) {
     using Cfg = PxCfg<T, W, C>;
     auto kern = px_gemm_kernel<T, W, C>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static SmemOptIn smem_ok;
+    if (cudaError_t e = smem_ok.allow(kern, (int)Cfg::SMEM)) return e;
     const CUtensorMapDataType dt =
         sizeof(T) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     CUtensorMap ma, mb;

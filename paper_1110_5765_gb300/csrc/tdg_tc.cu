@@ -45,10 +45,12 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "tdg_common.cuh"
 #include "tdg_internal.h"
+#include "tdg_optin.h"
 
 namespace tdg {
 
@@ -626,7 +628,13 @@ template <int FP8>
 static cudaError_t launch_tc(const TcArgs &a, const CUtensorMap &mapA, const CUtensorMap &mapB,
                              const CUtensorMap &mapC, cudaStream_t st) {
     auto kern = tc_gemm_kernel<FP8>;
-    static int max_clusters = 0;
+    // clusters that fit the device, by ordinal
+    static std::atomic<int> max_clusters[64];
+    static SmemOptIn smem_ok;
+    if (cudaError_t e = smem_ok.allow(kern, (int)SMEM_BYTES)) return e;
+    int dev = 0;
+    if (cudaError_t e = cudaGetDevice(&dev)) return e;
+    int clusters = dev < 64 ? max_clusters[dev].load(std::memory_order_relaxed) : 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -640,21 +648,14 @@ static cudaError_t launch_tc(const TcArgs &a, const CUtensorMap &mapA, const CUt
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;                    // the occupancy query: cluster shape only
-    if (!max_clusters) {
-        cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cfg.gridDim = dim3((unsigned)max(2, sms & ~1));
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, (void *)kern, &cfg);
-        if (e != cudaSuccess) return e;
-        max_clusters = max(1, n);
+    if (!clusters) {
+        cfg.gridDim = dim3((unsigned)max(2, device_sms() & ~1));
+        if (cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, (void *)kern, &cfg)) return e;
+        clusters = max(1, clusters);
+        if (dev < 64) max_clusters[dev].store(clusters, std::memory_order_relaxed);
     }
     const long long pairs = ((a.N + BN - 1) / BN) * (((a.M + BM - 1) / BM + 1) / 2);
-    cfg.gridDim = dim3((unsigned)(2 * std::min<long long>(pairs, max_clusters)));
+    cfg.gridDim = dim3((unsigned)(2 * std::min<long long>(pairs, clusters)));
     // the launch: cluster shape, and programmatic serialisation unless the grid
     // leaves SMs idle
     cfg.numAttrs = pdl_for_grid(cfg.gridDim.x) ? 2 : 1;
