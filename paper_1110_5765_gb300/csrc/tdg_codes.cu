@@ -14,8 +14,8 @@
 //   else    the statistics pass has run (target mode, L > 128): c from the
 //           block maxima and the plan's gammas.  Tiles are walked backwards: the
 //           statistics read op(A) and then op(B), so the last ones are in L2.
-// c is __fdiv_rn of two fp32 numbers: the fp64 quotient rounded to fp32 has the
-// same bits, since 53 >= 2 * 24 + 2.
+// c is __fdiv_rn of two fp32 numbers (gamma <= 2048): the fp64 quotient rounded to
+// fp32 has the same bits, since 53 >= 2 * 24 + 2.
 // Shared-memory layout: rows of TS values as stored, 16-byte chunks permuted
 // within the row so that the reads below have no bank conflicts.
 #include <cuda_fp16.h>

@@ -104,7 +104,8 @@ struct Job {
     double gamma;             // of the plan, or the manual compander itself
     long long row_end;        // rows (along k) that the product reads
     // c of the block at (x, k): the fp64 quotient rounded to T (fp32: the fp32
-    // quotient has the same bits, since 53 >= 2 * 24 + 2)
+    // quotient has the same bits, since 53 >= 2 * 24 + 2 and gamma is an fp32 number:
+    // below 2^19 for fixed bits <= 20, at most R_max / L <= 2^24 / 16 for targets)
     __device__ inline T compander(long long x, long long k) const {
         if (!compand) return T(1);
         if (manual) return (T)gamma;
