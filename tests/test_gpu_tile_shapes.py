@@ -10,9 +10,10 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 # (M, N, K) for fp64 on 152 SMs: 16-tiles (one, ragged, split over slabs, two per
-# SM), 32-tiles (143 of them), 64-tiles
+# SM), 32-tiles (143 of them; asymmetric 16), 16-tiles in many waves, 64-tiles (152 of
+# them; then, for the asymmetric form, 297)
 F64 = [(1, 1, 70), (17, 31, 130), (60, 70, 600), (257, 250, 130), (350, 410, 130),
-       (600, 930, 66)]
+       (600, 930, 66), (512, 1216, 66), (2048, 1728, 66)]
 
 
 @pytest.mark.parametrize("shape", F64)
@@ -33,8 +34,9 @@ def test_f64_tiles(orc, shape, form, W):
         assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
 
 
-# fp32: one ragged 64-tile, 64-tiles, 128 x 64 tiles (r = 1, 2), 128 x 128 tiles,
-# slabs split over CTAs
+# fp32, symmetric: one ragged 64-tile, 64-tiles (up to one and two an SM), 128 x 64
+# tiles, 128 x 128 tiles, slabs split over CTAs (asymmetric: 64-tiles; BY_RULE has the
+# others)
 F32 = [(60, 50, 130), (700, 690, 130), (1000, 777, 130), (1500, 1300, 130), (2000, 1900, 66),
        (129, 70, 1400)]
 
@@ -103,17 +105,28 @@ def test_fallback_apart(orc, dtype, shape, W, target, used):
         assert np.array_equal(C.cpu().numpy().view(np.uint8), ref.C.view(np.uint8))
 
 
-# asymmetric products in every tile of theirs, with W = 3 and 4 results a number, and
-# symmetric targets whose W is decided on the device
-@pytest.mark.parametrize("form,W,L,shape,kw", [
-    ("asym", 4, 64, (700, 900, 330), dict(bits=4)),         # 64 x 64, not split
-    ("asym", 4, 64, (100, 300, 1400), dict(bits=4)),        # 64 x 128, split
-    ("asym", 3, 64, (64, 40, 2000), dict(bits=4)),          # split, ragged digits
-    ("asym", 4, 64, (2300, 2500, 66), dict(bits=4)),        # 64 x 128, not split
-    ("sym", 4, 64, (130, 200, 2100), dict(target=15.0)),    # split
-    ("asym", 4, 64, (130, 200, 2100), dict(target=15.0)),   # split for some W
-    ("asym", 3, 64, (1300, 900, 260), dict(target=15.0)),
-])
+# the smallest products of a search that take each tile, whole and split (W of symmetric
+# targets: decided on the device, tiled for 2); test_tile_rule.py checks the tiles
+BY_RULE = [
+    ("asym", 2, 64, (4200, 2000, 60), dict(bits=4), "big", False),
+    ("asym", 2, 64, (130, 2000, 520), dict(bits=4), "big", True),
+    ("asym", 3, 64, (2600, 2000, 66), dict(bits=4), "big", False),
+    ("asym", 3, 64, (130, 2000, 520), dict(bits=4), "big", True),
+    ("asym", 4, 64, (4200, 2000, 66), dict(bits=4), "big", False),
+    ("asym", 4, 64, (260, 2000, 520), dict(bits=4), "big", True),
+    ("asym", 4, 64, (700, 900, 130), dict(bits=4), "small", False),
+    ("asym", 3, 64, (64, 40, 2000), dict(bits=4), "small", True),
+    ("sym", 2, 64, (1300, 3300, 60), dict(bits=6), "big", False),
+    ("sym", 2, 64, (260, 700, 3000), dict(bits=6), "big", True),
+    ("sym", 2, 64, (4200, 400, 60), dict(bits=6), "mid", False),
+    ("sym", 4, 64, (130, 130, 520), dict(bits=4), "small", True),
+    ("sym", 4, 64, (130, 200, 2100), dict(target=15.0), "small", True),
+    ("asym", 4, 64, (130, 200, 2100), dict(target=15.0), "small", True),
+    ("asym", 3, 64, (1300, 900, 260), dict(target=15.0), "small", False),
+]
+
+
+@pytest.mark.parametrize("form,W,L,shape,kw", [c[:5] for c in BY_RULE])
 def test_tiles_by_form_and_packing(orc, form, W, L, shape, kw):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")

@@ -8,6 +8,7 @@ import subprocess
 import pytest
 
 from paper_1110_5765_gb300 import build
+from test_gpu_tile_shapes import BY_RULE
 
 SHIM = r"""
 #include "tdg_tile_rule.h"
@@ -69,6 +70,13 @@ def _rule(host, form, W, L, M, N, K, target=0, may_split=1, sms=152):
 def test_measured_products(host, form, W, L, shape, tile, split):
     t, groups, _ = _rule(host, form, W, L, *shape)
     assert (t, groups > 1) == (tile, split)
+
+
+@pytest.mark.parametrize("form,W,L,shape,kw,tile,split", BY_RULE)
+def test_tiles_of_the_gpu_cases(host, form, W, L, shape, kw, tile, split):
+    target = "target" in kw
+    t, groups, _ = _rule(host, form, 2 if target and form == "sym" else W, L, *shape, int(target))
+    assert (t, groups > 1) == ({"big": BIG, "mid": MID, "small": SMALL}[tile], split)
 
 
 def test_a_split_runs_at_once(host):
