@@ -652,7 +652,8 @@ static tdg_status gemm_impl(tdgemm_plan_t p, T *C, double alpha, double beta, cu
     };
     // a distortion target's product: the symmetric form in one launch for every
     // candidate, the asymmetric one in a launch per W, the last of them holding
-    // the plain fallback too (mixed, pair-exact and large fp32 products: apart)
+    // the plain fallback too where that keeps its tile (mixed, pair-exact and large
+    // fp32 products: apart)
     bool one_launch = p->mode == MODE_TARGET && is_packed_form(p->form) && !p->kctrl_mode &&
                       !(p->flags & TDG_PAIR_EXACT);
     // mixed tiles (Sec. 6) keep the tile that the tile order was made for, kept slab

@@ -3,9 +3,9 @@
 // companders c = gamma / max|x| of each L x L block of op(X).
 //
 // One CTA of 512 threads per SM (two for 64-tiles) walks its share of TS x TS
-// tiles; three tiles are in flight to shared memory by cp.async while one is
-// encoded, so the memory system sees 96 to 192 KB of outstanding reads per SM
-// whatever the phase the threads are in.  HBM bounds the kernel: it reads 4
+// tiles; three tiles are in flight to shared memory by cp.async (two between the
+// wait for a tile and the refill of its stage), so the memory system sees 64 to 192
+// KB of outstanding reads per SM whatever the phase.  HBM bounds the kernel: it reads 4
 // bytes and writes 2 or 1 per value once.
 //   FUSED   companders that depend on their own block only (fixed bits, E4M3)
 //           with L = TS: the tile is a block; its maximum (and, for the integer

@@ -692,10 +692,11 @@ __global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W
 // A distortion target's product in one launch: the packing, and whether the
 // target was met at all, are known on the device only.  The packed product
 // (symmetric: of any W, only the operand rows differ) and the plain fallback (tile
-// CP, arguments gp) are one kernel.  As launches of their own, the ones not chosen
-// took 2 to 7 us each to return at entry.  Not for the unsplit fp32 product in 8 x 8 thread tiles, which has no
-// register to spare (1.155 ms instead of 1.106 at 4096^3): there both rounding
-// variants and the fallback are queued.
+// CP, arguments gp; fallback_keeps_tile) are one kernel.  As launches of their own,
+// the ones not chosen took 2 to 7 us each to return at entry.  Not for the unsplit
+// fp32 product in 8 x 8 thread tiles, which has no register to spare (1.155 ms
+// instead of 1.106 at 4096^3): there both rounding variants and the fallback are
+// queued.
 template <typename T, int FORM, int W, typename C, typename CP, bool KEEP>
 __global__ void __launch_bounds__(GemmCfg<T, FORM, W, C>::NT, GemmCfg<T, FORM, W, C>::MIN_CTAS)
     target_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
