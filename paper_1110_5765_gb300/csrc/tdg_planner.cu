@@ -358,9 +358,9 @@ cudaError_t launch_kernel_control(const PlanParams &pp, const double *mA, const 
     // Behind the statistics' full wave the few CTAs, launched early, pile up on the SMs
     // that are left first and share their fp64 pipes (fixed bits, 2048^3: the steps up to
     // the product took 73 us, with a plain launch 58).  A target's decision, one CTA,
-    // leaves them all; one or two CTAs have the pipes of an SM to themselves anyway
-    // (512^3: 83.6 us a call, with a plain launch 85.1).
-    const bool pdl = pp.mode == MODE_TARGET || ctas <= 2 || pdl_for_grid(ctas);
+    // leaves them all.  So few CTAs that no pile matters are launched early (1024^3,
+    // eight of them: 131.0 us a call, with a plain launch 132.9).
+    const bool pdl = pp.mode == MODE_TARGET || ctas <= 8 || pdl_for_grid(ctas);
     cudaError_t e = launch_pdl_if(pdl, kernel_ratio_kernel, dim3((unsigned)ctas), dim3(256), 0, st,
                                   pp, mA, vA, mB, vB, plan, ratio);
     if (e != cudaSuccess) return e;
